@@ -217,8 +217,9 @@ pos_status poseidon_eval_batch_host(void *handle, const pos_candidate *cands, in
  * Deterministic argmin over eval_batch outputs (hot-path step a9): the
  * smallest makespan among entries with feasible == 1, ties broken to the
  * lowest index.  Device pointers; *d_out (int64, device) receives the index
- * or -1 when no entry is feasible.  Asynchronous on `stream`; uses a
- * stream-ordered scratch allocation of at most 16 bytes per SM * 4.
+ * or -1 when no entry is feasible.  Asynchronous on `stream`; above 16384
+ * entries it uses a stream-ordered scratch allocation of at most 16 bytes per
+ * SM * 4 from the library's pool (per device, kept between calls).
  */
 pos_status poseidon_argmin(const int32_t *d_makespan, const uint8_t *d_feasible, int64_t n,
                            int64_t *d_out, void *stream);

@@ -13,12 +13,6 @@
 
 namespace pos {
 
-// the two kernels of poseidon_argmin (defined in eval.cu)
-__global__ void argmin_partial(const int32_t *T, const uint8_t *F, int64_t n, int32_t *part_t,
-                               long long *part_i);
-__global__ void argmin_final(const int32_t *part_t, const long long *part_i, int parts,
-                             int64_t *out);
-
 constexpr int kNoAllocParts = 4096;  // partial results the fixed scratch holds
 
 // 4096 x (int32 makespan, padded to 8 bytes) + 4096 x int64 index = 64 KB
@@ -54,9 +48,7 @@ extern "C" pos_status poseidon_argmin_noalloc(const int32_t *d_makespan,
                                               int64_t *d_out, void *stream) {
     if (n < 0 || !d_out || (n > 0 && (!d_makespan || !d_feasible)))
         return pos::fail(POS_EINVAL, "bad argmin arguments");
-    const int64_t parts = std::max<int64_t>(
-        1, std::min<int64_t>((n + pos::kArgminThreads - 1) / pos::kArgminThreads,
-                             4LL * pos::sm_count()));
+    const int64_t parts = pos::argmin_parts(n);
     if (parts > pos::kNoAllocParts)
         return pos::fail(POS_EINVAL,
                          "poseidon_argmin_noalloc: this GPU needs more than 4096 partial "
@@ -70,10 +62,5 @@ extern "C" pos_status poseidon_argmin_noalloc(const int32_t *d_makespan,
         reinterpret_cast<long long *>(static_cast<char *>(scratch) + pos::kNoAllocParts * 8);
     // every slot the final kernel reads is written by the partial kernel of
     // the same call, so nothing has to be cleared between calls
-    pos::argmin_partial<<<(int)parts, pos::kArgminThreads, 0, s>>>(d_makespan, d_feasible, n, pt,
-                                                                     pi);
-    pos::argmin_final<<<1, 32, 0, s>>>(pt, pi, (int)parts, d_out);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return pos::cuda_fail(e, "argmin_noalloc launch");
-    return POS_OK;
+    return pos::launch_argmin(d_makespan, d_feasible, n, pt, pi, d_out, s);
 }

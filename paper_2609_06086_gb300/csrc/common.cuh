@@ -119,10 +119,15 @@ struct Handle {
     int lim_off, lim_w, lim_bytes;
 };
 constexpr int kLimMaxBytes = 32768;
-// Threads per block of the argmin partial kernel (poseidon_argmin and
-// poseidon_argmin_noalloc): its shared arrays hold one entry per warp of a
-// block of this size, so every launch must use exactly this many threads.
+// Threads per block of the argmin kernels (poseidon_argmin and
+// poseidon_argmin_noalloc): their shared arrays hold one entry per warp of a
+// block of this size, so every launch uses exactly this many threads.
 constexpr int kArgminThreads = 256;
+// Partial results of an argmin over n entries (1: none are stored), and its
+// launches (eval.cu).
+int64_t argmin_parts(int64_t n);
+pos_status launch_argmin(const int32_t *T, const uint8_t *F, int64_t n, int32_t *part_t,
+                         long long *part_i, int64_t *out, cudaStream_t stream);
 
 pos_status validate_tables(const pos_tables *t);
 pos_status create_handle(const pos_tables *t, int sched, Handle **out);
