@@ -82,8 +82,12 @@ inline cudaError_t launch_dependent(void (*kern)(KArgs...), int grid, int block,
 //   binom  u64 [16][128]        C(n, k) at [k][n], k <= 15 (0 for n < k)
 //   Pw, Pa i64 [K][L+1] each    exclusive prefix sums of mem_w, mem_a
 //   cap    i64 [K]
-//   Pf, Pb, Pd i32 [K][L+1]     exclusive prefix sums of fwd, bwd, dsync
-//   p2f, p2b   i32 [K][K]       transfer times [src class][dst class]
+//   P      i32x4 [K][L+1]       exclusive prefix sums of fwd, bwd, dsync (and a
+//                               0): a stage's three sums take one 16-byte load
+//                               per end instead of three loads
+//   pp     i32x2 [K][K]         transfer times of the edge between a stage on
+//                               class a and the next one on class b, at [a][b]:
+//                               (p2p_f[a][b], p2p_b[b][a])
 // ---------------------------------------------------------------------------
 constexpr int kBinomN = 128;
 constexpr int kBinomK = 16;
@@ -92,15 +96,18 @@ struct BlobLayout {
     int L, K, n_types, n_tp;
     int sched;  // POS_SCHED_* (stage chains, in-flight counts; Interleaved 1F1B
                 // evaluates records with V < 2 as 1F1B)
-    int off_binom, off_Pw, off_Pa, off_cap, off_Pf, off_Pb, off_Pd, off_p2f, off_p2b;
+    int off_binom, off_Pw, off_Pa, off_cap, off_P, off_pp;
     int bytes;  // multiple of 16
 };
 
 BlobLayout make_layout(int L, int n_types, int n_tp);
-// The timing part of a blob (Pf, Pb, Pd, p2f, p2b: its last five tables),
-// rebased to start at byte 0, for kernels that read nothing else; the
-// timing part starts at byte ly.off_Pf of the full blob.
+// The timing part of a blob (P, pp: its last two tables), rebased to start
+// at byte 0, for kernels that read nothing else; the timing part starts at
+// byte ly.off_P of the full blob.
 BlobLayout timing_layout(const BlobLayout &ly);
+// The same with the memory part before it (everything but the binomials);
+// it starts at byte ly.off_Pw of the full blob.
+BlobLayout cost_layout(const BlobLayout &ly);
 // The memory part (Pw, Pa, cap: the three tables after the binomials),
 // rebased likewise; it starts at byte ly.off_Pw of the full blob.
 BlobLayout memory_layout(const BlobLayout &ly);
@@ -166,14 +173,19 @@ __device__ __forceinline__ Tab tab_at(const unsigned char *base, const BlobLayou
     return t;
 }
 
-__device__ __forceinline__ int32_t Pf(const Tab &t, int k, int c) {
-    return ld32(t.base, t.ly->off_Pf + 4u * (uint32_t)(k * (t.ly->L + 1) + c));
+// (forward, backward, all-reduce) sums over layers [0, c) on class k
+struct Sums {
+    int32_t f, b, d;
+};
+__device__ __forceinline__ Sums sums(const Tab &t, int k, int c) {
+    const int4 v = *reinterpret_cast<const int4 *>(t.base + t.ly->off_P +
+                                                   16u * (uint32_t)(k * (t.ly->L + 1) + c));
+    return {v.x, v.y, v.z};
 }
-__device__ __forceinline__ int32_t Pb(const Tab &t, int k, int c) {
-    return ld32(t.base, t.ly->off_Pb + 4u * (uint32_t)(k * (t.ly->L + 1) + c));
-}
-__device__ __forceinline__ int32_t Pd(const Tab &t, int k, int c) {
-    return ld32(t.base, t.ly->off_Pd + 4u * (uint32_t)(k * (t.ly->L + 1) + c));
+// ... over layers [a, c), the sums at a known
+__device__ __forceinline__ Sums sums_from(const Tab &t, int k, const Sums &at, int c) {
+    const Sums v = sums(t, k, c);
+    return {v.f - at.f, v.b - at.b, v.d - at.d};
 }
 __device__ __forceinline__ int64_t Pw(const Tab &t, int k, int c) {
     return ld64(t.base, t.ly->off_Pw + 8u * (uint32_t)(k * (t.ly->L + 1) + c));
@@ -184,11 +196,11 @@ __device__ __forceinline__ int64_t Pa(const Tab &t, int k, int c) {
 __device__ __forceinline__ int64_t cap_of(const Tab &t, int k) {
     return ld64(t.base, t.ly->off_cap + 8u * (uint32_t)k);
 }
-__device__ __forceinline__ int32_t p2f(const Tab &t, int a, int b) {
-    return ld32(t.base, t.ly->off_p2f + 4u * (uint32_t)(a * t.ly->K + b));
-}
-__device__ __forceinline__ int32_t p2b(const Tab &t, int a, int b) {
-    return ld32(t.base, t.ly->off_p2b + 4u * (uint32_t)(a * t.ly->K + b));
+// transfer times between a stage on class a and the next stage on class b:
+// x of the forward edge, y of the backward edge
+__device__ __forceinline__ int2 p2p(const Tab &t, int a, int b) {
+    return *reinterpret_cast<const int2 *>(t.base + t.ly->off_pp +
+                                           8u * (uint32_t)(a * t.ly->K + b));
 }
 // stored k-major ([k][n]) as 64-bit words, so that a warp reading
 // C(n_lane, k) for one k touches consecutive 8-byte words
@@ -423,14 +435,16 @@ __device__ __forceinline__ void stage_weights(const Tab &t, const int (&cut)[S +
                                               const int (&cls)[S], StageW<S> &w) {
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        w.F[s] = Pf(t, cls[s], cut[s + 1]) - Pf(t, cls[s], cut[s]);
-        w.B[s] = Pb(t, cls[s], cut[s + 1]) - Pb(t, cls[s], cut[s]);
-        w.d[s] = Pd(t, cls[s], cut[s + 1]) - Pd(t, cls[s], cut[s]);
-    }
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        w.pf[s] = (s + 1 < S) ? p2f(t, cls[s], cls[s + 1 < S ? s + 1 : s]) : 0;
-        w.pb[s] = (s + 1 < S) ? p2b(t, cls[s + 1 < S ? s + 1 : s], cls[s]) : 0;
+        const Sums v = sums_from(t, cls[s], sums(t, cls[s], cut[s]), cut[s + 1]);
+        w.F[s] = v.f;
+        w.B[s] = v.b;
+        w.d[s] = v.d;
+        w.pf[s] = w.pb[s] = 0;
+        if (s + 1 < S) {
+            const int2 e = p2p(t, cls[s], cls[s + 1 < S ? s + 1 : s]);
+            w.pf[s] = e.x;
+            w.pb[s] = e.y;
+        }
     }
 }
 
@@ -464,11 +478,11 @@ __device__ __forceinline__ bool plan_fits(const Tab &t, int M, const int (&cut)[
 // separate instantiation (kPathGeneric) whose schedule is unrolled for
 // each M in 1..S-1.
 // ---------------------------------------------------------------------------
-// Paths: 1F1B with M >= S (ramps + steady loop), 1F1B with M < S (unrolled
-// per M), Eager 1F1B with M >= 2S-1 (ramps + steady loop), Eager 1F1B with
-// M < 2S-1 as a level program (the search's leaf kernel) or unrolled per M
-// (the evaluator).
-enum { kPathFast = 0, kPathGeneric = 1, kPathEager = 2, kPathEagerShort = 3, kPathEagerUnrolled = 4 };
+// Paths: 1F1B with M >= S (ramps + steady loop), 1F1B with M < S (the search's
+// leaf kernel: unrolled per M), Eager 1F1B with M >= 2S-1 (ramps + steady
+// loop), Eager 1F1B with M < 2S-1 (leaf kernel: a level program).  The
+// evaluator's short pipelines have kernels of their own (ShortProgram).
+enum { kPathFast = 0, kPathGeneric = 1, kPathEager = 2, kPathEagerShort = 3 };
 
 // Op of 1-based stage s1 at ramp-up level t (1 <= t <= 2S-1) and at
 // ramp-down level 2M + tau (0 <= tau <= 2S-2), for M >= S: 0 none, 1 F, 2 B.
@@ -543,12 +557,6 @@ __device__ __forceinline__ void steady_op(int32_t (&Fo)[S], int32_t (&Bo)[S], co
     if constexpr ((s1 & 1) == P) relax_f<S, s>(Fo, w, Bo[s]);
     else relax_b<S, s>(Bo, w, Fo[s]);
 }
-template <int S, int P, int... i>
-__device__ __forceinline__ void steady_level(int32_t (&Fo)[S], int32_t (&Bo)[S], const StageW<S> &w,
-                                             std::integer_sequence<int, i...>) {
-    (steady_op<S, P, i>(Fo, Bo, w), ...);
-}
-
 // M < S: the same level order, with W_s = min(S-s1+1, M); every op and the
 // type of each stage's previous op are known at compile time for a given
 // (S, M), so the whole schedule is unrolled (M < S <= 16 keeps it small).
@@ -606,32 +614,177 @@ __device__ __forceinline__ int32_t makespan_short_dispatch(const StageW<S> &w, i
     return T;
 }
 
-template <int S, int PATH>
-__device__ __forceinline__ int32_t makespan_1f1b(const StageW<S> &w, int M) {
-    int32_t Fo[S], Bo[S];
+// ---------------------------------------------------------------------------
+// M >= S without running every steady step.  Let x be the finishes (Fo, Bo)
+// after some steady step, R the number of steady steps left.
+//  * Ramp-down.  T is a max-plus linear function of the state that enters
+//    the ramp-down: T = max_s max(Fo[s] + rF[s], Bo[s] + rB[s]), rF and rB
+//    the longest paths from those finishes to the end (all-reduce included).
+//    They depend on the weights alone and are built by walking the
+//    ramp-down's ops backwards, once per plan (tail_*).  A finish that no
+//    later op reads gets 0, which is valid too: T is at least every finish.
+//  * Upper bound.  A steady step is monotone and adds a constant to its
+//    result when the constant is added to its input, so no finish ever grows
+//    by more in a later step than the largest growth D of one step:
+//    T <= max_s max(Fo[s] + rF[s], Bo[s] + rB[s]) + R D.
+//  * Lower bound.  Stage s runs one forward and one backward per step, so its
+//    finishes grow by at least F[s] + B[s] in each:
+//    T >= max_s (max(Fo[s] + rF[s], Bo[s] + rB[s]) + R (F[s] + B[s])).
+// When the two are equal they are T and the remaining steps need not run;
+// at R = 0 they always are.  Whole numbers throughout, so nothing is
+// approximated.  On random plans (64 layers, 2..16 stages, 8..128
+// micro-batches) the bounds meet after three steps of the 61 on average
+// for 86 % (13..16 stages) to 99 % (1..4) of the plans.
+// ---------------------------------------------------------------------------
+template <int S>
+struct Tail {
+    int32_t F[S], B[S];
+};
+template <int S, int tau, int s1>
+__device__ __forceinline__ void tail_op(Tail<S> &r, const StageW<S> &w) {
+    constexpr int op = ramp_down_op(S, s1, tau);
+    constexpr bool last_b = down_last_is_b(S, s1, tau);
+    constexpr int s = s1 - 1;
+    if constexpr (op == 1) {
+        const int32_t t = r.F[s] + w.F[s];
+        if constexpr (last_b) {
+            r.F[s] = 0;  // the forward before this one is read by no later op
+            r.B[s] = max(r.B[s], t);
+        } else {
+            r.F[s] = t;
+        }
+        if constexpr (s > 0) r.F[s - 1] = add_max(t, w.pf[s - 1], r.F[s - 1]);
+    } else if constexpr (op == 2) {
+        const int32_t t = r.B[s] + w.B[s];
+        if constexpr (last_b) {
+            r.B[s] = t;
+        } else {
+            r.B[s] = 0;
+            r.F[s] = max(r.F[s], t);
+        }
+        if constexpr (s + 1 < S) r.B[s + 1] = add_max(t, w.pb[s], r.B[s + 1]);
+    }
+}
+// one level backwards: stages in ascending order
+template <int S, int tau, int... i>
+__device__ __forceinline__ void tail_level(Tail<S> &r, const StageW<S> &w,
+                                           std::integer_sequence<int, i...>) {
+    (tail_op<S, tau, i + 1>(r, w), ...);
+}
+template <int S, int... t>
+__device__ __forceinline__ void tail_ramp(Tail<S> &r, const StageW<S> &w,
+                                          std::integer_sequence<int, t...>) {
+    (tail_level<S, 2 * S - 2 - t>(r, w, std::make_integer_sequence<int, S>{}), ...);
+}
+
+// One steady step (two levels); GROWTH: its largest growth of a finish.
+template <int S, int P, bool GROWTH, int i>
+__device__ __forceinline__ void steady_op_growth(int32_t (&Fo)[S], int32_t (&Bo)[S],
+                                                 const StageW<S> &w, int32_t &grow) {
+    constexpr int s = S - i - 1;
+    const int32_t f = Fo[s], b = Bo[s];
+    steady_op<S, P, i>(Fo, Bo, w);
+    if constexpr (GROWTH) {
+        if constexpr (((s + 1) & 1) == P) grow = max(grow, Fo[s] - f);
+        else grow = max(grow, Bo[s] - b);
+    }
+}
+template <int S, bool GROWTH, int... i>
+__device__ __forceinline__ void steady_step(int32_t (&Fo)[S], int32_t (&Bo)[S], const StageW<S> &w,
+                                            int32_t &grow, std::integer_sequence<int, i...>) {
+    (steady_op_growth<S, 0, GROWTH, i>(Fo, Bo, w, grow), ...);
+    (steady_op_growth<S, 1, GROWTH, i>(Fo, Bo, w, grow), ...);
+}
+
+// Steady steps before the bounds are first compared and between later
+// comparisons (one of them costs about two and a half plain steps), the
+// fastest of 2, 3, 4, 6, 8 and 10 with 4, 12, 16 and 24 on random plans; the
+// bounds of Eager 1F1B meet for nine plans in ten after the second step.
+__host__ __device__ constexpr int first_steps(int S) { return S <= 4 ? 3 : 6; }
+constexpr int kFirstStepsEager = 2;
+constexpr int kNextSteps = 16;
+
+// What a caller does with a makespan: with no limit it needs the value; with
+// one it only needs to know that T * scale is above the limit (the search's
+// incumbent), so a lower bound above it ends the plan, and any value whose
+// product is above the limit may be returned.  The bounds are then compared
+// before the first steady step, where the lower one already ends 97 % of the
+// complete plans of the 70B-like search, and after every few steps from then.
+struct NoLimit {
+    static constexpr bool kOn = false;
+    __device__ __forceinline__ bool above(int32_t) const { return false; }
+};
+struct ObjLimit {
+    static constexpr bool kOn = true;
+    uint64_t scale, limit;
+    __device__ __forceinline__ bool above(int32_t T) const {
+        return (uint64_t)(uint32_t)T * scale > limit;
+    }
+};
+
+// Makespan of a plan with M >= S.  to_end: runs until the bounds meet;
+// otherwise the plan is given up after their first comparison and false is
+// returned when they differ there.
+template <int S, class Limit>
+__device__ __forceinline__ bool makespan_fast(const StageW<S> &w, int M, bool to_end,
+                                              const Limit &limit, int32_t &T) {
+    Tail<S> r;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        Fo[s] = 0;
-        Bo[s] = 0;
+        r.F[s] = 0;
+        r.B[s] = w.d[s];
     }
-    if constexpr (PATH == kPathFast) {
-        // ramp-up: levels 1 .. 2S-1
-        ramp<S, true, 1>(Fo, Bo, w, std::make_integer_sequence<int, 2 * S - 1>{});
-        // steady state: M - S steps of two levels (even, then odd)
-        for (int j = 0; j < M - S; ++j) {
-            steady_level<S, 0>(Fo, Bo, w, std::make_integer_sequence<int, S>{});
-            steady_level<S, 1>(Fo, Bo, w, std::make_integer_sequence<int, S>{});
-        }
-        // ramp-down: levels 2M + tau, tau = 0 .. 2S-2
-        ramp<S, false, 0>(Fo, Bo, w, std::make_integer_sequence<int, 2 * S - 1>{});
-    } else {
-        // M < S (kPathGeneric): fully unrolled instance for this M
-        if constexpr (S > 1) return makespan_short_dispatch<S>(w, M, std::make_integer_sequence<int, S - 1>{});
-    }
-    int32_t T = 0;
+    tail_ramp<S>(r, w, std::make_integer_sequence<int, 2 * S - 1>{});
+    int32_t Fo[S], Bo[S];
+    // Warm-up, levels 1 .. S: no backward yet.  The longest path to F_{s,m}
+    // visits every stage up to s once and repeats stages m - 1 times in all,
+    // so it repeats the slowest of them:
+    //   finish(F_{s,m}) = sum_{j<=s} F_j + sum_{j<s} pf_j + (m-1) max_{j<=s} F_j;
+    // stage s runs its m = S-s+1 warm-up forwards.
+    int32_t path = 0, slow = 0;
 #pragma unroll
-    for (int s = 0; s < S; ++s) T = max(T, Bo[s] + w.d[s]);
-    return T;
+    for (int s = 0; s < S; ++s) {
+        slow = max(slow, w.F[s]);
+        path += w.F[s];
+        Fo[s] = path + (S - 1 - s) * slow;
+        Bo[s] = 0;
+        path += w.pf[s];
+    }
+    // the rest of the ramp-up: levels S+1 .. 2S-1
+    ramp<S, true, S + 1>(Fo, Bo, w, std::make_integer_sequence<int, S - 1>{});
+    int left = M - S, steps = Limit::kOn ? 0 : first_steps(S);
+    if constexpr (Limit::kOn) {
+        int32_t lo = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+            lo = max(lo, add_max(Fo[s], r.F[s], Bo[s] + r.B[s]) + left * (w.F[s] + w.B[s]));
+        T = lo;
+        if (limit.above(lo)) return true;
+    }
+    for (;;) {
+        const int n = min(steps, left);
+        left -= n;
+        int32_t grow = 0;
+#pragma unroll 1
+        for (int j = 0; j < n; ++j)
+            steady_step<S, false>(Fo, Bo, w, grow, std::make_integer_sequence<int, S>{});
+        if (left > 0) {
+            steady_step<S, true>(Fo, Bo, w, grow, std::make_integer_sequence<int, S>{});
+            --left;
+        }
+        int32_t hi = 0, lo = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const int32_t m = add_max(Fo[s], r.F[s], Bo[s] + r.B[s]);
+            hi = max(hi, m);
+            lo = max(lo, m + left * (w.F[s] + w.B[s]));
+        }
+        T = lo;
+        // hi + left * grow == lo, without overflow
+        if ((int64_t)left * grow == (int64_t)(lo - hi) || limit.above(lo)) return true;
+        if (!to_end) return false;
+        steps = Limit::kOn ? 3 : kNextSteps;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -681,9 +834,15 @@ __host__ __device__ constexpr int eager_down_nf(int S, int s1, int tau) {
     for (int u = -2 * S + 2; u < tau; ++u) n += eager_down_op(S, s1, u) == 1;
     return n;
 }
-// forwards stage s1-1 has done beyond stage s1 before this op (1 or 2)
+// Is this op one of the warm-up forwards?  They are all done before the
+// ramp-up's other ops run.
+__host__ __device__ constexpr bool eager_up_warm(int S, int s1, int t) {
+    return t >= s1 && t <= 2 * S - s1;
+}
+// forwards stage s1-1 has done beyond stage s1 before this (later) forward
 __host__ __device__ constexpr int eager_up_lag(int S, int s1, int t) {
-    return eager_up_nf(S, s1 - 1, t) - eager_up_nf(S, s1, t);
+    const int warm = 2 * (S - (s1 - 1)) + 1, nf = eager_up_nf(S, s1 - 1, t);
+    return (nf > warm ? nf : warm) - eager_up_nf(S, s1, t);
 }
 __host__ __device__ constexpr int eager_down_lag(int S, int s1, int tau) {
     return (eager_down_nf(S, s1, 2 * S - 1) - eager_down_nf(S, s1 - 1, 2 * S - 1)) +
@@ -708,7 +867,9 @@ __device__ __forceinline__ void eager_ramp_op(int32_t (&Fo)[S], int32_t (&Fp)[S]
     constexpr int op = UP ? eager_up_op(S, s1, t) : eager_down_op(S, s1, t);
     constexpr bool last_b = UP ? eager_up_last_is_b(S, s1, t) : eager_down_last_is_b(S, s1, t);
     constexpr int s = s1 - 1;
-    if constexpr (op == 1) {
+    if constexpr (UP && op == 1 && eager_up_warm(S, s1, t)) {
+        // done already
+    } else if constexpr (op == 1) {
         constexpr int lag = s1 == 1 ? 1 : (UP ? eager_up_lag(S, s1, t) : eager_down_lag(S, s1, t));
         relax_f_lag<S, s, lag>(Fo, Fp, w, last_b ? Bo[s] : Fo[s]);
     } else if constexpr (op == 2) {
@@ -735,60 +896,172 @@ __device__ __forceinline__ void eager_steady_op(int32_t (&Fo)[S], int32_t (&Fp)[
     if constexpr ((s1 & 1) == P) relax_f_lag<S, s, 2>(Fo, Fp, w, Bo[s]);
     else relax_b<S, s>(Bo, w, Fo[s]);
 }
-template <int S, int P, int... i>
-__device__ __forceinline__ void eager_steady_level(int32_t (&Fo)[S], int32_t (&Fp)[S],
-                                                   int32_t (&Bo)[S], const StageW<S> &w,
-                                                   std::integer_sequence<int, i...>) {
-    (eager_steady_op<S, P, i>(Fo, Fp, Bo, w), ...);
+// Tail, bounds and early end of the steady steps as in makespan_fast, with
+// the previous forward Fp as a third finish per stage.
+template <int S>
+struct EagerTail {
+    int32_t F[S], P[S], B[S];  // longest paths from Fo, Fp, Bo to the end
+};
+template <int S, int tau, int s1>
+__device__ __forceinline__ void eager_tail_op(EagerTail<S> &r, const StageW<S> &w) {
+    constexpr int op = eager_down_op(S, s1, tau);
+    constexpr bool last_b = eager_down_last_is_b(S, s1, tau);
+    constexpr int s = s1 - 1;
+    if constexpr (op == 1) {
+        constexpr int lag = s1 == 1 ? 1 : eager_down_lag(S, s1, tau);
+        const int32_t t = r.F[s] + w.F[s];
+        // the forward before this one becomes Fp; the older one is gone
+        r.F[s] = last_b ? r.P[s] : max(r.P[s], t);
+        r.P[s] = 0;
+        if constexpr (last_b) r.B[s] = max(r.B[s], t);
+        if constexpr (s > 0) {
+            if constexpr (lag == 2) r.P[s - 1] = add_max(t, w.pf[s - 1], r.P[s - 1]);
+            else r.F[s - 1] = add_max(t, w.pf[s - 1], r.F[s - 1]);
+        }
+    } else if constexpr (op == 2) {
+        const int32_t t = r.B[s] + w.B[s];
+        if constexpr (last_b) {
+            r.B[s] = t;
+        } else {
+            r.B[s] = 0;
+            r.F[s] = max(r.F[s], t);
+        }
+        if constexpr (s + 1 < S) r.B[s + 1] = add_max(t, w.pb[s], r.B[s + 1]);
+    }
+}
+template <int S, int tau, int... i>
+__device__ __forceinline__ void eager_tail_level(EagerTail<S> &r, const StageW<S> &w,
+                                                 std::integer_sequence<int, i...>) {
+    (eager_tail_op<S, tau, i + 1>(r, w), ...);
+}
+template <int S, int... t>
+__device__ __forceinline__ void eager_tail_ramp(EagerTail<S> &r, const StageW<S> &w,
+                                                std::integer_sequence<int, t...>) {
+    (eager_tail_level<S, 2 * S - 2 - t>(r, w, std::make_integer_sequence<int, S>{}), ...);
+}
+
+template <int S, int P, bool GROWTH, int i>
+__device__ __forceinline__ void eager_steady_op_growth(int32_t (&Fo)[S], int32_t (&Fp)[S],
+                                                       int32_t (&Bo)[S], const StageW<S> &w,
+                                                       int32_t &grow) {
+    constexpr int s = S - i - 1;
+    const int32_t f = Fo[s], q = Fp[s], b = Bo[s];
+    eager_steady_op<S, P, i>(Fo, Fp, Bo, w);
+    if constexpr (GROWTH) {
+        if constexpr (((s + 1) & 1) == P) grow = max(grow, max(Fo[s] - f, f - q));
+        else grow = max(grow, Bo[s] - b);
+    }
+}
+template <int S, bool GROWTH, int... i>
+__device__ __forceinline__ void eager_steady_step(int32_t (&Fo)[S], int32_t (&Fp)[S],
+                                                  int32_t (&Bo)[S], const StageW<S> &w,
+                                                  int32_t &grow, std::integer_sequence<int, i...>) {
+    (eager_steady_op_growth<S, 0, GROWTH, i>(Fo, Fp, Bo, w, grow), ...);
+    (eager_steady_op_growth<S, 1, GROWTH, i>(Fo, Fp, Bo, w, grow), ...);
 }
 
 // Eager 1F1B, M >= 2S-1
-template <int S>
-__device__ __forceinline__ int32_t makespan_eager(const StageW<S> &w, int M) {
-    int32_t Fo[S], Fp[S], Bo[S];
+template <int S, class Limit>
+__device__ __forceinline__ bool makespan_eager(const StageW<S> &w, int M, bool to_end,
+                                               const Limit &limit, int32_t &T) {
+    EagerTail<S> r;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        Fo[s] = 0;
-        Fp[s] = 0;
+        r.F[s] = 0;
+        r.P[s] = 0;
+        r.B[s] = w.d[s];
+    }
+    eager_tail_ramp<S>(r, w, std::make_integer_sequence<int, 4 * S - 3>{});
+    // every stage's 2(S-s)+1 warm-up forwards by the closed form of
+    // makespan_fast (they precede its backwards in the chain and depend on
+    // forwards of earlier stages' warm-ups only), then the ramp-up's other ops
+    int32_t Fo[S], Fp[S], Bo[S];
+    int32_t path = 0, slow = 0;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        slow = max(slow, w.F[s]);
+        path += w.F[s];
+        Fo[s] = path + 2 * (S - 1 - s) * slow;
+        Fp[s] = s + 1 < S ? Fo[s] - slow : 0;
         Bo[s] = 0;
+        path += w.pf[s];
     }
     eager_ramp<S, true, 1>(Fo, Fp, Bo, w, std::make_integer_sequence<int, 2 * S - 1>{});
-    for (int j = 0; j < M - 2 * S + 1; ++j) {
-        eager_steady_level<S, 0>(Fo, Fp, Bo, w, std::make_integer_sequence<int, S>{});
-        eager_steady_level<S, 1>(Fo, Fp, Bo, w, std::make_integer_sequence<int, S>{});
-    }
-    eager_ramp<S, false, -2 * S + 2>(Fo, Fp, Bo, w, std::make_integer_sequence<int, 4 * S - 3>{});
-    int32_t T = 0;
+    int left = M - 2 * S + 1, steps = Limit::kOn ? 1 : kFirstStepsEager;
+    for (;;) {
+        const int n = min(steps, left);
+        left -= n;
+        int32_t grow = 0;
+#pragma unroll 1
+        for (int j = 0; j < n; ++j)
+            eager_steady_step<S, false>(Fo, Fp, Bo, w, grow, std::make_integer_sequence<int, S>{});
+        if (left > 0) {
+            eager_steady_step<S, true>(Fo, Fp, Bo, w, grow, std::make_integer_sequence<int, S>{});
+            --left;
+        }
+        int32_t hi = 0, lo = 0;
 #pragma unroll
-    for (int s = 0; s < S; ++s) T = max(T, Bo[s] + w.d[s]);
-    return T;
+        for (int s = 0; s < S; ++s) {
+            const int32_t m =
+                add_max(Fp[s], r.P[s], add_max(Fo[s], r.F[s], Bo[s] + r.B[s]));
+            hi = max(hi, m);
+            lo = max(lo, m + left * (w.F[s] + w.B[s]));
+        }
+        T = lo;
+        if ((int64_t)left * grow == (int64_t)(lo - hi) || limit.above(lo)) return true;
+        if (!to_end) return false;
+        steps = Limit::kOn ? 3 : kNextSteps;
+    }
 }
 
-// Eager 1F1B with M < 2S-1: the unit-weight ASAP level order has no closed
-// form, so it is computed at compile time for each (S, M) and unrolled like
-// the ramps.  Stage s (0-based) runs W = min(2(S-1-s)+1, M) forwards, then
-// (B_i, F_{W+i}) pairs, then the remaining backwards; an op's level is one
-// more than the later of its stage's previous op and its inter-stage
-// predecessor (F_{s-1,m} for F_{s,m}, B_{s+1,m} for B_{s,m}).  Within a
-// level the stages are visited in descending order, as in the ramps, and
-// while the program is built every op is checked to read the finish it
-// depends on: F_{s-1,m} from stage s-1's latest forward (lag 1) or the one
-// before (lag 2), B_{s+1,m} from stage s+1's latest backward.
-struct EagerShortOp {
+// ---------------------------------------------------------------------------
+// Short pipelines: M < S under 1F1B, M < 2S-1 under Eager 1F1B (the
+// evaluator; the search's leaf kernel has its own forms).
+//
+// The stages whose warm-up holds all M forwards run them all before their
+// first backward, so up to the last such stage the forwards form a plain
+// grid: F_{s,m} starts at the later of F_{s,m-1} and F_{s-1,m} + pf.  The
+// last C stages (C = M under 1F1B, M/2 + 1 under Eager 1F1B) are the ones
+// with shorter warm-ups and one stage before them; they are a small pipeline
+// of their own whose first stage's forwards start no earlier than the grid's
+// arrivals.  Their backwards then pass down the other S - C stages as a grid
+// again (B_{s,1} follows B_{s+1,1}, which follows F_{s+1,M} and so F_{s,M}:
+// the stage's own forwards never delay it).  So only the small pipeline has
+// to be unrolled, once per M for every S, and a plan costs its 2SM
+// relaxations (unrolled per (S, M) before: 120 and 240 instances, bound by
+// instruction fetch).
+//
+// The small pipeline's ops are visited in the unit-weight ASAP level order of
+// its chains, computed at compile time.  Stage s (0-based of C) runs W =
+// min(C-s, M) or min(2(C-1-s)+1, M) forwards, then (B_i, F_{W+i}) pairs,
+// then the remaining backwards; an op's level is one more than the later of
+// its stage's previous op and its inter-stage predecessor (F_{s-1,m} for
+// F_{s,m}, B_{s+1,m} for B_{s,m}).  Within a level the stages are visited in
+// descending order, and while the program is built every op is checked to
+// read the finish it depends on: F_{s-1,m} from stage s-1's latest forward
+// (lag 1) or the one before (lag 2), B_{s+1,m} from stage s+1's latest
+// backward.
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int short_stages(bool eager, int M) { return eager ? M / 2 + 1 : M; }
+
+struct ShortOp {
     int kind;      // 0 none, 1 forward, 2 backward
+    int m;         // micro-batch (0-based)
     int lag;       // forward of a stage s > 0: 1 or 2
     bool clock_b;  // the stage's previous op is a backward (else a forward)
 };
-template <int S, int M>
-struct EagerShortProgram {
-    static constexpr int kMaxLevels = 2 * (M + S) + 2;
-    EagerShortOp op[kMaxLevels][S];
+template <bool EAGER, int M>
+struct ShortProgram {
+    static constexpr int C = short_stages(EAGER, M);
+    static constexpr int kMaxLevels = 2 * (M + C) + 2;
+    ShortOp op[kMaxLevels][C];
     int n_levels;
     bool ok;
-    __host__ __device__ constexpr EagerShortProgram() : op{}, n_levels(0), ok(true) {
-        int kind[S][2 * M] = {}, mb[S][2 * M] = {};  // chains: op kind and micro-batch
-        for (int s = 0; s < S; ++s) {
-            const int W = 2 * (S - 1 - s) + 1 < M ? 2 * (S - 1 - s) + 1 : M;
+    __host__ __device__ constexpr ShortProgram() : op{}, n_levels(0), ok(true) {
+        int kind[C][2 * M] = {}, mb[C][2 * M] = {};  // chains: op kind and micro-batch
+        for (int s = 0; s < C; ++s) {
+            const int w = EAGER ? 2 * (C - 1 - s) + 1 : C - s;
+            const int W = w < M ? w : M;
             int n = 0;
             for (int m = 0; m < W; ++m) kind[s][n] = 1, mb[s][n++] = m;
             for (int i = 0; i < M - W; ++i) {
@@ -796,16 +1069,17 @@ struct EagerShortProgram {
                 kind[s][n] = 1, mb[s][n++] = W + i;
             }
             for (int m = M - W; m < M; ++m) kind[s][n] = 2, mb[s][n++] = m;
+            if (s == 0 && W != M) ok = false;  // the first stage runs every forward first
         }
-        int lf[S][M] = {}, lb[S][M] = {};  // ASAP levels (1-based)
+        int lf[C][M] = {}, lb[C][M] = {};  // ASAP levels (1-based)
         for (bool changed = true; changed;) {
             changed = false;
-            for (int s = 0; s < S; ++s) {
+            for (int s = 0; s < C; ++s) {
                 int prev = 0;
                 for (int n = 0; n < 2 * M; ++n) {
                     const int m = mb[s][n];
                     int p = prev;
-                    if (kind[s][n] == 2 && s + 1 < S && lb[s + 1][m] > p) p = lb[s + 1][m];
+                    if (kind[s][n] == 2 && s + 1 < C && lb[s + 1][m] > p) p = lb[s + 1][m];
                     if (kind[s][n] == 1 && s > 0 && lf[s - 1][m] > p) p = lf[s - 1][m];
                     int &v = kind[s][n] == 2 ? lb[s][m] : lf[s][m];
                     if (v != p + 1) {
@@ -816,7 +1090,7 @@ struct EagerShortProgram {
                 }
             }
         }
-        for (int s = 0; s < S; ++s)
+        for (int s = 0; s < C; ++s)
             for (int m = 0; m < M; ++m) {
                 if (lf[s][m] > n_levels) n_levels = lf[s][m];
                 if (lb[s][m] > n_levels) n_levels = lb[s][m];
@@ -827,11 +1101,11 @@ struct EagerShortProgram {
         }
         // registers: the micro-batch whose finish Fo / Fp / Bo of a stage
         // holds (-1: none yet) and whether its last op was a backward
-        int fo[S] = {}, fp[S] = {}, bo[S] = {};
-        bool last_b[S] = {};
-        for (int s = 0; s < S; ++s) fo[s] = fp[s] = bo[s] = -1;
+        int fo[C] = {}, fp[C] = {}, bo[C] = {};
+        bool last_b[C] = {};
+        for (int s = 0; s < C; ++s) fo[s] = fp[s] = bo[s] = -1;
         for (int l = 1; l <= n_levels; ++l)
-            for (int s = S - 1; s >= 0; --s) {
+            for (int s = C - 1; s >= 0; --s) {
                 int k = 0, m = -1;
                 for (int u = 0; u < M; ++u) {
                     if (lf[s][u] == l) k = k ? 3 : 1, m = u;
@@ -845,70 +1119,57 @@ struct EagerShortProgram {
                         else if (fp[s - 1] == m) lag = 2;
                         else ok = false;
                     }
-                    op[l - 1][s] = EagerShortOp{1, lag, last_b[s]};
+                    op[l - 1][s] = ShortOp{1, m, lag, last_b[s]};
                     fp[s] = fo[s];
                     fo[s] = m;
                     last_b[s] = false;
                 } else if (k == 2) {
-                    if (s + 1 < S && bo[s + 1] != m) ok = false;
-                    op[l - 1][s] = EagerShortOp{2, 0, last_b[s]};
+                    if (s + 1 < C && bo[s + 1] != m) ok = false;
+                    op[l - 1][s] = ShortOp{2, m, 0, last_b[s]};
                     bo[s] = m;
                     last_b[s] = true;
                 }
             }
     }
 };
-template <int S, int M>
-struct EagerShortTab {
-    static constexpr EagerShortProgram<S, M> value{};
-    static_assert(value.ok, "Eager 1F1B short level order: an op would read the wrong finish");
+template <bool EAGER, int M>
+struct ShortTab {
+    static constexpr ShortProgram<EAGER, M> value{};
+    static_assert(value.ok, "short pipeline: an op would read the wrong finish");
 };
 
-template <int S, int M, int l, int i>
-__device__ __forceinline__ void eager_short_op(int32_t (&Fo)[S], int32_t (&Fp)[S],
-                                               int32_t (&Bo)[S], const StageW<S> &w) {
-    constexpr int s = S - 1 - i;
-    constexpr EagerShortOp o = EagerShortTab<S, M>::value.op[l][s];
-    if constexpr (o.kind == 1)
-        relax_f_lag<S, s, (s > 0 ? o.lag : 1)>(Fo, Fp, w, o.clock_b ? Bo[s] : Fo[s]);
-    else if constexpr (o.kind == 2)
-        relax_b<S, s>(Bo, w, o.clock_b ? Bo[s] : Fo[s]);
-}
-template <int S, int M, int l, int... i>
-__device__ __forceinline__ void eager_short_level(int32_t (&Fo)[S], int32_t (&Fp)[S],
-                                                  int32_t (&Bo)[S], const StageW<S> &w,
-                                                  std::integer_sequence<int, i...>) {
-    (eager_short_op<S, M, l, i>(Fo, Fp, Bo, w), ...);
-}
-template <int S, int M, int... l>
-__device__ __forceinline__ void eager_short_all(int32_t (&Fo)[S], int32_t (&Fp)[S],
-                                                int32_t (&Bo)[S], const StageW<S> &w,
-                                                std::integer_sequence<int, l...>) {
-    (eager_short_level<S, M, l>(Fo, Fp, Bo, w, std::make_integer_sequence<int, S>{}), ...);
-}
-template <int S, int M>
-__device__ __forceinline__ int32_t makespan_eager_short(const StageW<S> &w) {
-    int32_t Fo[S], Fp[S], Bo[S];
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        Fo[s] = 0;
-        Fp[s] = 0;
-        Bo[s] = 0;
+// One op of the small pipeline.  at[m]: earliest start of the first stage's
+// forward m; once that has run, the finish of its backward m.
+template <bool EAGER, int M, int l, int i, int C>
+__device__ __forceinline__ void short_op_run(int32_t (&at)[M], int32_t (&Fo)[C], int32_t (&Fp)[C],
+                                             int32_t (&Bo)[C], const StageW<C> &w) {
+    constexpr int s = C - 1 - i;
+    constexpr ShortOp o = ShortTab<EAGER, M>::value.op[l][s];
+    if constexpr (o.kind == 1) {
+        const int32_t clock = o.clock_b ? Bo[s] : Fo[s];
+        if constexpr (s > 0) {
+            relax_f_lag<C, s, o.lag>(Fo, Fp, w, clock);
+        } else {
+            Fp[0] = Fo[0];
+            Fo[0] = max(at[o.m], clock) + w.F[0];
+        }
+    } else if constexpr (o.kind == 2) {
+        relax_b<C, s>(Bo, w, o.clock_b ? Bo[s] : Fo[s]);
+        if constexpr (s == 0) at[o.m] = Bo[0];
     }
-    eager_short_all<S, M>(Fo, Fp, Bo, w,
-                          std::make_integer_sequence<int, EagerShortTab<S, M>::value.n_levels>{});
-    int32_t T = 0;
-#pragma unroll
-    for (int s = 0; s < S; ++s) T = max(T, Bo[s] + w.d[s]);
-    return T;
 }
-// runtime M in 1..2S-2 -> its unrolled instance
-template <int S, int... m>
-__device__ __forceinline__ int32_t makespan_eager_short_dispatch(const StageW<S> &w, int M,
-                                                                 std::integer_sequence<int, m...>) {
-    int32_t T = -1;
-    ((M == m + 1 ? (T = makespan_eager_short<S, m + 1>(w), 0) : 0), ...);
-    return T;
+template <bool EAGER, int M, int l, int C, int... i>
+__device__ __forceinline__ void short_run_level(int32_t (&at)[M], int32_t (&Fo)[C],
+                                                int32_t (&Fp)[C], int32_t (&Bo)[C],
+                                                const StageW<C> &w,
+                                                std::integer_sequence<int, i...>) {
+    (short_op_run<EAGER, M, l, i>(at, Fo, Fp, Bo, w), ...);
+}
+template <bool EAGER, int M, int C, int... l>
+__device__ __forceinline__ void short_run(int32_t (&at)[M], int32_t (&Fo)[C], int32_t (&Fp)[C],
+                                          int32_t (&Bo)[C], const StageW<C> &w,
+                                          std::integer_sequence<int, l...>) {
+    (short_run_level<EAGER, M, l>(at, Fo, Fp, Bo, w, std::make_integer_sequence<int, C>{}), ...);
 }
 
 // Level program of one (schedule, S, M): per level one 64-bit word, bit s of
@@ -981,22 +1242,24 @@ struct Programs {
 // use, kept for the process); words = index = NULL for 1F1B.
 pos_status schedule_programs(int sched, Programs *out);
 
-// Makespan of one decoded plan on path PATH.
-template <int S, int PATH>
-__device__ __forceinline__ int32_t makespan_path(const StageW<S> &w, int M, const Programs &pg) {
-    if constexpr (PATH == kPathEager) {
-        return makespan_eager<S>(w, M);
+// Makespan of one decoded plan on path PATH (see makespan_fast for to_end,
+// the limit and the result; the short paths always finish).
+template <int S, int PATH, class Limit>
+__device__ __forceinline__ bool makespan_path(const StageW<S> &w, int M, const Programs &pg,
+                                              bool to_end, const Limit &limit, int32_t &T) {
+    T = -1;  // S = 1 has no short path
+    if constexpr (PATH == kPathFast) {
+        return makespan_fast<S>(w, M, to_end, limit, T);
+    } else if constexpr (PATH == kPathEager) {
+        return makespan_eager<S>(w, M, to_end, limit, T);
     } else if constexpr (PATH == kPathEagerShort) {
         const uint2 ix = __ldg(pg.index + (S - 1) * 32 + M);
-        return makespan_program<S>(w, pg.words + ix.x, (int)ix.y);
-    } else if constexpr (PATH == kPathEagerUnrolled) {
-        if constexpr (S > 1)
-            return makespan_eager_short_dispatch<S>(w, M, std::make_integer_sequence<int, 2 * S - 2>{});
-        else
-            return -1;  // S = 1 has no short case
+        T = makespan_program<S>(w, pg.words + ix.x, (int)ix.y);
     } else {
-        return makespan_1f1b<S, PATH>(w, M);
+        if constexpr (S > 1)
+            T = makespan_short_dispatch<S>(w, M, std::make_integer_sequence<int, S - 1>{});
     }
+    return true;
 }
 
 // Path of (schedule, S, M) and the first M of the fast path.

@@ -141,7 +141,7 @@ __device__ __forceinline__ int eval_key(int sched, uint32_t w, const int16_t *il
         if (S * V > POS_MAX_STAGES || M % S != 0) return -1;
         return kKeys + il_key[(S - 1) * 17 + V] + M / S;
     }
-    return M >= fast_min_m(sched, S) ? fast_key_begin(S) + M : generic_key_begin(S) + M;
+    return M >= fast_min_m(sched, S) ? fast_key_begin(S) + M : short_key_begin(M) + S - 1;
 }
 
 // global key histogram; invalid records are answered right here
@@ -502,8 +502,7 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
         p.dest = dest;
         p.offs = offs;
         p.cuts = cuts;
-        p.blob = h->d_blob;
-        p.lay = h->lay;
+        set_tables(p, h->d_blob, h->lay);
         for (int J = 1; J <= POS_MAX_STAGES; ++J) {  // smallest tripping M, by bisection
             int lo = 1, hi = 256;
             while (lo < hi) {
@@ -516,6 +515,7 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
         p.guard_m[0] = 0;
         p.pg = pg;
         p.nkeys = nk;
+        p.sms = sm_count();
         p.lim_off = h->lim_off;
         p.lim_w = h->lim_w;
         p.lim_bytes = h->lim_bytes;
@@ -561,13 +561,9 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
                 if (e == cudaSuccess) {
                     const cudaStream_t side = ss->s;
                     if (p.lay.sched == POS_SCHED_EAGER_1F1B) {
-                        if ((st = eval_eager_short_2_8(p, side)) == POS_OK &&
-                            (st = eval_eager_short_9_10(p, side)) == POS_OK &&
-                            (st = eval_eager_short_11_12(p, side)) == POS_OK &&
-                            (st = eval_eager_short_13_13(p, side)) == POS_OK &&
-                            (st = eval_eager_short_14_14(p, side)) == POS_OK &&
-                            (st = eval_eager_short_15_15(p, side)) == POS_OK &&
-                            (st = eval_eager_short_16_16(p, side)) == POS_OK &&
+                        if ((st = eval_eager_short_1_14(p, side)) == POS_OK &&
+                            (st = eval_eager_short_15_22(p, side)) == POS_OK &&
+                            (st = eval_eager_short_23_30(p, side)) == POS_OK &&
                             (st = eval_eager_1_6(p, side)) == POS_OK &&
                             (st = eval_eager_7_10(p, stream)) == POS_OK &&
                             (st = eval_eager_11_13(p, stream)) == POS_OK)
@@ -576,11 +572,8 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
                         // interleaved handle: the 1F1B ranges (records with
                         // V < 2, usually none) and the smallest interleaved
                         // range on the side, the other interleaved ranges here
-                        if ((st = eval_generic_2_8(p, side)) == POS_OK &&
-                            (st = eval_generic_9_12(p, side)) == POS_OK &&
-                            (st = eval_generic_13_14(p, side)) == POS_OK &&
-                            (st = eval_generic_15_15(p, side)) == POS_OK &&
-                            (st = eval_generic_16_16(p, side)) == POS_OK &&
+                        if ((st = eval_short_1_9(p, side)) == POS_OK &&
+                            (st = eval_short_10_15(p, side)) == POS_OK &&
                             (st = eval_fast_1_4(p, side)) == POS_OK &&
                             (st = eval_fast_5_8(p, side)) == POS_OK &&
                             (st = eval_fast_9_12(p, side)) == POS_OK &&
@@ -590,11 +583,8 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
                             (st = eval_il_12_22(p, stream)) == POS_OK &&
                             (st = eval_il_23_29(p, stream)) == POS_OK)
                             st = eval_il_32_33(p, stream);
-                    } else if ((st = eval_generic_2_8(p, side)) == POS_OK &&
-                               (st = eval_generic_9_12(p, side)) == POS_OK &&
-                               (st = eval_generic_13_14(p, side)) == POS_OK &&
-                               (st = eval_generic_15_15(p, side)) == POS_OK &&
-                               (st = eval_generic_16_16(p, side)) == POS_OK &&
+                    } else if ((st = eval_short_1_9(p, side)) == POS_OK &&
+                               (st = eval_short_10_15(p, side)) == POS_OK &&
                                (st = eval_fast_1_4(p, side)) == POS_OK &&
                                (st = eval_fast_5_8(p, stream)) == POS_OK &&
                                (st = eval_fast_9_12(p, stream)) == POS_OK) {

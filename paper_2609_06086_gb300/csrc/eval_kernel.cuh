@@ -8,16 +8,16 @@
 // costs ~6*S*M integer ops and its live registers grow with S (about 7*S),
 // so the batch is first counting-sorted by exact (S, M) (stream-ordered
 // scratch: every candidate's sorted position), and then a family of
-// kernels, each owning the candidates of one S range and either M >= S
-// (ramps unrolled, steady loop) or M < S (the whole schedule unrolled per
-// (S, M)), walks its contiguous range of the sorted records with launch
-// bounds matched to its register need.  Warps therefore see one (S, M)
+// kernels, each owning the candidates of one S range with M >= S (ramps
+// unrolled, steady loop) or of one M range with M < S (short_kernel), walks
+// its contiguous range of the sorted records with launch bounds matched to
+// its register need.  Warps therefore see one (S, M)
 // except at bucket boundaries, and no kernel waits at a block barrier after
 // staging the cost tables.
 //
 // Sort keys: fast path (M >= S for 1F1B, M >= 2S-1 for Eager 1F1B) ->
 // (S-1)*256 + M (the other slots of each S stay empty); short path ->
-// 4096 + (S-1)*32 + M; Interleaved 1F1B records with V >= 2 get keys after
+// 4096 + M*16 + S-1; Interleaved 1F1B records with V >= 2 get keys after
 // those (interleaved.cuh); records with S outside 1..16 or M = 0 are flagged
 // invalid by the sort pass and get no key.
 #pragma once
@@ -31,7 +31,7 @@ constexpr int kKeys = 4096 + 16 * 32;  // fast keys, then short-path keys
 constexpr int kEvalThreads = 128;
 
 __host__ __device__ inline int fast_key_begin(int S) { return (S - 1) * 256; }
-__host__ __device__ inline int generic_key_begin(int S) { return 4096 + (S - 1) * 32; }
+__host__ __device__ inline int short_key_begin(int M) { return 4096 + M * 16; }
 
 struct EvalParams {
     const uint4 *cands;    // 16-byte records (poseidon_eval_batch), or
@@ -54,11 +54,16 @@ struct EvalParams {
                            // kernels read 32 contiguous bytes and no record
     const void *blob;
     BlobLayout lay;
+    // the part of the blob that the makespan kernels stage: the timing
+    // tables, or with the memory tables before them for the interleaved ones
+    const void *tblob, *cblob;
+    BlobLayout tlay, clay;
     // guard_m[J]: the smallest M (1..255; 256 for none) at which the
     // overflow guard (guard_trips) trips for J (virtual) stages: U(J, M)
     // grows with M since every cost is non-negative
     uint16_t guard_m[POS_MAX_STAGES + 1];
     Programs pg;           // level programs of the schedule's short path
+    int sms;               // SMs of the device
     int nkeys;             // kKeys, or kKeysIl under Interleaved 1F1B
     int per_stage_tp;      // 1: records carry a TP index per stage (n_tp <= 4)
     // the handle's memory-limit table (Handle::lim_*): the decode pass stages
@@ -252,10 +257,11 @@ template <int PATH>
 struct EvalWith {
     template <int S>
     struct One {
-        // makespan of a decoded candidate (cuts packed by the decode pass)
-        static __device__ __forceinline__ void run(const Tab &t, const uint4 &rec,
+        // makespan of a decoded candidate (cuts packed by the decode pass);
+        // false when it was given up (to_end false, see makespan_fast)
+        static __device__ __forceinline__ bool run(const Tab &t, const uint4 &rec,
                                                    const uint4 &packed, const Programs &pg,
-                                                   int32_t &T) {
+                                                   bool to_end, int32_t &T) {
             // rec: x = per-stage TP code (0 for 16-byte records), z = type
             // code, w = S | M << 8 | tp << 16 | V << 24 (tp = 0 for 24-byte
             // records)
@@ -273,79 +279,256 @@ struct EvalWith {
             cut[S] = t.L();
             StageW<S> w;
             stage_weights<S>(t, cut, cls, w);
-            T = makespan_path<S, PATH>(w, M, pg);
+            return makespan_path<S, PATH>(w, M, pg, to_end, NoLimit{}, T);
         }
     };
 };
 
 template <int SLO, int SHI, int PATH>
-__device__ __forceinline__ void dispatch_range(int S, const Tab &t, const uint4 &rec,
+__device__ __forceinline__ bool dispatch_range(int S, const Tab &t, const uint4 &rec,
                                                const uint4 &packed, const Programs &pg,
-                                               int32_t &T) {
+                                               bool to_end, int32_t &T) {
 #define POS_EV(n)                                                                            \
-    if (n >= SLO && n <= SHI && S == n) {                                                    \
-        EvalWith<PATH>::template One<(n >= SLO && n <= SHI) ? n : SLO>::run(t, rec, packed, pg, T); \
-        return;                                                                              \
-    }
+    if (n >= SLO && n <= SHI && S == n)                                                      \
+        return EvalWith<PATH>::template One<(n >= SLO && n <= SHI) ? n : SLO>::run(          \
+            t, rec, packed, pg, to_end, T);
     POS_EV(1) POS_EV(2) POS_EV(3) POS_EV(4) POS_EV(5) POS_EV(6) POS_EV(7) POS_EV(8)
     POS_EV(9) POS_EV(10) POS_EV(11) POS_EV(12) POS_EV(13) POS_EV(14) POS_EV(15) POS_EV(16)
 #undef POS_EV
+    return true;
 }
 
 // Evaluates the sorted positions [offs[key_lo], offs[key_hi]): all
 // candidates with S in [SLO, SHI] on path PATH.
+//
+// Most plans need a few steady steps and some need nearly all (makespan_fast), so a warp that ran each of its 32 plans to the end
+// would run as long as the slowest.  A plan whose bounds still differ at
+// their first comparison is put on a queue of its warp instead, and 32 of
+// those are run to their end together.  A warp with at most two groups of
+// 32 plans has too few to fill such a group and runs every plan to its end
+// at once.
 template <int SLO, int SHI, int PATH, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
-    constexpr bool kFast = PATH == kPathFast || PATH == kPathEager;
-    const int key_lo = kFast ? fast_key_begin(SLO) : generic_key_begin(SLO);
-    const int key_hi = kFast ? fast_key_begin(SHI + 1) : generic_key_begin(SHI + 1);
+    constexpr int kWarps = kEvalThreads / 32;
+    __shared__ uint32_t s_queue[kWarps][64];
+    const int key_lo = fast_key_begin(SLO), key_hi = fast_key_begin(SHI + 1);
     // the key offsets come from the sort's scan, two or more kernels back
-    const int64_t begin = p.offs[key_lo], end = p.offs[key_hi];
+    const uint32_t begin = p.offs[key_lo], end = p.offs[key_hi];
     // blocks with no candidate (all of them when the range is empty) leave
     // without staging the tables, after the decode pass has completed
-    if ((int64_t)blockIdx.x * blockDim.x >= end - begin) {
+    if (end == begin) {
         grid_dep_wait();
         return;
     }
-    stage_blob(sm, p.blob, p.lay.bytes);
+    stage_blob(sm, p.tblob, p.tlay.bytes);
     __syncthreads();
     grid_dep_wait();  // the decoded records
     grid_dep_trigger();
-    const Tab t = tab_at(sm, p.lay);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const Tab t = tab_at(sm, p.tlay);
+    const int lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    uint32_t *queue = s_queue[threadIdx.x >> 5];
+    // blocks sms apart usually run on one SM: neighbours in the range, so
+    // that an SM's warps run the code of one stage count at a time
+    const uint32_t sms = (uint32_t)p.sms;
+    const uint32_t block = gridDim.x % sms == 0
+                               ? (blockIdx.x % sms) * (gridDim.x / sms) + blockIdx.x / sms
+                               : blockIdx.x;
+    const uint32_t warps = gridDim.x * kWarps, warp = block * kWarps + (threadIdx.x >> 5);
+    const uint32_t groups = (end - begin + 31) / 32;
+    const bool use_queue = groups > 2 * warps;
+    // The warp's groups of 32: every warps-th one, or, with a queue, two
+    // stretches (of half a warp's share each) as far from the range's middle
+    // as one another.  The plans of a stretch have one stage count and nearly
+    // one micro-batch count, so the queue's groups do too, and the cost of a
+    // plan grows over the range, so the two stretches balance.
+    const uint32_t half = use_queue ? (groups + 2 * warps - 1) / (2 * warps) : 0;
+    uint32_t g = use_queue ? warp * half : warp;
+    uint32_t g_end = use_queue ? min(groups, g + half) : groups;
+    bool second = !use_queue;  // no further stretch
+    int queued = 0;
     // whole warps iterate together (ballots below)
-    const int64_t span = ((end - begin) + 31) & ~(int64_t)31;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < span; j += stride) {
-        bool active = j < end - begin;
+    for (;;) {
+        if (g >= g_end && !second) {
+            second = true;
+            g = (2 * warps - 1 - warp) * half;
+            g_end = min(groups, g + half);
+        }
+        const bool from_queue = queued >= 32 || (queued > 0 && g >= g_end);
+        uint32_t j;
+        bool active;
+        if (from_queue) {
+            const int n = min(queued, 32);
+            queued -= n;
+            active = lane < n;
+            j = active ? queue[queued + lane] : 0u;
+            __syncwarp();  // read before later entries take their place
+        } else {
+            if (g >= g_end) break;
+            j = begin + 32 * g + lane;
+            active = j < end;
+            g += use_queue ? 1 : warps;
+        }
         uint32_t i = 0;
         uint4 rec = make_uint4(0, 0, 0, 0), packed = make_uint4(0, 0, 0, 0);
         if (active) {
-            packed = __ldcs(p.cuts + 2 * (begin + j));
-            const uint4 meta = __ldcs(p.cuts + 2 * (begin + j) + 1);
+            packed = __ldcs(p.cuts + 2 * (size_t)j);
+            const uint4 meta = __ldcs(p.cuts + 2 * (size_t)j + 1);
             active = (packed.w >> 24) == 0;  // not answered by the decode pass
             i = meta.x;
             rec = make_uint4(meta.w, 0u, meta.y, meta.z);
         }
         const int S = active ? (int)(rec.w & 0xff) : 0;
+        const bool to_end = from_queue || !use_queue;
         int32_t T = -1;
+        bool done = true;
         unsigned pending = __ballot_sync(0xffffffffu, active);
         while (pending) {
             const int leader = __ffs(pending) - 1;
             const int Sg = __shfl_sync(0xffffffffu, S, leader);
             const bool mine = active && S == Sg;
             const unsigned grp = __ballot_sync(0xffffffffu, mine);
-            if (mine) dispatch_range<SLO, SHI, PATH>(Sg, t, rec, packed, p.pg, T);
+            if (mine) done = dispatch_range<SLO, SHI, PATH>(Sg, t, rec, packed, p.pg, to_end, T);
             pending &= ~grp;
         }
-        if (active) p.T[i] = T;
+        if (active && done) p.T[i] = T;
+        const unsigned later = __ballot_sync(0xffffffffu, !done);
+        if (!done) queue[queued + __popc(later & lt_mask)] = j;
+        queued += __popc(later);
+        __syncwarp();
     }
 }
 
-template <int SLO, int SHI, int PATH, int MINB>
-pos_status launch_eval_range(const EvalParams &p, cudaStream_t stream) {
-    auto kern = eval_kernel<SLO, SHI, PATH, MINB>;
-    const int smem = p.lay.bytes;
+// Byte b (a runtime index) of a packed word, see push_cut.
+__device__ __forceinline__ int packed_byte(const uint4 &v, int b) {
+    const uint32_t w = b < 4 ? v.x : b < 8 ? v.y : b < 12 ? v.z : v.w;
+    return (int)((w >> (8 * (b & 3))) & 0xffu);
+}
+
+// Makespan of a decoded candidate of a short pipeline (see ShortProgram): S
+// and the grid stages at run time, the last C stages unrolled for this M.
+template <bool EAGER, int M>
+__device__ __forceinline__ int32_t makespan_short_one(const Tab &t, const uint4 &rec,
+                                                      const uint4 &packed) {
+    constexpr int C = short_stages(EAGER, M);
+    const int S = (int)(rec.w & 0xff), tp = (int)((rec.w >> 16) & 0xff), n_tp = t.n_tp();
+    const int G = S - C;  // grid stages 0..G-1
+    const uint32_t tcode = rec.z, tpc = rec.x;
+    auto class_of = [&](int s) { return stage_class(tcode, tpc, tp, n_tp, s); };
+    int32_t at[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) at[m] = 0;
+    int k = class_of(0), c = 0;
+#pragma unroll 1
+    for (int s = 0; s < G; ++s) {  // G < S: the next stage exists
+        const int c2 = packed_byte(packed, S - 2 - s), k2 = class_of(s + 1);
+        const Sums v = sums_from(t, k, sums(t, k, c), c2);
+        const int32_t pf = p2p(t, k, k2).x;
+        int32_t clock = 0;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            clock = max(at[m], clock) + v.f;
+            at[m] = clock + pf;
+        }
+        k = k2;
+        c = c2;
+    }
+    int32_t T = 0;
+    {
+        // the last C stages: cut[G + q] in byte C - 1 - q (1 <= q < C)
+        const uint32_t pw[4] = {packed.x, packed.y, packed.z, packed.w};
+        int cls[C], cut[C + 1];
+        cut[0] = c;
+#pragma unroll
+        for (int q = 1; q < C; ++q) cut[q] = packed_cut(pw, C, q);
+        cut[C] = t.L();
+#pragma unroll
+        for (int q = 0; q < C; ++q) cls[q] = class_of(G + q);
+        StageW<C> w;
+        stage_weights<C>(t, cut, cls, w);
+        int32_t Fo[C], Fp[C], Bo[C];
+#pragma unroll
+        for (int q = 0; q < C; ++q) Fo[q] = Fp[q] = Bo[q] = 0;
+        short_run<EAGER, M>(at, Fo, Fp, Bo, w,
+                            std::make_integer_sequence<int, ShortTab<EAGER, M>::value.n_levels>{});
+#pragma unroll
+        for (int q = 0; q < C; ++q) T = max(T, Bo[q] + w.d[q]);
+    }
+    int end = c;  // first layer of stage s + 1; k: its class
+#pragma unroll 1
+    for (int s = G - 1; s >= 0; --s) {
+        const int b = s > 0 ? packed_byte(packed, S - 1 - s) : 0, ks = class_of(s);
+        const Sums v = sums_from(t, ks, sums(t, ks, b), end);
+        const int32_t pb = p2p(t, ks, k).y;
+        int32_t clock = 0;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            clock = add_max(at[m], pb, clock) + v.b;
+            at[m] = clock;
+        }
+        T = max(T, clock + v.d);
+        k = ks;
+        end = b;
+    }
+    return T;
+}
+
+// runtime M in MLO..MHI -> its instance
+template <bool EAGER, int MLO, int... m>
+__device__ __forceinline__ int32_t short_dispatch(int M, const Tab &t, const uint4 &rec,
+                                                  const uint4 &packed,
+                                                  std::integer_sequence<int, m...>) {
+    int32_t T = -1;
+    ((M == MLO + m ? (T = makespan_short_one<EAGER, MLO + m>(t, rec, packed), 0) : 0), ...);
+    return T;
+}
+
+// Evaluates the sorted positions of the short pipelines with M in [MLO, MHI]
+// (sorted by M, then S: a warp's plans have one M except at a boundary).
+template <bool EAGER, int MLO, int MHI, int MINB>
+__global__ void __launch_bounds__(kEvalThreads, MINB) short_kernel(EvalParams p) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    // the key offsets come from the sort's scan, two or more kernels back
+    const uint32_t begin = p.offs[short_key_begin(MLO)], end = p.offs[short_key_begin(MHI + 1)];
+    if (blockIdx.x * blockDim.x >= end - begin) {
+        grid_dep_wait();
+        return;
+    }
+    stage_blob(sm, p.tblob, p.tlay.bytes);
+    __syncthreads();
+    grid_dep_wait();  // the decoded records
+    grid_dep_trigger();
+    const Tab t = tab_at(sm, p.tlay);
+    const uint32_t stride = gridDim.x * blockDim.x;
+    const uint32_t span = (end - begin + 31) & ~31u;  // whole warps iterate together
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < span; j += stride) {
+        bool active = j < end - begin;
+        uint32_t i = 0;
+        uint4 rec = make_uint4(0, 0, 0, 0), packed = make_uint4(0, 0, 0, 0);
+        if (active) {
+            packed = __ldcs(p.cuts + 2 * (size_t)(begin + j));
+            const uint4 meta = __ldcs(p.cuts + 2 * (size_t)(begin + j) + 1);
+            active = (packed.w >> 24) == 0;  // not answered by the decode pass
+            i = meta.x;
+            rec = make_uint4(meta.w, 0u, meta.y, meta.z);
+        }
+        const int M = active ? (int)((rec.w >> 8) & 0xff) : 0;
+        unsigned pending = __ballot_sync(0xffffffffu, active);
+        while (pending) {
+            const int Mg = __shfl_sync(0xffffffffu, M, __ffs(pending) - 1);
+            const bool mine = active && M == Mg;
+            if (mine)
+                p.T[i] = short_dispatch<EAGER, MLO>(Mg, t, rec, packed,
+                                                    std::make_integer_sequence<int, MHI - MLO + 1>{});
+            pending &= ~__ballot_sync(0xffffffffu, mine);
+        }
+    }
+}
+
+// Launch of a makespan kernel over the sorted records, as many blocks as fit.
+inline pos_status launch_ranged(void (*kern)(EvalParams), const EvalParams &p, int smem,
+                                cudaStream_t stream) {
     POS_TRY(ensure_smem(reinterpret_cast<const void *>(kern), smem));
     int per_sm = 0;
     POS_TRY(blocks_per_sm(reinterpret_cast<const void *>(kern), kEvalThreads, smem, &per_sm));
@@ -356,6 +539,26 @@ pos_status launch_eval_range(const EvalParams &p, cudaStream_t stream) {
     return POS_OK;
 }
 
+template <int SLO, int SHI, int PATH, int MINB>
+pos_status launch_eval_range(const EvalParams &p, cudaStream_t stream) {
+    return launch_ranged(eval_kernel<SLO, SHI, PATH, MINB>, p, p.tlay.bytes, stream);
+}
+template <bool EAGER, int MLO, int MHI, int MINB>
+pos_status launch_short_range(const EvalParams &p, cudaStream_t stream) {
+    return launch_ranged(short_kernel<EAGER, MLO, MHI, MINB>, p, p.tlay.bytes, stream);
+}
+
+// Sets the blob and the layouts of the parts that the kernels stage.
+inline void set_tables(EvalParams &p, const void *blob, const BlobLayout &lay) {
+    const unsigned char *b = static_cast<const unsigned char *>(blob);
+    p.blob = blob;
+    p.lay = lay;
+    p.tblob = b + lay.off_P;
+    p.tlay = timing_layout(lay);
+    p.cblob = b + lay.off_Pw;
+    p.clay = cost_layout(lay);
+}
+
 pos_status launch_decode(const EvalParams &p, cudaStream_t stream);
 
 // one launcher per instantiation unit (eval_range_*.cu)
@@ -363,21 +566,14 @@ pos_status eval_fast_1_4(const EvalParams &p, cudaStream_t s);
 pos_status eval_fast_5_8(const EvalParams &p, cudaStream_t s);
 pos_status eval_fast_9_12(const EvalParams &p, cudaStream_t s);
 pos_status eval_fast_13_16(const EvalParams &p, cudaStream_t s);
-pos_status eval_generic_2_8(const EvalParams &p, cudaStream_t s);
-pos_status eval_generic_9_12(const EvalParams &p, cudaStream_t s);
-pos_status eval_generic_13_14(const EvalParams &p, cudaStream_t s);
-pos_status eval_generic_15_15(const EvalParams &p, cudaStream_t s);
-pos_status eval_generic_16_16(const EvalParams &p, cudaStream_t s);
+pos_status eval_short_1_9(const EvalParams &p, cudaStream_t s);
+pos_status eval_short_10_15(const EvalParams &p, cudaStream_t s);
 pos_status eval_eager_1_6(const EvalParams &p, cudaStream_t s);
 pos_status eval_eager_7_10(const EvalParams &p, cudaStream_t s);
 pos_status eval_eager_11_13(const EvalParams &p, cudaStream_t s);
 pos_status eval_eager_14_16(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_2_8(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_9_10(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_11_12(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_13_13(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_14_14(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_15_15(const EvalParams &p, cudaStream_t s);
-pos_status eval_eager_short_16_16(const EvalParams &p, cudaStream_t s);
+pos_status eval_eager_short_1_14(const EvalParams &p, cudaStream_t s);
+pos_status eval_eager_short_15_22(const EvalParams &p, cudaStream_t s);
+pos_status eval_eager_short_23_30(const EvalParams &p, cudaStream_t s);
 
 }  // namespace pos

@@ -195,15 +195,17 @@ __device__ __forceinline__ void il_eval_one(const Tab &t, const uint4 &rec, cons
 #pragma unroll
     for (int d = 0; d < N; ++d) {
         dsum[d] = 0;
-        s.pf[d] = p2f(t, cls[d], cls[(d + 1) % N]);
-        s.pb[d] = p2b(t, cls[(d + 1) % N], cls[d]);
+        const int2 e = p2p(t, cls[d], cls[(d + 1) % N]);
+        s.pf[d] = e.x;
+        s.pb[d] = e.y;
     }
 #pragma unroll
     for (int j = 0; j < J; ++j) {
         const int k = cls[j % N];
-        s.F[j] = Pf(t, k, cut[j + 1]) - Pf(t, k, cut[j]);
-        s.B[j] = Pb(t, k, cut[j + 1]) - Pb(t, k, cut[j]);
-        dsum[j % N] += Pd(t, k, cut[j + 1]) - Pd(t, k, cut[j]);
+        const Sums v = sums_from(t, k, sums(t, k, cut[j]), cut[j + 1]);
+        s.F[j] = v.f;
+        s.B[j] = v.b;
+        dsum[j % N] += v.d;
     }
     il_makespan_ops<N, V>(s, q);
     int32_t best = 0;
@@ -237,11 +239,11 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) il_eval_kernel(EvalParams 
         grid_dep_wait();
         return;
     }
-    stage_blob(sm, p.blob, p.lay.bytes);
+    stage_blob(sm, p.cblob, p.clay.bytes);
     __syncthreads();
     grid_dep_wait();  // the decoded records
     grid_dep_trigger();
-    const Tab t = tab_at(sm, p.lay);
+    const Tab t = tab_at(sm, p.clay);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t span = ((end - begin) + 31) & ~(int64_t)31;
     int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) il_eval_kernel(EvalParams 
 template <int PLO, int PHI, int MINB>
 pos_status launch_il_range(const EvalParams &p, cudaStream_t stream) {
     auto kern = il_eval_kernel<PLO, PHI, MINB>;
-    const int smem = p.lay.bytes;
+    const int smem = p.clay.bytes;
     POS_TRY(ensure_smem(reinterpret_cast<const void *>(kern), smem));
     int per_sm = 0;
     POS_TRY(blocks_per_sm(reinterpret_cast<const void *>(kern), kEvalThreads, smem, &per_sm));

@@ -173,19 +173,19 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
         const uint32_t vslot = sr.vslot;
         for (int x = S - 1; x >= 0; --x) {
             const int k = sr.cls[x];
-            const int32_t pf = x + 1 < S ? p2f(t, k, sr.cls[x + 1]) : 0;
-            const int32_t pb = x + 1 < S ? p2b(t, sr.cls[x + 1], k) : 0;
+            const int2 e = x + 1 < S ? p2p(t, k, sr.cls[x + 1]) : make_int2(0, 0);
+            const int32_t pf = e.x, pb = e.y;
             int64_t v1 = INT64_MAX, v2 = INT64_MAX;
             int best_l = 0;
             if (c < L) {
                 const int most = lim[((size_t)sr.gid * S + x) * 128 + c];
-                const int32_t f0 = Pf(t, k, c), b0 = Pb(t, k, c), d0 = Pd(t, k, c);
+                const Sums at = sums(t, k, c);
                 const int l_lo = x == S - 1 ? L - c : 1;
                 const int l_hi = x == S - 1 ? L - c : min(most, L - c - (S - 1 - x));
                 for (int l = l_lo + part; l <= l_hi && l <= most; l += 4) {
                     const int c2 = c + l;
-                    const int64_t F = Pf(t, k, c2) - f0, B = Pb(t, k, c2) - b0;
-                    const int64_t d = Pd(t, k, c2) - d0;
+                    const Sums v = sums_from(t, k, at, c2);
+                    const int64_t F = v.f, B = v.b, d = v.d;
                     const int64_t a = (int64_t)M * (F + B);
                     int64_t w1, w2;
                     if (x == S - 1) {
@@ -360,7 +360,7 @@ __device__ __forceinline__ int last_true(int hi, Pred pred) {
 // parent cut c, class k of the new stage, prefix sums at c.
 struct ParentCtx {
     int c, k;
-    int32_t f0, b0, d0;
+    Sums at;  // prefix sums at c on class k
     int32_t pf, pb;  // prune 2: F and B edge between the new stage and the next one
     // ridge rule: state of the prefix, device types of the new and the next
     // stage, most layers the new stage may take (127: no cap)
@@ -383,9 +383,7 @@ __device__ __forceinline__ ParentCtx parent_ctx(const Tab &t, int k, int c) {
     ParentCtx q;
     q.c = c;
     q.k = k;
-    q.f0 = Pf(t, k, c);
-    q.b0 = Pb(t, k, c);
-    q.d0 = Pd(t, k, c);
+    q.at = sums(t, k, c);
     q.pf = 0;
     q.pb = 0;
     q.rstate = 0;
@@ -415,8 +413,8 @@ __device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, i
         int lo = 0;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1, c2 = q.c + mid;
-            const int64_t F = Pf(t, q.k, c2) - q.f0, B = Pb(t, q.k, c2) - q.b0;
-            const int64_t d = Pd(t, q.k, c2) - q.d0;
+            const Sums v = sums_from(t, q.k, q.at, c2);
+            const int64_t F = v.f, B = v.b, d = v.d;
             if ((uint64_t)(A + (int64_t)M * (F + B) + max(Bm, d)) * scale <= thr) lo = mid;
             else hi = mid - 1;
         }
@@ -452,8 +450,8 @@ __device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, i
                 for (int u = 0; u < 4; ++u) {
                     if (bb[u] < 0) continue;
                     const int c2 = 32 * wd + bb[u];
-                    const int64_t F = Pf(t, q.k, c2) - q.f0, B = Pb(t, q.k, c2) - q.b0;
-                    const int64_t d = Pd(t, q.k, c2) - q.d0;
+                    const Sums add = sums_from(t, q.k, q.at, c2);
+                    const int64_t F = add.f, B = add.b, d = add.d;
                     const int64_t A2 = A + F + q.pf, Bm2 = max(Bm, d) + B + q.pb;
                     if (v[u].x == kNoCompletion || (uint64_t)(A2 + v[u].x) * scale > thr ||
                         (uint64_t)(A2 + Bm2 + v[u].y) * scale > thr) {
@@ -488,8 +486,8 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
         int lo = 0;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1, c2 = c + mid;
-            const int64_t F = Pf(t, q.k, c2) - q.f0, B = Pb(t, q.k, c2) - q.b0;
-            const int64_t d = Pd(t, q.k, c2) - q.d0;
+            const Sums v = sums_from(t, q.k, q.at, c2);
+            const int64_t F = v.f, B = v.b, d = v.d;
             if ((uint64_t)(A + (int64_t)M * (F + B) + max(Bm, d)) * scale <= thr) lo = mid;
             else hi = mid - 1;
         }
@@ -505,7 +503,7 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
     const int lo = first - c;
     for (int i = 0; i < 4; ++i) acc.w[i] = 0;
     int n = 0;
-    const int32_t fbL = Pf(t, kb, L), bbL = Pb(t, kb, L), dbL = Pd(t, kb, L);
+    const Sums end = sums(t, kb, L);
     for (int l = lo; l <= hi; ++l) {
         const int c2 = c + l;
         // ridge rule for the last stage, after this one took l layers
@@ -514,10 +512,9 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
             continue;
         }
         if (p.prune) {
-            const int64_t Fa = Pf(t, q.k, c2) - q.f0, Ba = Pb(t, q.k, c2) - q.b0;
-            const int64_t da = Pd(t, q.k, c2) - q.d0;
-            const int64_t Fb = fbL - Pf(t, kb, c2), Bb = bbL - Pb(t, kb, c2);
-            const int64_t db = dbL - Pd(t, kb, c2);
+            const Sums va = sums_from(t, q.k, q.at, c2), vb = sums(t, kb, c2);
+            const int64_t Fa = va.f, Ba = va.b, da = va.d;
+            const int64_t Fb = end.f - vb.f, Bb = end.b - vb.b, db = end.d - vb.d;
             const int64_t g =
                 A + Fa + q.pf + (int64_t)M * (Fb + Bb) + max(max(Bm, da) + Ba + q.pb, db);
             if ((uint64_t)g * scale > thr) {
@@ -565,8 +562,8 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
         ParentCtx q = parent_ctx(t, sr.cls[X], c);
         const int kb = sr.cls[X + 1];  // X + 1 <= S - 1
         ridge_ctx(q, p.ridge != 0, pv.b.z, q.k, kb, t.n_tp());
-        const int32_t pf = p.prune == 2 ? p2f(t, q.k, kb) : 0;
-        const int32_t pb = p.prune == 2 ? p2b(t, kb, q.k) : 0;
+        const int2 edge = p.prune == 2 ? p2p(t, q.k, kb) : make_int2(0, 0);
+        const int32_t pf = edge.x, pb = edge.y;
         const uint64_t scale = sr.scale;
         const uint32_t gid = sr.gid;
         const int64_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
@@ -587,8 +584,8 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
             const bool in_mem = l <= hi_mem;
             bool g_ok = false, cand = false, ok = false;
             if (in_mem) {
-                const int64_t F = Pf(t, q.k, c2) - q.f0, B = Pb(t, q.k, c2) - q.b0;
-                const int64_t d = Pd(t, q.k, c2) - q.d0;
+                const Sums v = sums_from(t, q.k, q.at, c2);
+                const int64_t F = v.f, B = v.b, d = v.d;
                 g_ok = !p.prune ||
                        (uint64_t)(A + (int64_t)M * (F + B) + max(Bm, d)) * scale <= thr;
                 const uint32_t word2 = (c2 >> 5) == 0 ? f.x : (c2 >> 5) == 1 ? f.y
@@ -603,16 +600,15 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
                     const int64_t A2 = A + F + pf, Bm2 = max(Bm, d) + B + pb;
                     if (COMPLETE) {
                         if (p.prune) {
-                            const int64_t Fb = Pf(t, kb, L) - Pf(t, kb, c2);
-                            const int64_t Bb = Pb(t, kb, L) - Pb(t, kb, c2);
-                            const int64_t db = Pd(t, kb, L) - Pd(t, kb, c2);
+                            const Sums w = sums_from(t, kb, sums(t, kb, c2), L);
+                            const int64_t Fb = w.f, Bb = w.b, db = w.d;
                             ok = (uint64_t)(A2 + (int64_t)M * (Fb + Bb) + max(Bm2, db)) * scale <=
                                  thr;
                         }
                     } else if (p.prune == 2) {
-                        const int2 v = vrow[c2];
-                        ok = v.x != kNoCompletion && (uint64_t)(A2 + v.x) * scale <= thr &&
-                             (uint64_t)(A2 + Bm2 + v.y) * scale <= thr;
+                        const int2 n = vrow[c2];
+                        ok = n.x != kNoCompletion && (uint64_t)(A2 + n.x) * scale <= thr &&
+                             (uint64_t)(A2 + Bm2 + n.y) * scale <= thr;
                     }
                 }
             }
@@ -666,8 +662,8 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
                     set_byte<4 + X>(out, (uint32_t)c2);
                     store32(p.leaves + at, out);
                 } else {
-                    const int32_t F = Pf(t, q.k, c2) - q.f0, B = Pb(t, q.k, c2) - q.b0;
-                    const int32_t d = Pd(t, q.k, c2) - q.d0;
+                    const Sums v = sums_from(t, q.k, q.at, c2);
+                    const int32_t F = v.f, B = v.b, d = v.d;
                     out.a = pv.a;
                     out.b = make_uint4((uint32_t)((int32_t)pv.b.x + F + pf),
                                        (uint32_t)(max((int32_t)pv.b.y, d) + B + pb),
@@ -747,7 +743,7 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
         Bits128 acc = {{0u, 0u, 0u, 0u}};
         unsigned long long lb = 0, lm = 0, lr = 0;
         int n = 0;
-        ParentCtx q = {0, 0, 0, 0, 0};
+        ParentCtx q = {};
         if (live) {
             const SliceRec &sr = p.slices[slice];
             // X = depth of the parents = index of the stage placed here;
@@ -756,8 +752,9 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
             q = parent_ctx(t, sr.cls[X], c);
             ridge_ctx(q, p.ridge != 0, pv.b.z, sr.cls[X], sr.cls[X + 1], t.n_tp());
             if (p.prune == 2) {  // X + 1 <= S - 1: the next stage exists
-                q.pf = p2f(t, sr.cls[X], sr.cls[X + 1]);
-                q.pb = p2b(t, sr.cls[X + 1], sr.cls[X]);
+                const int2 e = p2p(t, sr.cls[X], sr.cls[X + 1]);
+                q.pf = e.x;
+                q.pb = e.y;
             }
             const uint64_t scale = sr.scale;
             const int64_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
@@ -807,9 +804,9 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
                     } else {
                         Vec32 ch = pv;
                         set_byte<2 + (X < 14 ? X : 0)>(ch, (uint32_t)c2);
-                        ch.b.x = (uint32_t)((int32_t)pv.b.x + (Pf(t, q.k, c2) - q.f0) + q.pf);
-                        ch.b.y = (uint32_t)(max((int32_t)pv.b.y, Pd(t, q.k, c2) - q.d0) +
-                                            (Pb(t, q.k, c2) - q.b0) + q.pb);
+                        const Sums v = sums_from(t, q.k, q.at, c2);
+                        ch.b.x = (uint32_t)((int32_t)pv.b.x + v.f + q.pf);
+                        ch.b.y = (uint32_t)(max((int32_t)pv.b.y, v.d) + v.b + q.pb);
                         ch.b.z = p.ridge ? ridge_next(q.rstate, q.rta, c2 - q.c) : 0u;
                         store32(p.out + pos++, ch);
                     }
@@ -1283,7 +1280,7 @@ static ExpandParams base_params(Search &s, const SliceRec *batch, int M) {
     p.inc = static_cast<const Key128 *>(s.d_inc.p);
     p.stats = s.stats;
     // level kernels read only the timing tables: stage that part alone
-    p.blob = static_cast<const unsigned char *>(s.h->d_blob) + s.h->lay.off_Pf;
+    p.blob = static_cast<const unsigned char *>(s.h->d_blob) + s.h->lay.off_P;
     p.lay = timing_layout(s.h->lay);
     return p;
 }
@@ -1551,7 +1548,7 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
             static_cast<const uint8_t *>(s.ws.d_lim.p), static_cast<int2 *>(s.ws.d_vb.p),
             static_cast<Leaf *>(s.ws.d_greedy.p), static_cast<unsigned long long *>(s.ws.d_lb.p),
             static_cast<const void *>(static_cast<const unsigned char *>(s.h->d_blob) +
-                                      s.h->lay.off_Pf),
+                                      s.h->lay.off_P),
             tl, s.stats));
         if (p->profile) POS_CUDA(cudaEventRecord(s.ev[1], s.stream));
         s.launches++;
@@ -1619,7 +1616,7 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
             d_all, static_cast<const uint32_t *>(s.ws.d_rows.p), nullptr, (int)rows.size(), s.S,
             static_cast<const uint8_t *>(s.ws.d_lim.p), static_cast<int2 *>(s.ws.d_vb.p),
             static_cast<Leaf *>(s.ws.d_greedy.p), static_cast<unsigned long long *>(s.ws.d_lb.p),
-            static_cast<const unsigned char *>(s.h->d_blob) + s.h->lay.off_Pf, tl, s.stats);
+            static_cast<const unsigned char *>(s.h->d_blob) + s.h->lay.off_P, tl, s.stats);
         POS_CUDA(cudaGetLastError());
         if (p->profile) POS_CUDA(cudaEventRecord(s.ev[1], s.stream));
         s.launches++;

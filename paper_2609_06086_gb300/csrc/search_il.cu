@@ -87,8 +87,8 @@ __device__ __forceinline__ void il_add(IlAcc<N> &a, const Tab &t, const int (&cl
     int k = cls[0];
 #pragma unroll
     for (int dd = 1; dd < N; ++dd) k = dd == d ? cls[dd] : k;
-    const int32_t F = Pf(t, k, c1) - Pf(t, k, c0), B = Pb(t, k, c1) - Pb(t, k, c0);
-    const int32_t D = Pd(t, k, c1) - Pd(t, k, c0);
+    const Sums v = sums_from(t, k, sums(t, k, c0), c1);
+    const int32_t F = v.f, B = v.b, D = v.d;
     const int64_t W = Pw(t, k, c1) - Pw(t, k, c0);
 #pragma unroll
     for (int dd = 0; dd < N; ++dd)
@@ -106,8 +106,9 @@ __device__ __forceinline__ void il_add(IlAcc<N> &a, const Tab &t, const int (&cl
         int kn = cls[0];
 #pragma unroll
         for (int dd = 0; dd < N; ++dd) kn = dd == (d + 1) % N ? cls[dd] : kn;
-        a.runF += F + p2f(t, k, kn);
-        a.runB += B + p2b(t, kn, k);
+        const int2 e = p2p(t, k, kn);
+        a.runF += F + e.x;
+        a.runB += B + e.y;
     }
     a.placed = i + 1;
 }
@@ -508,10 +509,11 @@ __global__ void __launch_bounds__(32 * kSeedWarps) il_seed_kernel(
             for (int c = lane; c <= L; c += 32) {
                 int32_t v = kSeedInf;
                 int al = 0;
-                const int32_t f0 = Pf(t, k, c < L ? c : L), b0 = Pb(t, k, c < L ? c : L);
+                const Sums at = sums(t, k, c);
                 if (j == J - 1) {
                     if (c < L) {
-                        v = M * (Pf(t, k, L) - f0 + Pb(t, k, L) - b0);
+                        const Sums all = sums_from(t, k, at, L);
+                        v = M * (all.f + all.b);
                         al = L - c;
                     }
                 } else {
@@ -519,8 +521,8 @@ __global__ void __launch_bounds__(32 * kSeedWarps) il_seed_kernel(
                     for (int l = 1; l <= lmax; ++l) {
                         const int32_t nb = best[(j + 1) * (L + 1) + c + l];
                         if (nb == kSeedInf) continue;
-                        const int32_t m =
-                            max(M * (Pf(t, k, c + l) - f0 + Pb(t, k, c + l) - b0), nb);
+                        const Sums part = sums_from(t, k, at, c + l);
+                        const int32_t m = max(M * (part.f + part.b), nb);
                         if (m < v) {
                             v = m;
                             al = l;
@@ -602,8 +604,7 @@ pos_status il_leaves(IlRun &r, const unsigned long long *count) {
     ep.F = static_cast<uint8_t *>(r.ws.il_F.p);
     ep.offs = static_cast<const uint32_t *>(r.ws.il_offs.p);
     ep.cuts = static_cast<uint4 *>(r.ws.il_rec.p);
-    ep.blob = r.blob;
-    ep.lay = r.lay;
+    set_tables(ep, r.blob, r.lay);
     ep.nkeys = kKeysIl;
     POS_TRY(eval_interleaved(ep, r.st));
     POS_TRY(ensure_smem(reinterpret_cast<const void *>(il_consider_kernel), r.lay.bytes));

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(256, leaf_min_blocks(S, PATH)) leaf_kernel(Lea
     // latency overlaps the current plan's wavefront
     Vec32 next = i < n ? load32(p.leaves + i) : none;
     for (; i < n_round; i += stride) {
-        unsigned long long obj = ~0ull, idx = ~0ull;
+        unsigned long long obj = ~0ull, idx = ~0ull, best = 0;
         const Vec32 lv = next;
         next = i + stride < n ? load32(p.leaves + i + stride) : none;
         const uint32_t sl = lv.a.x;
@@ -211,19 +211,26 @@ __global__ void __launch_bounds__(256, leaf_min_blocks(S, PATH)) leaf_kernel(Lea
             const uint64_t scale = __ldg(&sr.scale);
             // enumerated plans are ridge-like already; warm-up plans may not be
             cand = !p.ridge || ridge_plan_ok<S>(cut, cls, t.n_tp());
+            // A plan whose objective is above the incumbent's cannot lower
+            // it (the incumbent only decreases, so a stale read lets more
+            // through, never fewer), so its evaluation ends as soon as a
+            // lower bound shows that; warm-up plans that order the slices
+            // need their objective.
+            best = p.slice_best ? ~0ull : __ldcg(&p.inc->obj);
             StageW<S> w;
             stage_weights<S>(t, cut, cls, w);
-            const int32_t T = makespan_path<S, PATH>(w, p.M, p.pg);
+            int32_t T;
+            makespan_path<S, PATH>(w, p.M, p.pg, true, ObjLimit{scale, best}, T);
             obj = (unsigned long long)T * scale;
             ++evaluated;
-            if (p.slice_best) atomicMin(p.slice_best + sl, obj);  // ordering hint only
+            if (p.slice_best) {
+                atomicMin(p.slice_best + sl, obj);  // ordering hint only
+                best = __ldcg(&p.inc->obj);
+            }
         }
-        // A plan whose objective is above the incumbent's cannot lower it
-        // (the incumbent only decreases, so a stale read lets more through,
-        // never fewer): most warps stop here, and only the candidates pay
-        // for their global index (the composition's rank) and the warp
-        // minimum.
-        cand = cand && obj <= __ldcg(&p.inc->obj);
+        // most warps stop here, and only the candidates pay for their global
+        // index (the composition's rank) and the warp minimum
+        cand = cand && obj <= best;
         if (!__any_sync(0xffffffffu, cand)) continue;
         if (cand) {
             int cut[S + 1];

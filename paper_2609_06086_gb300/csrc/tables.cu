@@ -94,29 +94,33 @@ BlobLayout make_layout(int L, int n_types, int n_tp) {
     off = align16(off + K * Lp1 * 8);
     ly.off_cap = off;
     off = align16(off + K * 8);
-    ly.off_Pf = off;
-    off = align16(off + K * Lp1 * 4);
-    ly.off_Pb = off;
-    off = align16(off + K * Lp1 * 4);
-    ly.off_Pd = off;
-    off = align16(off + K * Lp1 * 4);
-    ly.off_p2f = off;
-    off = align16(off + K * K * 4);
-    ly.off_p2b = off;
-    off = align16(off + K * K * 4);
+    ly.off_P = off;
+    off = align16(off + K * Lp1 * 16);
+    ly.off_pp = off;
+    off = align16(off + K * K * 8);
     ly.bytes = off;
     return ly;
 }
 
 BlobLayout timing_layout(const BlobLayout &ly) {
     BlobLayout t = ly;
-    const int base = ly.off_Pf;
+    const int base = ly.off_P;
     t.off_binom = t.off_Pw = t.off_Pa = t.off_cap = -1;  // not staged
-    t.off_Pf -= base;
-    t.off_Pb -= base;
-    t.off_Pd -= base;
-    t.off_p2f -= base;
-    t.off_p2b -= base;
+    t.off_P -= base;
+    t.off_pp -= base;
+    t.bytes = ly.bytes - base;
+    return t;
+}
+
+BlobLayout cost_layout(const BlobLayout &ly) {
+    BlobLayout t = ly;
+    const int base = ly.off_Pw;
+    t.off_binom = -1;  // not staged
+    t.off_Pw -= base;
+    t.off_Pa -= base;
+    t.off_cap -= base;
+    t.off_P -= base;
+    t.off_pp -= base;
     t.bytes = ly.bytes - base;
     return t;
 }
@@ -124,39 +128,43 @@ BlobLayout timing_layout(const BlobLayout &ly) {
 BlobLayout memory_layout(const BlobLayout &ly) {
     BlobLayout t = ly;
     const int base = ly.off_Pw;
-    t.off_binom = t.off_Pf = t.off_Pb = t.off_Pd = t.off_p2f = t.off_p2b = -1;  // not staged
+    t.off_binom = t.off_P = t.off_pp = -1;  // not staged
     t.off_Pw -= base;
     t.off_Pa -= base;
     t.off_cap -= base;
-    t.bytes = ly.off_Pf - base;
+    t.bytes = ly.off_P - base;
     return t;
 }
 
-// One thread per (table, class) row: the raw per-layer row sits at entries
-// 1..L of the row; turn it into an exclusive prefix sum with P[0] = 0.
-__global__ void prefix_rows_kernel(unsigned char *blob, BlobLayout ly) {
+// One block per (table, class) row, a thread per layer: the raw per-layer
+// row sits at entries 1..L of the row; turn it into an exclusive prefix sum
+// with P[0] = 0.  Bound by latency: one load, a scan by shuffles within the
+// warps and over the four warp totals, one store per thread (a thread
+// walking its row took 13 us for 80 layers, now under 4).
+constexpr int kPrefixThreads = 128;
+static_assert(kPrefixThreads > POS_MAX_LAYERS, "a thread per layer");
+__global__ void __launch_bounds__(kPrefixThreads) prefix_rows_kernel(unsigned char *blob,
+                                                                     BlobLayout ly) {
     const int K = ly.K, Lp1 = ly.L + 1;
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= 5 * K) return;
-    const int table = row / K, k = row % K;
-    if (table < 2) {
-        int64_t *P = reinterpret_cast<int64_t *>(blob + (table == 0 ? ly.off_Pw : ly.off_Pa)) +
-                     (int64_t)k * Lp1;
-        int64_t acc = 0;
-        P[0] = 0;
-        for (int l = 1; l <= ly.L; ++l) {
-            acc += P[l];
-            P[l] = acc;
-        }
-    } else {
-        const int off = table == 2 ? ly.off_Pf : (table == 3 ? ly.off_Pb : ly.off_Pd);
-        int32_t *P = reinterpret_cast<int32_t *>(blob + off) + (int64_t)k * Lp1;
-        int32_t acc = 0;
-        P[0] = 0;
-        for (int l = 1; l <= ly.L; ++l) {
-            acc += P[l];
-            P[l] = acc;
-        }
+    const int table = blockIdx.x / K, k = blockIdx.x % K, l = threadIdx.x;
+    int64_t *P8 = reinterpret_cast<int64_t *>(blob + (table == 0 ? ly.off_Pw : ly.off_Pa)) +
+                  (int64_t)k * Lp1;
+    int32_t *P4 = reinterpret_cast<int32_t *>(blob + ly.off_P) + (int64_t)k * Lp1 * 4 + (table - 2);
+    int64_t v = 0;
+    if (l >= 1 && l <= ly.L) v = table < 2 ? P8[l] : (int64_t)P4[4 * l];
+    const int lane = l & 31, wid = l >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    __shared__ int64_t total[kPrefixThreads / 32];
+    if (lane == 31) total[wid] = v;
+    __syncthreads();
+    for (int w = 0; w < wid; ++w) v += total[w];
+    if (l <= ly.L) {
+        if (table < 2) P8[l] = v;
+        else P4[4 * l] = (int32_t)v;
     }
 }
 
@@ -232,21 +240,23 @@ pos_status build_blob(const pos_tables *t, int sched, std::vector<unsigned char>
     // raw rows at entries 1..L; prefix_rows_kernel turns them into sums
     int64_t *Pw_ = reinterpret_cast<int64_t *>(host.data() + ly.off_Pw);
     int64_t *Pa_ = reinterpret_cast<int64_t *>(host.data() + ly.off_Pa);
-    int32_t *Pf_ = reinterpret_cast<int32_t *>(host.data() + ly.off_Pf);
-    int32_t *Pb_ = reinterpret_cast<int32_t *>(host.data() + ly.off_Pb);
-    int32_t *Pd_ = reinterpret_cast<int32_t *>(host.data() + ly.off_Pd);
+    int32_t *P_ = reinterpret_cast<int32_t *>(host.data() + ly.off_P);
+    int32_t *pp_ = reinterpret_cast<int32_t *>(host.data() + ly.off_pp);
     for (int k = 0; k < K; ++k)
         for (int l = 0; l < L; ++l) {
             const int64_t src = (int64_t)k * L + l, dst = (int64_t)k * Lp1 + l + 1;
             Pw_[dst] = t->mem_w[src];
             Pa_[dst] = t->mem_a[src];
-            Pf_[dst] = t->fwd[src];
-            Pb_[dst] = t->bwd[src];
-            Pd_[dst] = t->dsync[src];
+            P_[4 * dst] = t->fwd[src];
+            P_[4 * dst + 1] = t->bwd[src];
+            P_[4 * dst + 2] = t->dsync[src];
         }
     std::memcpy(host.data() + ly.off_cap, t->cap, sizeof(int64_t) * K);
-    std::memcpy(host.data() + ly.off_p2f, t->p2p_f, sizeof(int32_t) * K * K);
-    std::memcpy(host.data() + ly.off_p2b, t->p2p_b, sizeof(int32_t) * K * K);
+    for (int a = 0; a < K; ++a)
+        for (int b = 0; b < K; ++b) {
+            pp_[2 * (a * K + b)] = t->p2p_f[a * K + b];
+            pp_[2 * (a * K + b) + 1] = t->p2p_b[b * K + a];
+        }
     int64_t A = 0, D = 0, P = 0;
     for (int l = 0; l < L; ++l) {
         int64_t mfb = 0, md = 0;
@@ -267,8 +277,7 @@ pos_status build_blob(const pos_tables *t, int sched, std::vector<unsigned char>
 }
 
 pos_status launch_prefix_rows(void *d_blob, const BlobLayout &ly, cudaStream_t stream) {
-    const int rows = 5 * ly.K;
-    prefix_rows_kernel<<<(rows + 127) / 128, 128, 0, stream>>>(
+    prefix_rows_kernel<<<5 * ly.K, kPrefixThreads, 0, stream>>>(
         static_cast<unsigned char *>(d_blob), ly);
     POS_CUDA(cudaGetLastError());
     return POS_OK;
