@@ -208,7 +208,8 @@ pos_status poseidon_eval_batch_ex(void *handle, const pos_candidate_ex *d_cands,
 /*
  * Same as poseidon_eval_batch but with HOST buffers: copies the candidates
  * to the device, evaluates, copies the results back and synchronises.
- * Allocates n*21 bytes of device memory for the duration of the call.
+ * Takes n*21 bytes from the library's memory pool for the duration of the
+ * call (the default stream orders the work).
  */
 pos_status poseidon_eval_batch_host(void *handle, const pos_candidate *cands, int64_t n,
                                     int32_t *makespan, uint8_t *feasible);

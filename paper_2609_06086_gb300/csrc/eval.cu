@@ -463,15 +463,45 @@ static pos_status side_stream(SideStream **out) {
     return POS_OK;
 }
 
+// Kernel parameters of candidates [base, base + m) of a batch, without the
+// sorted path's scratch.
+static EvalParams eval_params(const Handle *h, const void *d_cands, bool per_stage_tp, int64_t base,
+                              int64_t m, int32_t *d_T, uint8_t *d_F) {
+    EvalParams p = {};
+    p.per_stage_tp = per_stage_tp ? 1 : 0;
+    p.cands = per_stage_tp ? nullptr : static_cast<const uint4 *>(d_cands) + base;
+    p.cands_ex = per_stage_tp ? static_cast<const uint2 *>(d_cands) + 3 * base : nullptr;
+    p.n = m;
+    p.T = d_T + base;
+    p.F = d_F + base;
+    set_tables(p, h->d_blob, h->lay);
+    for (int J = 1; J <= POS_MAX_STAGES; ++J) {  // smallest tripping M, by bisection
+        int lo = 1, hi = 256;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (guard_trips(h->guard_A, h->guard_D, h->guard_P, J, mid)) hi = mid;
+            else lo = mid + 1;
+        }
+        p.guard_m[J] = (uint16_t)lo;
+    }
+    p.guard_m[0] = 0;
+    p.sms = sm_count();
+    p.lim_off = h->lim_off;
+    p.lim_w = h->lim_w;
+    p.lim_bytes = h->lim_bytes;
+    return p;
+}
+
 // d_cands: 16-byte records, or 24-byte records when per_stage_tp.
 pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_t n,
                        int32_t *d_T, uint8_t *d_F, cudaStream_t stream) {
     if (n == 0) return POS_OK;
+    const bool il = h->lay.sched == POS_SCHED_INTERLEAVED_1F1B;
+    if (n <= lane_max(h->lay.sched))
+        return launch_lanes(eval_params(h, d_cands, per_stage_tp, 0, n, d_T, d_F), stream);
     cudaMemPool_t pool;
     pos_status st = scratch_pool(&pool);
     if (st != POS_OK) return st;
-    Programs pg;  // the schedule's level programs (Eager 1F1B, few micro-batches)
-    if ((st = schedule_programs(h->lay.sched, &pg)) != POS_OK) return st;
     // batches above 2^24 candidates go in chunks of 2^24: a chunk's outputs
     // (5 bytes per candidate, 80 MB), written in sorted order and so
     // scattered over the output arrays, stay in L2 until whole sectors are
@@ -480,7 +510,6 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
     for (int64_t base = 0; base < n; base += chunk) {
         const int64_t m = std::min(chunk, n - base);
         void *scratch = nullptr;
-        const bool il = h->lay.sched == POS_SCHED_INTERLEAVED_1F1B;
         const int nk = il ? kKeysIl : kKeys;
         // scratch: decoded records (32 B per candidate), the sort arrays, the keys
         const size_t sbytes = 32 * (size_t)m + sizeof(uint32_t) * (3 * (size_t)nk + 1 + (size_t)m) +
@@ -492,33 +521,11 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
         uint32_t *cursor = offs + nk + 1;
         uint32_t *dest = cursor + nk;
         uint16_t *keys = reinterpret_cast<uint16_t *>(dest + m);
-        EvalParams p;
-        p.per_stage_tp = per_stage_tp ? 1 : 0;
-        p.cands = per_stage_tp ? nullptr : static_cast<const uint4 *>(d_cands) + base;
-        p.cands_ex = per_stage_tp ? static_cast<const uint2 *>(d_cands) + 3 * base : nullptr;
-        p.n = m;
-        p.T = d_T + base;
-        p.F = d_F + base;
+        EvalParams p = eval_params(h, d_cands, per_stage_tp, base, m, d_T, d_F);
         p.dest = dest;
         p.offs = offs;
         p.cuts = cuts;
-        set_tables(p, h->d_blob, h->lay);
-        for (int J = 1; J <= POS_MAX_STAGES; ++J) {  // smallest tripping M, by bisection
-            int lo = 1, hi = 256;
-            while (lo < hi) {
-                const int mid = (lo + hi) / 2;
-                if (guard_trips(h->guard_A, h->guard_D, h->guard_P, J, mid)) hi = mid;
-                else lo = mid + 1;
-            }
-            p.guard_m[J] = (uint16_t)lo;
-        }
-        p.guard_m[0] = 0;
-        p.pg = pg;
         p.nkeys = nk;
-        p.sms = sm_count();
-        p.lim_off = h->lim_off;
-        p.lim_w = h->lim_w;
-        p.lim_bytes = h->lim_bytes;
         // histogram pass: 256 threads, four candidates per thread and round
         const int grid = (int)std::max<int64_t>(
             1, std::min<int64_t>((m + 1023) / 1024, 4LL * sm_count()));
@@ -643,21 +650,27 @@ pos_status poseidon_eval_batch_host(void *handle, const pos_candidate *cands, in
     if (n < 0) return pos::fail(POS_EINVAL, "n < 0");
     if (n == 0) return POS_OK;
     if (!cands || !makespan || !feasible) return pos::fail(POS_EINVAL, "NULL buffer");
+    // stream-ordered on the default stream, from the library's pool: a
+    // cudaMalloc and cudaFree pair takes 60 us per call here
+    cudaMemPool_t pool;
+    POS_TRY(pos::scratch_pool(&pool));
     void *d = nullptr;
     const size_t bc = sizeof(pos_candidate) * (size_t)n, bt = sizeof(int32_t) * (size_t)n;
-    POS_CUDA(cudaMalloc(&d, bc + bt + (size_t)n));
+    POS_CUDA(cudaMallocFromPoolAsync(&d, bc + bt + (size_t)n, pool, 0));
     pos_candidate *dc = static_cast<pos_candidate *>(d);
     int32_t *dt = reinterpret_cast<int32_t *>(static_cast<char *>(d) + bc);
     uint8_t *df = reinterpret_cast<uint8_t *>(static_cast<char *>(d) + bc + bt);
     pos_status st = POS_OK;
-    cudaError_t e = cudaMemcpy(dc, cands, bc, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(dc, cands, bc, cudaMemcpyHostToDevice, 0);
     if (e == cudaSuccess) {
         st = pos::launch_eval(static_cast<pos::Handle *>(handle), dc, false, n, dt, df, 0);
-        if (st == POS_OK) e = cudaMemcpy(makespan, dt, bt, cudaMemcpyDeviceToHost);
+        if (st == POS_OK) e = cudaMemcpyAsync(makespan, dt, bt, cudaMemcpyDeviceToHost, 0);
         if (st == POS_OK && e == cudaSuccess)
-            e = cudaMemcpy(feasible, df, (size_t)n, cudaMemcpyDeviceToHost);
+            e = cudaMemcpyAsync(feasible, df, (size_t)n, cudaMemcpyDeviceToHost, 0);
     }
-    cudaFree(d);
+    const cudaError_t e2 = cudaFreeAsync(d, 0);
+    const cudaError_t e3 = cudaStreamSynchronize(0);
+    if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
     if (e != cudaSuccess) return pos::cuda_fail(e, "eval_batch_host copies");
     return st;
 }

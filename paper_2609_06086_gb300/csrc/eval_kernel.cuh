@@ -62,7 +62,6 @@ struct EvalParams {
     // overflow guard (guard_trips) trips for J (virtual) stages: U(J, M)
     // grows with M since every cost is non-negative
     uint16_t guard_m[POS_MAX_STAGES + 1];
-    Programs pg;           // level programs of the schedule's short path
     int sms;               // SMs of the device
     int nkeys;             // kKeys, or kKeysIl under Interleaved 1F1B
     int per_stage_tp;      // 1: records carry a TP index per stage (n_tp <= 4)
@@ -260,8 +259,8 @@ struct EvalWith {
         // makespan of a decoded candidate (cuts packed by the decode pass);
         // false when it was given up (to_end false, see makespan_fast)
         static __device__ __forceinline__ bool run(const Tab &t, const uint4 &rec,
-                                                   const uint4 &packed, const Programs &pg,
-                                                   bool to_end, int32_t &T) {
+                                                   const uint4 &packed, bool to_end,
+                                                   int32_t &T) {
             // rec: x = per-stage TP code (0 for 16-byte records), z = type
             // code, w = S | M << 8 | tp << 16 | V << 24 (tp = 0 for 24-byte
             // records)
@@ -279,19 +278,18 @@ struct EvalWith {
             cut[S] = t.L();
             StageW<S> w;
             stage_weights<S>(t, cut, cls, w);
-            return makespan_path<S, PATH>(w, M, pg, to_end, NoLimit{}, T);
+            return makespan_path<S, PATH>(w, M, Programs{}, to_end, NoLimit{}, T);
         }
     };
 };
 
 template <int SLO, int SHI, int PATH>
 __device__ __forceinline__ bool dispatch_range(int S, const Tab &t, const uint4 &rec,
-                                               const uint4 &packed, const Programs &pg,
-                                               bool to_end, int32_t &T) {
+                                               const uint4 &packed, bool to_end, int32_t &T) {
 #define POS_EV(n)                                                                            \
     if (n >= SLO && n <= SHI && S == n)                                                      \
         return EvalWith<PATH>::template One<(n >= SLO && n <= SHI) ? n : SLO>::run(          \
-            t, rec, packed, pg, to_end, T);
+            t, rec, packed, to_end, T);
     POS_EV(1) POS_EV(2) POS_EV(3) POS_EV(4) POS_EV(5) POS_EV(6) POS_EV(7) POS_EV(8)
     POS_EV(9) POS_EV(10) POS_EV(11) POS_EV(12) POS_EV(13) POS_EV(14) POS_EV(15) POS_EV(16)
 #undef POS_EV
@@ -389,7 +387,7 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) 
             const int Sg = __shfl_sync(0xffffffffu, S, leader);
             const bool mine = active && S == Sg;
             const unsigned grp = __ballot_sync(0xffffffffu, mine);
-            if (mine) done = dispatch_range<SLO, SHI, PATH>(Sg, t, rec, packed, p.pg, to_end, T);
+            if (mine) done = dispatch_range<SLO, SHI, PATH>(Sg, t, rec, packed, to_end, T);
             pending &= ~grp;
         }
         if (active && done) p.T[i] = T;
@@ -560,6 +558,17 @@ inline void set_tables(EvalParams &p, const void *blob, const BlobLayout &lay) {
 }
 
 pos_status launch_decode(const EvalParams &p, cudaStream_t stream);
+
+// Batches up to this many candidates take the lane-per-stage kernel of
+// eval_lanes.cu.  Random plans of 64 layers, 2..16 stages and 8..128
+// micro-batches on a GB300, lanes / sorted path: 1F1B 14.9 / 68 us at 3,001,
+// 36.6 / 63 us at 32,768 and 61.5 / 70 us at 65,536; Eager 1F1B 18.6 / 120,
+// 59.6 / 88 and 104.9 / 104 us.  The limits stay below the crossing because
+// plans that reach the steady state late cost the lanes more.
+inline int64_t lane_max(int sched) {
+    return sched == POS_SCHED_1F1B ? 49152 : sched == POS_SCHED_EAGER_1F1B ? 32768 : 0;
+}
+pos_status launch_lanes(const EvalParams &p, cudaStream_t stream);
 
 // one launcher per instantiation unit (eval_range_*.cu)
 pos_status eval_fast_1_4(const EvalParams &p, cudaStream_t s);
