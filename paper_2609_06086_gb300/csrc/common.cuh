@@ -143,8 +143,44 @@ pos_status build_blob(const pos_tables *t, int sched, std::vector<unsigned char>
                       BlobLayout &ly, int64_t &guard_A, int64_t &guard_D, int64_t &guard_P);
 // device part: per-class prefix sums in place, asynchronous on `stream`
 pos_status launch_prefix_rows(void *d_blob, const BlobLayout &ly, cudaStream_t stream);
+// lim[k][w-1][a] (K * wmax * (L+1) bytes, see Handle): asynchronous, after
+// the kernel queued before it on the stream (the prefix sums)
+pos_status launch_lim(const void *d_blob, const BlobLayout &ly, int wmax, uint8_t *lim,
+                      cudaStream_t stream);
 void destroy_handle(Handle *h);
 int sm_count();
+
+// One block (kPrefixThreads threads) per row of the five per-class tables, a
+// thread per layer: the raw per-layer row sits at entries 1..L of the row;
+// turn it into an exclusive prefix sum with P[0] = 0.  Bound by latency: one
+// load, a scan by shuffles within the warps and over the four warp totals,
+// one store per thread (a thread walking its row took 13 us for 80 layers,
+// now under 4).
+constexpr int kPrefixThreads = 128;
+static_assert(kPrefixThreads > POS_MAX_LAYERS, "a thread per layer");
+__device__ __forceinline__ void prefix_row(unsigned char *blob, const BlobLayout &ly, int row) {
+    const int K = ly.K, Lp1 = ly.L + 1;
+    const int table = row / K, k = row % K, l = threadIdx.x;
+    int64_t *P8 = reinterpret_cast<int64_t *>(blob + (table == 0 ? ly.off_Pw : ly.off_Pa)) +
+                  (int64_t)k * Lp1;
+    int32_t *P4 = reinterpret_cast<int32_t *>(blob + ly.off_P) + (int64_t)k * Lp1 * 4 + (table - 2);
+    int64_t v = 0;
+    if (l >= 1 && l <= ly.L) v = table < 2 ? P8[l] : (int64_t)P4[4 * l];
+    const int lane = l & 31, wid = l >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    __shared__ int64_t total[kPrefixThreads / 32];
+    if (lane == 31) total[wid] = v;
+    __syncthreads();
+    for (int w = 0; w < wid; ++w) v += total[w];
+    if (l <= ly.L) {
+        if (table < 2) P8[l] = v;
+        else P4[4 * l] = (int32_t)v;
+    }
+}
 
 // View of the blob staged in shared memory.  It keeps the shared-memory
 // base and a pointer to the layout in kernel parameter space; every access

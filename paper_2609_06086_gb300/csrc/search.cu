@@ -50,63 +50,80 @@ __device__ __forceinline__ int popc128(const Bits128 &b) {
 }
 
 // ---------------------------------------------------------------------------
-// suffix feasibility: one block per slice, thread c
+// suffix feasibility: one warp per slice, lane j on the starts c = j + 32 q
 // ---------------------------------------------------------------------------
-// Also fills lim[(gid*S + x)*128 + c] = the largest l such that stage x
-// holds layers [c, c+l) within memory (0 if none), capped at L - c, and
-// root[gid] = 1 when the slice has a memory-feasible plan.
-__global__ void feas_kernel(const SliceRec *slices, int n_slices, int S, uint4 *feas,
-                            uint8_t *lim, uint8_t *root, const void *blob, BlobLayout lay,
-                            unsigned long long *stats) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ uint32_t prev[4], cur[4];
-    __shared__ uint64_t bar;
-    if (!stage_blob_bulk(sm, blob, lay.bytes, &bar)) {
-        if (threadIdx.x == 0) atomicAdd(stats + kStBulkTimeout, 1ull);
-        return;
-    }
-    const Tab t = tab_at(sm, lay);
-    const int L = lay.L, c = threadIdx.x;
-    for (int sl = blockIdx.x; sl < n_slices; sl += gridDim.x) {
+// From the last stage back: a start c of stage x is feasible when some end in
+// (c, limtab] is a feasible start of stage x + 1, where limtab[k][w-1][c]
+// (lim_kernel) is the largest end that class k holds from c with w
+// micro-batches in flight, so a stage costs a byte load per start and a few
+// bit operations (a binary search over the memory sums by a block per slice
+// before: 1262 us for 168,000 slices, 420 of them feasible).  A slice whose
+// set empties on the way is infeasible and left alone; only the feasible ones
+// write their rows: feas[gid*(S+1) + x], lim[(gid*S + x)*128 + c] = the most
+// layers stage x holds from c (0 if none).  root[gid] = 1 when the slice has a
+// memory-feasible plan.
+constexpr int kFeasThreads = 128;
+
+__global__ void __launch_bounds__(kFeasThreads) feas_kernel(const SliceRec *slices, int n_slices,
+                                                            int S, const uint8_t *limtab, int wmax,
+                                                            uint4 *feas, uint8_t *lim,
+                                                            uint8_t *root, int L, int sched) {
+    __shared__ uint4 s_rows[kFeasThreads / 32][POS_MAX_STAGES + 1];
+    const int lane = threadIdx.x & 31;
+    uint4 *rows = s_rows[threadIdx.x >> 5];
+    grid_dep_wait();  // the slices and the memory limits
+    grid_dep_trigger();
+    const int warps = gridDim.x * (kFeasThreads / 32);
+    for (int sl = blockIdx.x * (kFeasThreads / 32) + (threadIdx.x >> 5); sl < n_slices; sl += warps) {
         const SliceRec &sr = slices[sl];
         const int M = sr.M;
-        uint4 *row = feas + (size_t)sr.gid * (S + 1);
+        const uint4 cw = *reinterpret_cast<const uint4 *>(sr.cls);
+        auto limits = [&](int x) {
+            const uint32_t w = (x >> 2) == 0 ? cw.x : (x >> 2) == 1 ? cw.y : (x >> 2) == 2 ? cw.z : cw.w;
+            const int k = (int)((w >> (8 * (x & 3))) & 0xffu);
+            return limtab + (size_t)(k * wmax + inflight(sched, S, M, x) - 1) * (L + 1);
+        };
         // x = S: only the empty suffix starting at c = L
-        if (c < 4) prev[c] = (L >> 5) == c ? (1u << (L & 31)) : 0u;
-        __syncthreads();
-        if (c == 0) row[S] = make_uint4(prev[0], prev[1], prev[2], prev[3]);
-        for (int x = S - 1; x >= 0; --x) {
-            bool ok = false;
-            int most = 0;
-            if (c < L) {
-                // memory grows with the layer count: binary search for the
-                // largest l that fits, then any suffix start in (c, c+l]
-                const int k = sr.cls[x];
-                int lo = 0, hi = L - c;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (stage_fits(t, S, M, x, k, c, c + mid)) lo = mid;
-                    else hi = mid - 1;
+        Bits128 prev = range_bits(L, L);
+        if (lane == 0) rows[S] = make_uint4(prev.w[0], prev.w[1], prev.w[2], prev.w[3]);
+        bool some = true;
+        for (int x = S - 1; x >= 0 && some; --x) {
+            const uint8_t *most = limits(x);
+            Bits128 cur;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int c = lane + 32 * q;
+                bool ok = false;
+                if (c < L) {
+                    const Bits128 win = range_bits(c + 1, (int)__ldg(most + c));
+                    ok = ((prev.w[0] & win.w[0]) | (prev.w[1] & win.w[1]) | (prev.w[2] & win.w[2]) |
+                          (prev.w[3] & win.w[3])) != 0u;
                 }
-                most = lo;
-                const Bits128 win = range_bits(c + 1, c + most);
-                ok = ((prev[0] & win.w[0]) | (prev[1] & win.w[1]) | (prev[2] & win.w[2]) |
-                      (prev[3] & win.w[3])) != 0u;
+                cur.w[q] = __ballot_sync(0xffffffffu, ok);
             }
-            if (c < 128) lim[((size_t)sr.gid * S + x) * 128 + c] = (uint8_t)most;
-            const unsigned b = __ballot_sync(0xffffffffu, ok);
-            if ((c & 31) == 0) cur[c >> 5] = b;
-            __syncthreads();
-            if (c < 4) prev[c] = cur[c];
-            __syncthreads();
-            if (c == 0) row[x] = make_uint4(prev[0], prev[1], prev[2], prev[3]);
+            prev = cur;
+            some = (prev.w[0] | prev.w[1] | prev.w[2] | prev.w[3]) != 0u;
+            if (lane == 0) rows[x] = make_uint4(prev.w[0], prev.w[1], prev.w[2], prev.w[3]);
         }
-        // root[gid] = the whole model fits the slice's stages (bit c = 0 of row 0)
-        if (c == 0) root[sr.gid] = (uint8_t)(prev[0] & 1u);
-        __syncthreads();
+        // root: the whole model fits the slice's stages (bit c = 0 of row 0)
+        const bool fits = some && (prev.w[0] & 1u);
+        if (lane == 0) root[sr.gid] = fits ? 1 : 0;
+        __syncwarp();
+        if (fits) {
+            if (lane <= S) feas[(size_t)sr.gid * (S + 1) + lane] = rows[lane];
+            for (int x = 0; x < S; ++x) {
+                const uint8_t *most = limits(x);
+                uint8_t *out = lim + ((size_t)sr.gid * S + x) * 128;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int c = lane + 32 * q;
+                    out[c] = c < L ? (uint8_t)(__ldg(most + c) - c) : 0;
+                }
+            }
+        }
+        __syncwarp();  // the rows are rewritten for the next slice
     }
 }
-
 
 // ---------------------------------------------------------------------------
 // completion bounds (prune mode 2).  For a complete plan and 0-based stages
@@ -135,14 +152,16 @@ __global__ void feas_kernel(const SliceRec *slices, int n_slices, int S, uint4 *
 // keeps the smallest l attaining V1[x][c], and thread 0 follows it from
 // (0, 0) to write the slice's argmin completion as a plan: a memory-feasible
 // plan whose makespan is usually close to the slice's best (warm-up seed).
-// root_lb[slice] = V1[0][0] * scale, a lower bound on the slice's objective.
+// root_lb[r] = V1[0][0] * scale, a lower bound on the objective of row r's
+// slice.
 constexpr int kBoundThreads = 512;
 
-// rows = NULL: row r is slice r, for every slice (n_rows = the slice count);
+// Row r is slice rows[r], whose table row (vslot) it becomes.  rows = NULL:
+// row r is slice r, for every slice (n_rows = the slice count);
 // a slice whose root is infeasible (root[r] == 0) then gets a hole for its
 // greedy plan and an infinite root bound, and no table rows.
 __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
-    const SliceRec *slices, const uint32_t *rows, const uint8_t *root, int n_rows, int S,
+    SliceRec *slices, const uint32_t *rows, const uint8_t *root, int n_rows, int S,
     const uint8_t *lim, int2 *vb, Leaf *greedy, unsigned long long *root_lb, const void *blob,
     BlobLayout lay, unsigned long long *stats) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -164,13 +183,14 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
             if (threadIdx.x == 0) {
                 const Vec32 hole = {make_uint4(kLeafHole, 0, 0, 0), make_uint4(0, 0, 0, 0)};
                 store32(greedy + r, hole);
-                root_lb[sl] = ~0ull;
+                root_lb[r] = ~0ull;
             }
             continue;
         }
         const SliceRec &sr = slices[sl];
         const int M = sr.M;
-        const uint32_t vslot = sr.vslot;
+        const uint32_t vslot = (uint32_t)r;
+        if (rows && threadIdx.x == 0) slices[sl].vslot = vslot;
         for (int x = S - 1; x >= 0; --x) {
             const int k = sr.cls[x];
             const int2 e = x + 1 < S ? p2p(t, k, sr.cls[x + 1]) : make_int2(0, 0);
@@ -241,10 +261,32 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
             store32(greedy + r, lf);
             // the slice's root bound V1[0][0] = min over plans of max_y P(y, y),
             // as an objective (orders the slices)
-            root_lb[sl] = (unsigned long long)nxt[0].x * sr.scale;
+            root_lb[r] = (unsigned long long)nxt[0].x * sr.scale;
         }
         __syncthreads();
     }
+}
+
+// The slices of the batches in processing order, the root prefixes (slot j of
+// a batch, no stage placed; the first nb serve a batch of nb) and the batches'
+// counters, cleared.
+__global__ void gather_kernel(const SliceRec *slices, const uint32_t *order, uint32_t n,
+                              SliceRec *batch, uint32_t n_roots, Prefix *roots,
+                              unsigned long long *ctr, uint32_t n_ctr) {
+    const uint32_t stride = gridDim.x * blockDim.x;
+    const uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    for (uint32_t i = i0; i < n; i += stride) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(slices + order[i]);
+        uint4 *dst = reinterpret_cast<uint4 *>(batch + i);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) dst[q] = src[q];
+    }
+    for (uint32_t i = i0; i < n_roots; i += stride) {
+        const Vec32 root = {make_uint4(i & 0xffffu, 0u, 0u, 0u),
+                            make_uint4(0u, 0xffffffffu, 0u, 0u)};  // A = 0, Bm = -1
+        store32(roots + i, root);
+    }
+    for (uint32_t i = i0; i < n_ctr; i += stride) ctr[i] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -889,6 +931,7 @@ struct Search {
     explicit Search(Workspace &w) : ws(w), stream(w.stream), ev(w.ev), d_slices(w.d_slices),
         d_feas(w.d_feas), d_batch(w.d_batch), d_inc(w.d_inc), d_ctr(w.d_ctr), d_best(w.d_best),
         d_feasible(w.d_feasible), d_leaves(w.d_leaves), d_roots(w.d_roots), d_root(w.d_root),
+        d_order(w.d_order),
         d_front(w.d_front), d_defer(w.d_defer) {}
     const pos_problem *pb = nullptr;
     Handle hd{};
@@ -900,9 +943,8 @@ struct Search {
     long long cap = 0;
     int grid_level = 0;
     const SliceSpace *sp = nullptr;  // the slices' identities, global-index order
-    std::vector<SliceRec> slices;
     DevBuf &d_slices, &d_feas, &d_batch, &d_inc, &d_ctr, &d_best, &d_feasible, &d_leaves,
-        &d_roots, &d_root;
+        &d_roots, &d_root, &d_order;
     DevBuf (&d_front)[POS_MAX_STAGES + 1];
     DevBuf (&d_defer)[2 * (POS_MAX_STAGES + 1)];
     unsigned long long *ctr = nullptr;  // device counters, see search_impl
@@ -970,174 +1012,6 @@ static pos_status validate_problem(const pos_problem *p) {
     if (p->schedule == POS_SCHED_INTERLEAVED_1F1B && (p->V < 2 || p->S * p->V > POS_MAX_STAGES))
         return fail(POS_EINVAL, "Interleaved 1F1B needs V >= 2 and S*V <= 16");
     return POS_OK;
-}
-
-// POS_PLACE_DEVICES: the class sequences of one D in lexicographic order,
-// by a depth-first walk that keeps only prefixes with a completion: the
-// remaining r stages can use up every type's remaining devices iff there
-// are counts n_t (sum r) such that each remainder, in units of D, is a sum
-// of exactly n_t TP degrees (reach[n][v]).
-static pos_status device_sequences(const pos_problem *p, int units, int D,
-                                   std::vector<uint8_t> &out, uint64_t *total) {
-    const int T = p->tables.n_types, n_tp = p->tables.n_tp, K = T * n_tp;
-    const uint64_t limit = 1ull << 22;
-    int bud[POS_MAX_TYPES];
-    int vmax = 0;
-    for (int t = 0; t < T; ++t) {
-        if (p->type_counts[t] % D != 0) return POS_OK;  // no stage split uses them up
-        bud[t] = p->type_counts[t] / D;
-        vmax = std::max(vmax, bud[t]);
-    }
-    // reach[v], bit n: v is a sum of exactly n TP degrees (n <= units)
-    std::vector<uint32_t> reach((size_t)vmax + 1, 0u);
-    reach[0] = 1u;
-    for (int v = 1; v <= vmax; ++v)
-        for (int j = 0; j < n_tp; ++j) {
-            const int d = p->tp_list[j];
-            if (d <= v) reach[v] |= (reach[v - d] << 1) & ((2u << units) - 1u);
-        }
-    // completes(r): the remaining budgets bud[] split over exactly r stages;
-    // memoised over (r, budgets) when that table is small
-    size_t states = (size_t)units + 1;
-    int radix[POS_MAX_TYPES];
-    for (int t = 0; t < T; ++t) {
-        radix[t] = bud[t] + 1;
-        states = states <= ((size_t)1 << 24) / (size_t)radix[t] ? states * radix[t] : 0;
-        if (states == 0) break;
-    }
-    std::vector<uint8_t> memo(states, 0);  // 0 unknown, 1 no, 2 yes
-    auto completes = [&](int r) -> bool {
-        size_t key = 0;
-        if (!memo.empty()) {
-            for (int t = T - 1; t >= 0; --t) key = key * radix[t] + bud[t];
-            key = key * (units + 1) + r;
-            if (memo[key]) return memo[key] == 2;
-        }
-        uint32_t mask = 1u;  // bit n: n stages used by the types seen so far
-        for (int t = 0; t < T && mask; ++t) {
-            uint32_t next = 0, m = reach[bud[t]] & ((2u << r) - 1u);
-            while (m) {
-                next |= mask << __builtin_ctz(m);
-                m &= m - 1u;
-            }
-            mask = next & ((2u << r) - 1u);
-        }
-        const bool ok = (mask >> r) & 1u;
-        if (!memo.empty()) memo[key] = ok ? 2 : 1;
-        return ok;
-    };
-    if (!completes(units)) return POS_OK;
-    uint8_t seq[POS_MAX_STAGES];
-    int k_at[POS_MAX_STAGES];
-    int u = 0;
-    k_at[0] = -1;
-    while (u >= 0) {  // iterative depth-first walk, classes in ascending order
-        if (u == units - 1) {
-            // the last stage takes what is left: the one type with a budget
-            // left, with a TP degree equal to it (the prefix was kept only if
-            // such a class exists)
-            int t = 0;
-            while (t < T && bud[t] == 0) ++t;
-            for (int j = 0; t < T && j < n_tp; ++j) {
-                if (p->tp_list[j] != bud[t]) continue;
-                seq[u] = (uint8_t)(t * n_tp + j);
-                const size_t at = out.size();
-                out.resize(at + units);
-                std::memcpy(out.data() + at, seq, units);
-                if (++*total > limit) return fail(POS_EINVAL, "more than 2^22 class sequences");
-            }
-            --u;  // the parent's class is undone on its next step
-            continue;
-        }
-        int k = k_at[u] + 1;
-        if (k_at[u] >= 0) bud[k_at[u] / n_tp] += p->tp_list[k_at[u] % n_tp];  // undo
-        for (; k < K; ++k) {
-            const int t = k / n_tp, d = p->tp_list[k % n_tp];
-            if (bud[t] < d) continue;
-            bud[t] -= d;
-            if (completes(units - u - 1)) break;
-            bud[t] += d;
-        }
-        if (k == K) {  // no further class at this position: back up
-            k_at[u] = -1;
-            --u;
-            continue;
-        }
-        k_at[u] = k;
-        seq[u] = (uint8_t)k;
-        k_at[++u] = -1;
-    }
-    return POS_OK;
-}
-
-pos_status build_slice_space(const pos_problem *p, int units, SliceSpace &sp) {
-    const int T = p->tables.n_types, n_tp = p->tables.n_tp;
-    const uint64_t limit = 1ull << 22;
-    sp = SliceSpace();
-    sp.units = units;
-    sp.per_stage = p->placement == POS_PLACE_DEVICES;
-    sp.n_grp = sp.per_stage ? p->n_D : n_tp;
-    if (sp.per_stage) {
-        uint64_t total = 0;
-        sp.seqs.resize(p->n_D);
-        for (int g = 0; g < p->n_D; ++g) {
-            POS_TRY(device_sequences(p, units, p->D_list[g], sp.seqs[g], &total));
-            sp.D.push_back(p->D_list[g]);
-        }
-    } else {
-        sp.seqs.resize(1);
-        std::vector<uint8_t> &places = sp.seqs[0];
-        std::vector<uint8_t> seq;
-        if (p->placement == POS_PLACE_EXACT) {
-            // the distinct permutations of the multiset, in lexicographic order
-            int sum = 0;
-            for (int ty = 0; ty < T; ++ty) sum += p->type_counts[ty];
-            if (sum != units) return fail(POS_EINVAL, "type_counts must sum to S");
-            for (int ty = 0; ty < T; ++ty) seq.insert(seq.end(), p->type_counts[ty], (uint8_t)ty);
-            do {
-                places.insert(places.end(), seq.begin(), seq.end());
-                if (places.size() > limit * units) return fail(POS_EINVAL, "too many placements");
-            } while (std::next_permutation(seq.begin(), seq.end()));
-        } else {
-            // every sequence in T^S, as an odometer (last stage fastest)
-            double total = 1;
-            for (int x = 0; x < units; ++x) total *= T;
-            if (total > (double)limit) return fail(POS_EINVAL, "too many placements");
-            seq.assign(units, 0);
-            for (;;) {
-                places.insert(places.end(), seq.begin(), seq.end());
-                int x = units - 1;
-                while (x >= 0 && seq[x] == T - 1) seq[x--] = 0;
-                if (x < 0) break;
-                seq[x]++;
-            }
-        }
-        for (int g = 0; g < n_tp; ++g) sp.D.push_back(p->dp_list[g]);
-    }
-    sp.grp_off.assign(sp.n_grp + 1, 0);
-    for (int g = 0; g < sp.n_grp; ++g) sp.grp_off[g + 1] = sp.grp_off[g] + sp.n_seq(g);
-    sp.per_m = sp.grp_off[sp.n_grp];
-    if ((uint64_t)p->n_M * sp.per_m > limit) return fail(POS_EINVAL, "more than 2^22 slices");
-    return POS_OK;
-}
-
-void plan_slice_fields(const pos_problem *p, const SliceSpace &sp, uint64_t ord, pos_plan *out) {
-    int mi = 0, g = 0;
-    uint64_t pr = 0;
-    sp.decode(ord, &mi, &g, &pr);
-    const int n_tp = p->tables.n_tp;
-    out->m_idx = mi;
-    out->M = p->M_list[mi];
-    out->D = sp.D[g];
-    out->place_rank = pr;
-    out->tp_idx = sp.per_stage ? -1 : g;
-    out->tp = sp.per_stage ? -1 : p->tp_list[g];
-    out->d_idx = sp.per_stage ? g : -1;
-    for (int x = 0; x < POS_MAX_STAGES; ++x) {
-        const int k = x < sp.units ? sp.cls(g, pr, x, n_tp) : -1;
-        out->type[x] = k < 0 ? -1 : k / n_tp;
-        out->tp_stage[x] = k < 0 ? -1 : k % n_tp;
-    }
 }
 
 // Size limits of the search space that do not need the slices, checked on
@@ -1248,6 +1122,18 @@ static pos_status reserve_stage(Search &s, size_t bytes) {
     s.ws.h_stage_cap = 0;
     POS_CUDA(cudaMallocHost(&s.ws.h_stage, bytes));
     s.ws.h_stage_cap = bytes;
+    return POS_OK;
+}
+
+// Pinned landing area of n root bounds.
+static pos_status reserve_lb(Search &s, size_t n) {
+    if (n <= s.ws.h_lb_cap) return POS_OK;
+    POS_CUDA(cudaStreamSynchronize(s.stream));  // no copy into the old area in flight
+    if (s.ws.h_lb) cudaFreeHost(s.ws.h_lb);
+    s.ws.h_lb = nullptr;
+    s.ws.h_lb_cap = 0;
+    POS_CUDA(cudaMallocHost(&s.ws.h_lb, sizeof(unsigned long long) * n));
+    s.ws.h_lb_cap = n;
     return POS_OK;
 }
 
@@ -1443,80 +1329,73 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
     // after the side-stream work of an earlier search (which may have
     // returned early), since this one reuses its buffers
     POS_CUDA(cudaStreamWaitEvent(s.stream, s.ws.ev_join, 0));
-    // pinned staging for this search's uploads (tables, slice records, lists)
-    if ((st = reserve_stage(s, ((size_t)256 << 10) + (size_t)n_slices * 320 +
-                                   (size_t)p->n_M * 16)) != POS_OK)
-        return st;
+    if (n_slices == 0) {
+        std::memset(out, 0, sizeof(*out));
+        if (stats) std::memset(stats, 0, sizeof(*stats));
+        return fail(POS_EINFEASIBLE, "no placement uses the devices exactly");
+    }
+    // objective scale: Q = lcm(D*M); T*Q/(D*M) orders plans by time per sample
+    const uint64_t Q = objective_scale(p, sp);
+    SetupPack pk;
     {
         std::vector<unsigned char> host;
         st = build_blob(&p->tables, p->schedule, host, s.hd.lay, s.hd.guard_A, s.hd.guard_D,
                         s.hd.guard_P);
         if (st != POS_OK) return st;
-        POS_CUDA(cudaGetDevice(&s.hd.device));
-        POS_CUDA(s.ws.blob.reserve(s.hd.lay.bytes));
-        s.hd.d_blob = s.ws.blob.p;
-        POS_TRY(upload(s, s.hd.d_blob, host.data(), s.hd.lay.bytes));
-        if ((st = launch_prefix_rows(s.hd.d_blob, s.hd.lay, s.stream)) != POS_OK) return st;
+        std::vector<int32_t> mis(p->n_M);
+        std::iota(mis.begin(), mis.end(), 0);
+        pack_setup(p, sp, mis, Q, host, pk);
     }
     // overflow guard for every M (Sec. 4.1 path-length bound)
     for (int i = 0; i < p->n_M; ++i)
         if (guard_trips(s.h->guard_A, s.h->guard_D, s.h->guard_P, s.S, p->M_list[i]))
             return fail(POS_EOVERFLOW, "makespan bound reaches 2^31 for some M");
-    // objective scale: Q = lcm(D*M); T*Q/(D*M) orders plans by time per sample
-    const uint64_t Q = objective_scale(p, sp);
-    s.slices.resize(n_slices);
-    {
-        uint64_t ord = 0;
-        for (int mi = 0; mi < p->n_M; ++mi)
-            for (int g = 0; g < sp.n_grp; ++g)
-                for (uint64_t pr = 0; pr < sp.n_seq(g); ++pr, ++ord) {
-                    SliceRec &r = s.slices[ord];
-                    std::memset(&r, 0, sizeof(r));
-                    r.ordinal = ord;
-                    r.M = p->M_list[mi];
-                    r.scale = Q / ((uint64_t)sp.D[g] * p->M_list[mi]);
-                    r.gid = (uint32_t)ord;
-                    r.vslot = (uint32_t)ord;  // bound-table row when every slice has one
-                    for (int x = 0; x < s.S; ++x) r.cls[x] = (uint8_t)sp.cls(g, pr, x, s.n_tp);
-                }
-    }
-    const int smem = s.h->lay.bytes;
+    // pinned staging for this search's uploads (set-up, lists of slices)
+    if ((st = reserve_stage(s, pk.bytes.size() + ((size_t)64 << 10) + (size_t)n_slices * 32 +
+                                   (size_t)p->n_M * 1024)) != POS_OK)
+        return st;
+    POS_CUDA(cudaGetDevice(&s.hd.device));
+    POS_CUDA(s.ws.blob.reserve(pk.bytes.size()));
+    s.hd.d_blob = s.ws.blob.p;
+    POS_CUDA(s.d_slices.reserve(sizeof(SliceRec) * n_slices));
+    POS_CUDA(s.d_inc.reserve(sizeof(Key128)));
+    POS_CUDA(s.d_ctr.reserve(sizeof(unsigned long long) * kCounters));
+    POS_CUDA(s.d_best.reserve(sizeof(unsigned long long) * n_slices));
+    s.ctr = static_cast<unsigned long long *>(s.d_ctr.p);
+    s.stats = s.ctr + 40;  // ctr[0..33]: per-depth counters, ctr[36]: leaf count
+    static_assert(40 + kStCount <= kCounters, "counter block");
+    SliceRec *d_all = static_cast<SliceRec *>(s.d_slices.p);
+    POS_TRY(upload(s, s.ws.blob.p, pk.bytes.data(), pk.bytes.size()));
+    if ((st = launch_setup(pk, sp, s.n_tp, s.hd.lay, s.ws.blob.p, d_all,
+                           static_cast<unsigned long long *>(s.d_best.p),
+                           static_cast<Key128 *>(s.d_inc.p), s.ctr, s.stream)) != POS_OK)
+        return st;
+    s.launches++;
     int per_sm = 0;
-    POS_TRY(ensure_smem(reinterpret_cast<const void *>(level_kernel<false, 0>), smem));
-    POS_TRY(ensure_smem(reinterpret_cast<const void *>(feas_kernel), smem));
-    POS_TRY(ensure_smem(reinterpret_cast<const void *>(bound_kernel), smem));
     POS_TRY(blocks_per_sm(reinterpret_cast<const void *>(level_kernel<false, 0>), kThreads,
                           timing_layout(s.h->lay).bytes, &per_sm));
     s.grid_level = std::max(1, per_sm) * sm_count();
 
-    POS_CUDA(s.d_slices.reserve(sizeof(SliceRec) * n_slices));
     POS_CUDA(s.d_feas.reserve(sizeof(uint4) * (size_t)n_slices * (s.S + 1)));
     POS_CUDA(s.ws.d_lim.reserve((size_t)n_slices * s.S * 128));
-    POS_CUDA(s.d_inc.reserve(sizeof(Key128)));
-    POS_CUDA(s.d_ctr.reserve(sizeof(unsigned long long) * 128));
-    POS_CUDA(s.d_best.reserve(sizeof(unsigned long long) * n_slices));
     POS_CUDA(s.d_leaves.reserve(sizeof(Leaf) * (size_t)s.cap));
-    s.ctr = static_cast<unsigned long long *>(s.d_ctr.p);
-    s.stats = s.ctr + 40;  // ctr[0..33]: per-depth counters, ctr[36]: leaf count
-    static_assert(40 + kStCount <= 128, "counter block");
-    POS_TRY(upload(s, s.d_slices.p, s.slices.data(), sizeof(SliceRec) * n_slices));
-    POS_CUDA(cudaMemsetAsync(s.d_inc.p, 0xff, sizeof(Key128), s.stream));
-    POS_CUDA(cudaMemsetAsync(s.d_ctr.p, 0, sizeof(unsigned long long) * 128, s.stream));
-    POS_CUDA(cudaMemsetAsync(s.d_best.p, 0xff, sizeof(unsigned long long) * n_slices, s.stream));
-    const SliceRec *d_all = static_cast<const SliceRec *>(s.d_slices.p);
     DevBuf &d_root = s.d_root;
     POS_CUDA(d_root.reserve(n_slices));
     {
-        // the memory tables alone (Pw, Pa, cap) are staged per block
-        const BlobLayout ml = memory_layout(s.h->lay);
-        POS_TRY(ensure_smem(reinterpret_cast<const void *>(feas_kernel), ml.bytes));
-        feas_kernel<<<std::min(n_slices, 16 * sm_count()), 128, ml.bytes, s.stream>>>(
-            d_all, n_slices, s.S, static_cast<uint4 *>(s.d_feas.p),
-            static_cast<uint8_t *>(s.ws.d_lim.p), static_cast<uint8_t *>(d_root.p),
-            static_cast<const unsigned char *>(s.h->d_blob) + s.h->lay.off_Pw, ml, s.stats);
+        // memory limits per (class, micro-batches in flight), then the slices
+        const int wmax = p->schedule == POS_SCHED_EAGER_1F1B ? 2 * s.S - 1 : s.S;
+        POS_CUDA(s.ws.d_limtab.reserve((size_t)s.h->lay.K * wmax * (s.L + 1)));
+        uint8_t *limtab = static_cast<uint8_t *>(s.ws.d_limtab.p);
+        POS_TRY(launch_lim(s.h->d_blob, s.h->lay, wmax, limtab, s.stream));
+        constexpr int kPer = kFeasThreads / 32;
+        POS_CUDA(launch_dependent(
+            feas_kernel, std::min((n_slices + kPer - 1) / kPer, 16 * sm_count()), kFeasThreads, 0,
+            s.stream, static_cast<const SliceRec *>(d_all), n_slices, s.S,
+            static_cast<const uint8_t *>(limtab), wmax, static_cast<uint4 *>(s.d_feas.p),
+            static_cast<uint8_t *>(s.ws.d_lim.p), static_cast<uint8_t *>(d_root.p), s.L,
+            p->schedule));
+        s.launches += 2;
     }
-    POS_CUDA(cudaGetLastError());
-    s.launches++;
     std::vector<uint8_t> root(n_slices);
     std::vector<std::vector<uint32_t>> feas_by_m(p->n_M);  // feasible slices per M index
     uint64_t n_feasible = 0;
@@ -1556,27 +1435,18 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         // the greedy plans of each M index (holes for the infeasible slices),
         // on the side stream: they only lower the incumbent, which the
         // enumeration reads after the join below
-        std::vector<unsigned long long> gc(p->n_M, (unsigned long long)sp.per_m);
-        POS_CUDA(s.ws.d_wcnt.reserve(sizeof(unsigned long long) * p->n_M));
-        POS_TRY(upload(s, s.ws.d_wcnt.p, gc.data(), sizeof(unsigned long long) * p->n_M));
+        unsigned long long *counts = reinterpret_cast<unsigned long long *>(
+            static_cast<unsigned char *>(s.ws.blob.p) + pk.off_counts);
         POS_CUDA(cudaEventRecord(s.ws.ev_fork, s.stream));
         POS_CUDA(cudaStreamWaitEvent(s.ws.side, s.ws.ev_fork, 0));
         for (int mi = 0; mi < p->n_M && st == POS_OK; ++mi)
             st = run_leaves(s, static_cast<const Leaf *>(s.ws.d_greedy.p) + mi * sp.per_m,
-                            static_cast<unsigned long long *>(s.ws.d_wcnt.p) + mi, d_all,
-                            p->M_list[mi], static_cast<unsigned long long *>(s.d_best.p),
-                            s.ws.side);
+                            counts + mi, d_all, p->M_list[mi],
+                            static_cast<unsigned long long *>(s.d_best.p), s.ws.side);
         // recorded also after a failed launch: the next search waits on it
         POS_CUDA(cudaEventRecord(s.ws.ev_join, s.ws.side));
         if (st != POS_OK) return st;
-        if ((size_t)n_slices > s.ws.h_lb_cap) {
-            POS_CUDA(cudaStreamSynchronize(s.stream));  // no copy into the old area in flight
-            if (s.ws.h_lb) cudaFreeHost(s.ws.h_lb);
-            s.ws.h_lb = nullptr;
-            s.ws.h_lb_cap = 0;
-            POS_CUDA(cudaMallocHost(&s.ws.h_lb, sizeof(unsigned long long) * n_slices));
-            s.ws.h_lb_cap = (size_t)n_slices;
-        }
+        POS_TRY(reserve_lb(s, (size_t)n_slices));
         const ReadPart parts[2] = {{root.data(), d_root.p, (size_t)n_slices},
                                    {s.ws.h_lb, s.ws.d_lb.p, sizeof(unsigned long long) * n_slices}};
         if ((st = sync_read_many(s, parts, 2)) != POS_OK) return st;
@@ -1597,17 +1467,13 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         std::vector<uint32_t> rows;
         rows.reserve(n_feasible);
         for (int mi = 0; mi < p->n_M; ++mi)
-            for (uint32_t g : feas_by_m[mi]) {
-                s.slices[g].vslot = (uint32_t)rows.size();
-                rows.push_back(g);
-            }
+            rows.insert(rows.end(), feas_by_m[mi].begin(), feas_by_m[mi].end());
         s.n_vrows = (int)rows.size();
         POS_CUDA(s.ws.d_rows.reserve(sizeof(uint32_t) * rows.size()));
         POS_CUDA(s.ws.d_vb.reserve(sizeof(int2) * 128 * (size_t)s.S * rows.size()));
         POS_CUDA(s.ws.d_greedy.reserve(sizeof(Leaf) * rows.size()));
-        POS_CUDA(s.ws.d_lb.reserve(sizeof(unsigned long long) * n_slices));
+        POS_CUDA(s.ws.d_lb.reserve(sizeof(unsigned long long) * rows.size()));
         POS_TRY(upload(s, s.ws.d_rows.p, rows.data(), sizeof(uint32_t) * rows.size()));
-        POS_TRY(upload(s, s.d_slices.p, s.slices.data(), sizeof(SliceRec) * n_slices));
         const BlobLayout tl = timing_layout(s.h->lay);
         POS_TRY(ensure_smem(reinterpret_cast<const void *>(bound_kernel), tl.bytes));
         if (p->profile) POS_CUDA(cudaEventRecord(s.ev[0], s.stream));
@@ -1624,15 +1490,8 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         // the root bounds order the slices: their copy to the host is queued
         // here and waited for alone, so the warm-up kernels queued next run
         // while the host plans the batches
-        if ((size_t)n_slices > s.ws.h_lb_cap) {
-            POS_CUDA(cudaStreamSynchronize(s.stream));  // no copy into the old area in flight
-            if (s.ws.h_lb) cudaFreeHost(s.ws.h_lb);
-            s.ws.h_lb = nullptr;
-            s.ws.h_lb_cap = 0;
-            POS_CUDA(cudaMallocHost(&s.ws.h_lb, sizeof(unsigned long long) * n_slices));
-            s.ws.h_lb_cap = (size_t)n_slices;
-        }
-        POS_CUDA(cudaMemcpyAsync(s.ws.h_lb, s.ws.d_lb.p, sizeof(unsigned long long) * n_slices,
+        POS_TRY(reserve_lb(s, n_feasible));
+        POS_CUDA(cudaMemcpyAsync(s.ws.h_lb, s.ws.d_lb.p, sizeof(unsigned long long) * n_feasible,
                                  cudaMemcpyDeviceToHost, s.stream));
         POS_CUDA(cudaEventRecord(s.ws.ev_lb, s.stream));
         // counts of the greedy plans per M index, then one leaf launch each
@@ -1686,13 +1545,18 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
     // their copy only; otherwise by the best warm-up plan of the slice,
     // after the warm-up
     const bool by_bound = p->prune == 2 && n_feasible > 0;
-    std::vector<unsigned long long> key(n_slices);
+    std::vector<unsigned long long> read;
+    const unsigned long long *key;  // of slice i, or of feasible row r (rows path)
+    const bool key_by_row = by_bound && !bound_all;
     if (by_bound) {
         if (!bound_all) POS_CUDA(cudaEventSynchronize(s.ws.ev_lb));  // else read already
-        std::memcpy(key.data(), s.ws.h_lb, sizeof(unsigned long long) * n_slices);
-    } else if ((st = sync_read(s, key.data(), s.d_best.p,
-                               sizeof(unsigned long long) * n_slices)) != POS_OK) {
-        return st;
+        key = s.ws.h_lb;
+    } else {
+        read.resize(n_slices);
+        if ((st = sync_read(s, read.data(), s.d_best.p, sizeof(unsigned long long) * n_slices)) !=
+            POS_OK)
+            return st;
+        key = read.data();
     }
     if (p->profile && s.n_bound) {
         float ms_b = 0;
@@ -1708,12 +1572,16 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         unsigned long long best;
     };
     std::vector<Group> groups;
+    std::vector<std::pair<unsigned long long, uint32_t>> order;
     for (int mi = 0; mi < p->n_M; ++mi) {
-        if (feas_by_m[mi].empty()) continue;
         auto &fl = feas_by_m[mi];
-        std::stable_sort(fl.begin(), fl.end(),
-                         [&](uint32_t a, uint32_t b) { return key[a] < key[b]; });
-        groups.push_back({mi, key[fl[0]]});
+        if (fl.empty()) continue;
+        order.clear();
+        for (size_t j = 0; j < fl.size(); ++j)
+            order.push_back({key[key_by_row ? feas_off[mi] + j : fl[j]], fl[j]});
+        std::sort(order.begin(), order.end());  // ties: the lower slice first
+        for (size_t j = 0; j < fl.size(); ++j) fl[j] = order[j].second;
+        groups.push_back({mi, order[0].first});
     }
     std::stable_sort(groups.begin(), groups.end(),
                      [](const Group &a, const Group &b) { return a.best < b.best; });
@@ -1722,7 +1590,7 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         int M;
         size_t off, nb;
     };
-    std::vector<SliceRec> ordered;
+    std::vector<uint32_t> ordered;  // slices
     std::vector<Batch> batches;
     size_t max_nb = 1;
     for (const Group &g : groups) {
@@ -1740,24 +1608,26 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         for (size_t b0 = 0; b0 < fl.size();) {
             const size_t nb = std::min(b0 == 0 ? first : bsz, fl.size() - b0);
             batches.push_back({p->M_list[g.mi], ordered.size(), nb});
-            for (size_t j = 0; j < nb; ++j) ordered.push_back(s.slices[fl[b0 + j]]);
+            ordered.insert(ordered.end(), fl.begin() + b0, fl.begin() + b0 + nb);
             max_nb = std::max(max_nb, nb);
             b0 += nb;
         }
     }
     POS_CUDA(s.d_batch.reserve(sizeof(SliceRec) * std::max<size_t>(1, ordered.size())));
-    if (!ordered.empty())
-        POS_TRY(upload(s, s.d_batch.p, ordered.data(), sizeof(SliceRec) * ordered.size()));
-    // roots: slot j of a batch, no stage placed (the first nb serve a batch of nb)
-    std::vector<Prefix> roots(max_nb);
-    for (size_t j = 0; j < max_nb; ++j) {
-        std::memset(&roots[j], 0, sizeof(Prefix));
-        roots[j].slice = (uint16_t)j;
-        roots[j].A = 0;
-        roots[j].Bm = -1;
-    }
     POS_CUDA(s.d_roots.reserve(sizeof(Prefix) * max_nb));
-    POS_TRY(upload(s, s.d_roots.p, roots.data(), sizeof(Prefix) * max_nb));
+    const size_t n_b = batches.size();
+    POS_CUDA(s.ws.d_bctr.reserve(sizeof(unsigned long long) * 32 * std::max<size_t>(1, n_b)));
+    POS_CUDA(s.d_order.reserve(sizeof(uint32_t) * std::max<size_t>(1, ordered.size())));
+    if (!ordered.empty()) {
+        POS_TRY(upload(s, s.d_order.p, ordered.data(), sizeof(uint32_t) * ordered.size()));
+        gather_kernel<<<(int)((ordered.size() + kThreads - 1) / kThreads), kThreads, 0, s.stream>>>(
+            d_all, static_cast<const uint32_t *>(s.d_order.p), (uint32_t)ordered.size(),
+            static_cast<SliceRec *>(s.d_batch.p), (uint32_t)max_nb,
+            static_cast<Prefix *>(s.d_roots.p), static_cast<unsigned long long *>(s.ws.d_bctr.p),
+            (uint32_t)(32 * n_b));
+        POS_CUDA(cudaGetLastError());
+        s.launches++;
+    }
     const SliceRec *d_ordered = static_cast<const SliceRec *>(s.d_batch.p);
     const Prefix *d_rootp = static_cast<const Prefix *>(s.d_roots.p);
 
@@ -1792,10 +1662,7 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
             if ((st = ensure_depth(s, x)) != POS_OK) return st;
         for (int x = 0; x <= S - 2; ++x)
             if ((st = ensure_defer(s, x, (s.cap + 31) / 32 + 1)) != POS_OK) return st;
-        const size_t n_b = batches.size();
-        POS_CUDA(s.ws.d_bctr.reserve(sizeof(unsigned long long) * 32 * std::max<size_t>(1, n_b)));
         unsigned long long *bctr = static_cast<unsigned long long *>(s.ws.d_bctr.p);
-        POS_CUDA(cudaMemsetAsync(bctr, 0, sizeof(unsigned long long) * 32 * n_b, s.stream));
         // timing events (profile only), S + 1 per batch: before level 0,
         // after each level kernel, after the leaf kernel
         const bool prof = p->profile != 0;
@@ -1936,12 +1803,11 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         return fail(POS_EINFEASIBLE, "no memory-feasible plan");
     }
     const uint64_t ord = inc.idx / s.n_map;
-    const SliceRec &sr = s.slices[ord];
     out->found = 1;
     out->map_rank = inc.idx % s.n_map;
     plan_slice_fields(p, sp, ord, out);
     out->S = s.S;
-    out->makespan = (int32_t)(inc.obj / sr.scale);
+    out->makespan = (int32_t)(inc.obj / (Q / ((uint64_t)out->D * out->M)));
     out->global_index = inc.idx;
     for (int x = 0; x < POS_MAX_STAGES; ++x) out->layers[x] = 0;
     host_unrank(s.L, s.S, out->map_rank, out->layers);

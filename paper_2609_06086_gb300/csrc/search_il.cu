@@ -757,10 +757,6 @@ pos_status search_interleaved(Workspace &ws, const pos_problem *p, const SliceSp
     // after the side-stream work of an earlier search, whose buffers this
     // one reuses
     POS_CUDA(cudaStreamWaitEvent(r.st, ws.ev_join, 0));
-    POS_CUDA(ws.blob.reserve(r.lay.bytes));
-    r.blob = ws.blob.p;
-    POS_CUDA(cudaMemcpyAsync(r.blob, host.data(), r.lay.bytes, cudaMemcpyHostToDevice, r.st));
-    POS_TRY(launch_prefix_rows(r.blob, r.lay, r.st));
     // slices: M values that are multiples of N, then the groups (TP index or
     // D) and their sequences in global-index order
     uint64_t Q = 1;
@@ -769,44 +765,35 @@ pos_status search_interleaved(Workspace &ws, const pos_problem *p, const SliceSp
             const uint64_t dm = (uint64_t)D * p->M_list[i];
             Q = Q / gcd64(Q, dm) * dm;
         }
-    std::vector<SliceRec> slices;
-    for (int mi = 0; mi < p->n_M; ++mi) {
-        if (p->M_list[mi] % N != 0) continue;
-        uint64_t ord = (uint64_t)mi * sp.per_m;
-        for (int g = 0; g < sp.n_grp; ++g)
-            for (uint64_t pr = 0; pr < sp.n_seq(g); ++pr, ++ord) {
-                SliceRec sr;
-                std::memset(&sr, 0, sizeof(sr));
-                sr.ordinal = ord;
-                sr.M = p->M_list[mi];
-                sr.scale = Q / ((uint64_t)sp.D[g] * p->M_list[mi]);
-                sr.gid = (uint32_t)slices.size();
-                for (int d = 0; d < N; ++d) sr.cls[d] = (uint8_t)sp.cls(g, pr, d, r.n_tp);
-                slices.push_back(sr);
-            }
-    }
-    const long long n_slices = (long long)slices.size();
+    std::vector<int32_t> mis;
+    for (int mi = 0; mi < p->n_M; ++mi)
+        if (p->M_list[mi] % N == 0) mis.push_back(mi);
+    SetupPack pk;
+    pack_setup(p, sp, mis, Q, host, pk);
+    const long long n_slices = (long long)pk.n_slices;
     r.cap = p->frontier_cap > 0 ? p->frontier_cap : (1ll << 24);
     r.cap = std::max<long long>({r.cap, 32LL * r.L, n_slices});
     std::memset(out, 0, sizeof(*out));
     if (stats) std::memset(stats, 0, sizeof(*stats));
-    if (n_slices == 0) return fail(POS_EINFEASIBLE, "no M value is a multiple of S");
+    if (mis.empty()) return fail(POS_EINFEASIBLE, "no M value is a multiple of S");
+    if (n_slices == 0) return fail(POS_EINFEASIBLE, "no placement uses the devices exactly");
+    POS_CUDA(ws.blob.reserve(pk.bytes.size()));
+    r.blob = ws.blob.p;
     POS_CUDA(ws.d_slices.reserve(sizeof(SliceRec) * n_slices));
     POS_CUDA(ws.d_inc.reserve(sizeof(Key128)));
-    POS_CUDA(ws.d_ctr.reserve(sizeof(unsigned long long) * 128));
+    POS_CUDA(ws.d_ctr.reserve(sizeof(unsigned long long) * kCounters));
     POS_CUDA(ws.il_rec.reserve(2 * sizeof(uint4) * (size_t)r.cap));
     POS_CUDA(ws.il_slice.reserve(sizeof(uint32_t) * (size_t)r.cap));
     POS_CUDA(ws.il_T.reserve(sizeof(int32_t) * (size_t)r.cap));
     POS_CUDA(ws.il_F.reserve((size_t)r.cap));
     POS_CUDA(ws.il_offs.reserve(sizeof(uint32_t) * (kKeysIl + 1)));
     POS_CUDA(ws.d_front[0].reserve(sizeof(Vec32) * n_slices));
-    POS_CUDA(cudaMemcpyAsync(ws.d_slices.p, slices.data(), sizeof(SliceRec) * n_slices,
-                             cudaMemcpyHostToDevice, r.st));
-    POS_CUDA(cudaMemsetAsync(ws.d_inc.p, 0xff, sizeof(Key128), r.st));
-    POS_CUDA(cudaMemsetAsync(ws.d_ctr.p, 0, sizeof(unsigned long long) * 128, r.st));
+    POS_CUDA(cudaMemcpyAsync(r.blob, pk.bytes.data(), pk.bytes.size(), cudaMemcpyHostToDevice, r.st));
     r.d_slices = static_cast<const SliceRec *>(ws.d_slices.p);
     r.ctr = static_cast<unsigned long long *>(ws.d_ctr.p);
     r.stats = r.ctr + 40;
+    POS_TRY(launch_setup(pk, sp, r.n_tp, r.lay, r.blob, static_cast<SliceRec *>(ws.d_slices.p),
+                         nullptr, static_cast<Key128 *>(ws.d_inc.p), r.ctr, r.st));
     int per_sm = 0;
     {
         const void *lk = nullptr;

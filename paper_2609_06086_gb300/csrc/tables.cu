@@ -136,47 +136,22 @@ BlobLayout memory_layout(const BlobLayout &ly) {
     return t;
 }
 
-// One block per (table, class) row, a thread per layer: the raw per-layer
-// row sits at entries 1..L of the row; turn it into an exclusive prefix sum
-// with P[0] = 0.  Bound by latency: one load, a scan by shuffles within the
-// warps and over the four warp totals, one store per thread (a thread
-// walking its row took 13 us for 80 layers, now under 4).
-constexpr int kPrefixThreads = 128;
-static_assert(kPrefixThreads > POS_MAX_LAYERS, "a thread per layer");
 __global__ void __launch_bounds__(kPrefixThreads) prefix_rows_kernel(unsigned char *blob,
                                                                      BlobLayout ly) {
-    const int K = ly.K, Lp1 = ly.L + 1;
-    const int table = blockIdx.x / K, k = blockIdx.x % K, l = threadIdx.x;
-    int64_t *P8 = reinterpret_cast<int64_t *>(blob + (table == 0 ? ly.off_Pw : ly.off_Pa)) +
-                  (int64_t)k * Lp1;
-    int32_t *P4 = reinterpret_cast<int32_t *>(blob + ly.off_P) + (int64_t)k * Lp1 * 4 + (table - 2);
-    int64_t v = 0;
-    if (l >= 1 && l <= ly.L) v = table < 2 ? P8[l] : (int64_t)P4[4 * l];
-    const int lane = l & 31, wid = l >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += u;
-    }
-    __shared__ int64_t total[kPrefixThreads / 32];
-    if (lane == 31) total[wid] = v;
-    __syncthreads();
-    for (int w = 0; w < wid; ++w) v += total[w];
-    if (l <= ly.L) {
-        if (table < 2) P8[l] = v;
-        else P4[4 * l] = (int32_t)v;
-    }
+    prefix_row(blob, ly, blockIdx.x);
 }
 
 // One block per (class, in-flight count w): lim[k][w-1][a] for every start
 // a, by binary search (the memory need grows with the layer count, the
 // tables being non-negative).
-__global__ void lim_kernel(unsigned char *blob, BlobLayout ly, int wmax, int lim_off) {
+__global__ void lim_kernel(const unsigned char *blob, BlobLayout ly, int wmax, uint8_t *lim) {
+    grid_dep_wait();  // the prefix sums
+    grid_dep_trigger();
     const int k = blockIdx.x / wmax, w = blockIdx.x % wmax + 1, L = ly.L;
     const int64_t *Pw = reinterpret_cast<const int64_t *>(blob + ly.off_Pw) + (int64_t)k * (L + 1);
     const int64_t *Pa = reinterpret_cast<const int64_t *>(blob + ly.off_Pa) + (int64_t)k * (L + 1);
     const int64_t cap = reinterpret_cast<const int64_t *>(blob + ly.off_cap)[k];
-    uint8_t *out = blob + lim_off + (size_t)blockIdx.x * (L + 1);
+    uint8_t *out = lim + (size_t)blockIdx.x * (L + 1);
     for (int a = threadIdx.x; a <= L; a += blockDim.x) {
         int lo = a, hi = L;
         while (lo < hi) {
@@ -283,6 +258,13 @@ pos_status launch_prefix_rows(void *d_blob, const BlobLayout &ly, cudaStream_t s
     return POS_OK;
 }
 
+pos_status launch_lim(const void *d_blob, const BlobLayout &ly, int wmax, uint8_t *lim,
+                      cudaStream_t stream) {
+    POS_CUDA(launch_dependent(lim_kernel, ly.K * wmax, 128, 0, stream,
+                              static_cast<const unsigned char *>(d_blob), ly, wmax, lim));
+    return POS_OK;
+}
+
 pos_status create_handle(const pos_tables *t, int sched, Handle **out) {
     std::vector<unsigned char> host;
     BlobLayout ly;
@@ -306,9 +288,9 @@ pos_status create_handle(const pos_tables *t, int sched, Handle **out) {
     if (e == cudaSuccess) e = cudaMemcpy(h->d_blob, host.data(), ly.bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && launch_prefix_rows(h->d_blob, ly, 0) != POS_OK) e = cudaErrorLaunchFailure;
     if (e == cudaSuccess && h->lim_bytes > 0) {
-        lim_kernel<<<ly.K * h->lim_w, 128>>>(static_cast<unsigned char *>(h->d_blob), ly,
-                                            h->lim_w, h->lim_off);
-        e = cudaGetLastError();
+        if (launch_lim(h->d_blob, ly, h->lim_w, static_cast<uint8_t *>(h->d_blob) + h->lim_off, 0) !=
+            POS_OK)
+            e = cudaErrorLaunchFailure;
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
