@@ -385,19 +385,6 @@ struct ExpandParams {
 };
 
 
-// Largest l in [0, hi] with pred(l), for pred true up to some l and false
-// after (pred(0) is taken as true).
-template <class Pred>
-__device__ __forceinline__ int last_true(int hi, Pred pred) {
-    int lo = 0;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pred(mid)) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 // Per-parent quantities shared by the search for children and the writes:
 // parent cut c, class k of the new stage, prefix sums at c.
 struct ParentCtx {
@@ -440,28 +427,31 @@ __device__ __forceinline__ ParentCtx parent_ctx(const Tab &t, int k, int c) {
 // [1, hi] found by binary search; the children are the positions in
 // (c, c+hi] from which the remaining layers still fit the remaining stages
 // (feasibility bits).
-__device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, int64_t A,
-                                          int64_t Bm, const ParentCtx &q, uint32_t gid,
-                                          const int2 *vrow, uint64_t scale,
-                                          uint64_t thr, Bits128 &acc, unsigned long long &cut_b,
-                                          unsigned long long &cut_m, unsigned long long &cut_r) {
+// `top` is the largest makespan that does not beat the incumbent's objective
+// in the parent's slice (top_makespan).  Every bound tested is the length of a
+// DAG path of a plan of the slice, so it fits in 32 bits under the overflow
+// guard.
+__device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, int32_t A,
+                                          int32_t Bm, const ParentCtx &q, uint32_t gid,
+                                          const int2 *vrow, int32_t top, Bits128 &acc,
+                                          unsigned long long &cut_b, unsigned long long &cut_m,
+                                          unsigned long long &cut_r) {
     const int S = p.S, M = p.M, x = p.x, L = t.L();
     const int lmax = L - q.c - (S - x - 1);
     const int hi_mem0 = min(lmax, (int)__ldg(p.lim + ((size_t)gid * S + x) * 128 + q.c));
+    const uint4 f = __ldg(p.feas + (size_t)gid * (S + 1) + x + 1);
     const int hi_mem = min(hi_mem0, q.rcap);  // ridge rule: a cap on the layer count
     cut_r += (unsigned long long)(hi_mem0 - hi_mem);
     int hi = hi_mem;
     if (p.prune) {  // g(S_{x+1}) grows with l: binary search for the last l within the bound
         int lo = 0;
         while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1, c2 = q.c + mid;
-            const Sums v = sums_from(t, q.k, q.at, c2);
-            const int64_t F = v.f, B = v.b, d = v.d;
-            if ((uint64_t)(A + (int64_t)M * (F + B) + max(Bm, d)) * scale <= thr) lo = mid;
+            const int mid = (lo + hi + 1) >> 1;
+            const Sums v = sums_from(t, q.k, q.at, q.c + mid);
+            if (A + M * (v.f + v.b) + max(Bm, v.d) <= top) lo = mid;
             else hi = mid - 1;
         }
     }
-    const uint4 f = __ldg(p.feas + (size_t)gid * (S + 1) + x + 1);
     const Bits128 win = range_bits(q.c + 1, q.c + hi);
     acc.w[0] = f.x & win.w[0];
     acc.w[1] = f.y & win.w[1];
@@ -491,12 +481,9 @@ __device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, i
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     if (bb[u] < 0) continue;
-                    const int c2 = 32 * wd + bb[u];
-                    const Sums add = sums_from(t, q.k, q.at, c2);
-                    const int64_t F = add.f, B = add.b, d = add.d;
-                    const int64_t A2 = A + F + q.pf, Bm2 = max(Bm, d) + B + q.pb;
-                    if (v[u].x == kNoCompletion || (uint64_t)(A2 + v[u].x) * scale > thr ||
-                        (uint64_t)(A2 + Bm2 + v[u].y) * scale > thr) {
+                    const Sums w = sums_from(t, q.k, q.at, 32 * wd + bb[u]);
+                    const int32_t A2 = A + w.f + q.pf, Bm2 = max(Bm, w.d) + w.b + q.pb;
+                    if (v[u].x == kNoCompletion || A2 + v[u].x > top || A2 + Bm2 + v[u].y > top) {
                         acc.w[wd] &= ~(1u << bb[u]);
                         --n;
                         ++cut_b;
@@ -511,32 +498,32 @@ __device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, i
 // Completion (parent depth S-2): stage a = S-2 takes l layers, stage
 // b = S-1 the rest.  Stage a's memory and g(S_{S-1}) bound l from above,
 // stage b's memory from below (fewer layers as l grows); inside that window
-// each l is checked against g(S_S).
-__device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t, int64_t A,
-                                            int64_t Bm, const ParentCtx &q, int kb, uint32_t gid,
-                                            uint64_t scale,
-                                            uint64_t thr, Bits128 &acc, unsigned long long &cut_b,
+// each l is checked against g(S_S), from the largest down: A + M (F_b + B_b),
+// a part of it, grows as l falls, so the first l where it alone is too large
+// ends the walk (most parents of the paper's bound end at their first l).
+__device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t, int32_t A,
+                                            int32_t Bm, const ParentCtx &q, int kb, uint32_t gid,
+                                            int32_t top, Bits128 &acc, unsigned long long &cut_b,
                                             unsigned long long &cut_m, unsigned long long &cut_r) {
     const int S = p.S, M = p.M, L = t.L(), a = S - 2, b = S - 1;
     const int c = q.c;
     const int lmax = L - c - 1;
     const int hi_mem0 = min(lmax, (int)__ldg(p.lim + ((size_t)gid * S + a) * 128 + c));
+    // stage b fits [c2, L) exactly for the set feasibility bits of depth b,
+    // a suffix of positions: the smallest l is the first set bit above c
+    const uint4 fb = __ldg(p.feas + (size_t)gid * (S + 1) + b);
     const int hi_mem = min(hi_mem0, q.rcap);
     cut_r += (unsigned long long)(hi_mem0 - hi_mem);
     int hi = hi_mem;
     if (p.prune) {  // g(S_{S-1}) grows with l
         int lo = 0;
         while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1, c2 = c + mid;
-            const Sums v = sums_from(t, q.k, q.at, c2);
-            const int64_t F = v.f, B = v.b, d = v.d;
-            if ((uint64_t)(A + (int64_t)M * (F + B) + max(Bm, d)) * scale <= thr) lo = mid;
+            const int mid = (lo + hi + 1) >> 1;
+            const Sums v = sums_from(t, q.k, q.at, c + mid);
+            if (A + M * (v.f + v.b) + max(Bm, v.d) <= top) lo = mid;
             else hi = mid - 1;
         }
     }
-    // stage b fits [c2, L) exactly for the set feasibility bits of depth b,
-    // a suffix of positions: the smallest l is the first set bit above c
-    const uint4 fb = __ldg(p.feas + (size_t)gid * (S + 1) + b);
     const Bits128 above = range_bits(c + 1, L - 1);
     const uint32_t m0 = fb.x & above.w[0], m1 = fb.y & above.w[1], m2 = fb.z & above.w[2],
                    m3 = fb.w & above.w[3];
@@ -546,7 +533,7 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
     for (int i = 0; i < 4; ++i) acc.w[i] = 0;
     int n = 0;
     const Sums end = sums(t, kb, L);
-    for (int l = lo; l <= hi; ++l) {
+    for (int l = hi; l >= lo; --l) {
         const int c2 = c + l;
         // ridge rule for the last stage, after this one took l layers
         if (p.ridge && L - c2 > ridge_cap(ridge_next(q.rstate, q.rta, l), q.rtb)) {
@@ -554,12 +541,16 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
             continue;
         }
         if (p.prune) {
-            const Sums va = sums_from(t, q.k, q.at, c2), vb = sums(t, kb, c2);
-            const int64_t Fa = va.f, Ba = va.b, da = va.d;
-            const int64_t Fb = end.f - vb.f, Bb = end.b - vb.b, db = end.d - vb.d;
-            const int64_t g =
-                A + Fa + q.pf + (int64_t)M * (Fb + Bb) + max(max(Bm, da) + Ba + q.pb, db);
-            if ((uint64_t)g * scale > thr) {
+            const Sums vb = sums(t, kb, c2);
+            const int32_t least = A + M * (end.f - vb.f + end.b - vb.b);
+            if (least > top && !p.ridge) {  // and so for every smaller l
+                cut_b += (unsigned long long)(l - lo + 1);
+                break;
+            }
+            const Sums va = sums_from(t, q.k, q.at, c2);
+            const int32_t g =
+                least + va.f + q.pf + max(max(Bm, va.d) + va.b + q.pb, end.d - vb.d);
+            if (g > top) {
                 ++cut_b;
                 continue;
             }
@@ -571,6 +562,13 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
     cut_m += (unsigned long long)(lmax - hi_mem0) + (unsigned long long)(lo - 1 < hi ? lo - 1 : hi);
     cut_b += (unsigned long long)(hi_mem - hi);
     return n;
+}
+
+// Largest makespan T of a slice with T * scale <= thr (thr = ~0: no
+// incumbent).  Makespans are below 2^31.
+__device__ __forceinline__ int32_t top_makespan(uint64_t thr, uint64_t scale) {
+    const uint64_t top = scale == 1 ? thr : thr / scale;
+    return top > 0x7fffffffull ? 0x7fffffff : (int32_t)top;
 }
 
 // Small frontiers: one warp per parent.  Lane j tests the layer counts
@@ -606,9 +604,9 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
         ridge_ctx(q, p.ridge != 0, pv.b.z, q.k, kb, t.n_tp());
         const int2 edge = p.prune == 2 ? p2p(t, q.k, kb) : make_int2(0, 0);
         const int32_t pf = edge.x, pb = edge.y;
-        const uint64_t scale = sr.scale;
+        const int32_t top = top_makespan(thr, sr.scale);
         const uint32_t gid = sr.gid;
-        const int64_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
+        const int32_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
         const int lmax = COMPLETE ? L - c - 1 : L - c - (S - X - 1);
         const int hi_mem0 = min(lmax, (int)__ldg(p.lim + ((size_t)gid * S + X) * 128 + c));
         const int hi_mem = min(hi_mem0, q.rcap);  // ridge rule: a cap on the layer count
@@ -627,9 +625,7 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
             bool g_ok = false, cand = false, ok = false;
             if (in_mem) {
                 const Sums v = sums_from(t, q.k, q.at, c2);
-                const int64_t F = v.f, B = v.b, d = v.d;
-                g_ok = !p.prune ||
-                       (uint64_t)(A + (int64_t)M * (F + B) + max(Bm, d)) * scale <= thr;
+                g_ok = !p.prune || A + M * (v.f + v.b) + max(Bm, v.d) <= top;
                 const uint32_t word2 = (c2 >> 5) == 0 ? f.x : (c2 >> 5) == 1 ? f.y
                                      : (c2 >> 5) == 2 ? f.z : f.w;
                 cand = g_ok && ((word2 >> (c2 & 31)) & 1u);
@@ -639,18 +635,15 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
                     cand = false, ++n_ridge_b;
                 ok = cand;
                 if (cand) {
-                    const int64_t A2 = A + F + pf, Bm2 = max(Bm, d) + B + pb;
+                    const int32_t A2 = A + v.f + pf, Bm2 = max(Bm, v.d) + v.b + pb;
                     if (COMPLETE) {
                         if (p.prune) {
                             const Sums w = sums_from(t, kb, sums(t, kb, c2), L);
-                            const int64_t Fb = w.f, Bb = w.b, db = w.d;
-                            ok = (uint64_t)(A2 + (int64_t)M * (Fb + Bb) + max(Bm2, db)) * scale <=
-                                 thr;
+                            ok = A2 + M * (w.f + w.b) + max(Bm2, w.d) <= top;
                         }
                     } else if (p.prune == 2) {
                         const int2 n = vrow[c2];
-                        ok = n.x != kNoCompletion && (uint64_t)(A2 + n.x) * scale <= thr &&
-                             (uint64_t)(A2 + Bm2 + n.y) * scale <= thr;
+                        ok = n.x != kNoCompletion && A2 + n.x <= top && A2 + Bm2 + n.y <= top;
                     }
                 }
             }
@@ -798,14 +791,13 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
                 q.pf = e.x;
                 q.pb = e.y;
             }
-            const uint64_t scale = sr.scale;
-            const int64_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
-            n = COMPLETE ? complete_set(p, t, A, Bm, q, sr.cls[X + 1], sr.gid, scale, thr, acc, lb,
-                                        lm, lr)
+            const int32_t top = top_makespan(thr, sr.scale);
+            const int32_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
+            n = COMPLETE ? complete_set(p, t, A, Bm, q, sr.cls[X + 1], sr.gid, top, acc, lb, lm, lr)
                          : expand_set(p, t, A, Bm, q, sr.gid,
                                       vsm ? vsm + (size_t)slice * 128
                                           : (vdepth ? vdepth + (size_t)sr.vslot * 128 : nullptr),
-                                      scale, thr, acc, lb, lm, lr);
+                                      top, acc, lb, lm, lr);
         }
         int incl = n;
 #pragma unroll

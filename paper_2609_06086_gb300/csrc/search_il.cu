@@ -68,82 +68,102 @@ __device__ __forceinline__ void put_cut(Vec32 &v, int i, int c) {
     else v.b.x = (v.b.x & m) | b;
 }
 
-// Per-device sums over the virtual stages placed so far (stages 0..placed-1).
+// Per-device sums over the virtual stages placed so far.  Times are lengths of
+// DAG paths of a plan, so they fit in 32 bits under the overflow guard.
 template <int N>
 struct IlAcc {
     int32_t ser[N];  // M * sum (F + B) over the device's placed chunks
     int32_t ds[N];   // sum dsync over them
     int64_t wt[N];   // resident bytes (weights, optimizer state) over them
     int32_t A[N], Bs[N];  // prune 2: fill and drain sums before the device's first chunk
-    int32_t runF, runB;   // running sums over the placed chunk-0 stages
-    int placed;
 };
 
-// Adds virtual stage i = layers [c0, c1) to the sums (device i % N).
+// The sums of the first x virtual stages of an entry; *c: where they end.
+// The stages go by rounds over the devices, so a stage's device is a constant
+// after unrolling (with the device a runtime value, every sum was selected
+// from all of them).
 template <int N>
-__device__ __forceinline__ void il_add(IlAcc<N> &a, const Tab &t, const int (&cls)[N], int M,
-                                       int i, int c0, int c1) {
-    const int d = i % N;
-    int k = cls[0];
+__device__ __forceinline__ void il_sums(IlAcc<N> &a, const Tab &t, const int (&cls)[N], int M,
+                                        const Vec32 &pv, int x, int *c) {
+    int c0 = 0, runF = 0, runB = 0;
 #pragma unroll
-    for (int dd = 1; dd < N; ++dd) k = dd == d ? cls[dd] : k;
-    const Sums v = sums_from(t, k, sums(t, k, c0), c1);
-    const int32_t F = v.f, B = v.b, D = v.d;
-    const int64_t W = Pw(t, k, c1) - Pw(t, k, c0);
+    for (int d = 0; d < N; ++d) {  // chunk 0
+        a.ser[d] = a.ds[d] = a.A[d] = a.Bs[d] = 0;
+        a.wt[d] = 0;
+        if (d < x) {
+            const int c1 = cut_byte(pv, d), k = cls[d];
+            const Sums v = sums_from(t, k, sums(t, k, c0), c1);
+            a.ser[d] = M * (v.f + v.b);
+            a.ds[d] = v.d;
+            a.wt[d] = Pw(t, k, c1) - Pw(t, k, c0);
+            a.A[d] = runF;
+            a.Bs[d] = runB;
+            // the edge from device d to the next one
+            const int2 e = p2p(t, k, cls[(d + 1) % N]);
+            runF += v.f + e.x;
+            runB += v.b + e.y;
+            c0 = c1;
+        }
+    }
+    // the fill and drain sums of a device whose first chunk comes next
 #pragma unroll
-    for (int dd = 0; dd < N; ++dd)
-        if (dd == d) {
-            a.ser[dd] += M * (F + B);
-            a.ds[dd] += D;
-            a.wt[dd] += W;
-            if (i < N) {
-                a.A[dd] = a.runF;
-                a.Bs[dd] = a.runB;
+    for (int d = 0; d < N; ++d)
+        if (d == x) {
+            a.A[d] = runF;
+            a.Bs[d] = runB;
+        }
+#pragma unroll 1
+    for (int s = N; s < x; s += N) {
+#pragma unroll
+        for (int d = 0; d < N; ++d)
+            if (s + d < x) {
+                const int c1 = cut_byte(pv, s + d), k = cls[d];
+                const Sums v = sums_from(t, k, sums(t, k, c0), c1);
+                a.ser[d] += M * (v.f + v.b);
+                a.ds[d] += v.d;
+                a.wt[d] += Pw(t, k, c1) - Pw(t, k, c0);
+                c0 = c1;
+            }
+    }
+    *c = c0;
+}
+
+// v[d] for a runtime d
+template <int N, class T>
+__device__ __forceinline__ T il_pick(const T (&v)[N], int d) {
+    T r = v[0];
+#pragma unroll
+    for (int dd = 1; dd < N; ++dd) r = dd == d ? v[dd] : r;
+    return r;
+}
+
+// Device d's term of the lower bound with its chunks' totals ser and ds, and
+// ds0 the all-reduce of device 0's chunks.
+__device__ __forceinline__ int32_t il_term(int prune, int32_t A, int32_t Bs, int32_t ser,
+                                           int32_t ds, int32_t ds0) {
+    return prune == 2 ? A + ser + max(ds, Bs + ds0) : ser + ds;
+}
+
+// Lower bound over the devices other than u and v whose first chunk is among
+// the first `placed` virtual stages (all of them for prune 1: a device without
+// chunks has no serial work), in the two parts that device 0's all-reduce ds0
+// splits it into: max(*fixed, *moving + ds0).
+template <int N>
+__device__ __forceinline__ void il_others(const IlAcc<N> &a, int prune, int placed, int u, int v,
+                                          int32_t *fixed, int32_t *moving) {
+    int32_t f = 0, m = INT32_MIN / 2;
+#pragma unroll
+    for (int d = 0; d < N; ++d)
+        if (d != u && d != v) {
+            if (prune == 2 && d < placed) {
+                f = max(f, a.A[d] + a.ser[d] + a.ds[d]);
+                m = max(m, a.A[d] + a.ser[d] + a.Bs[d]);
+            } else if (prune != 2) {
+                f = max(f, a.ser[d] + a.ds[d]);
             }
         }
-    if (i < N) {
-        // the edge from virtual stage i (device d) to i + 1 (device (d+1) % N)
-        int kn = cls[0];
-#pragma unroll
-        for (int dd = 0; dd < N; ++dd) kn = dd == (d + 1) % N ? cls[dd] : kn;
-        const int2 e = p2p(t, k, kn);
-        a.runF += F + e.x;
-        a.runB += B + e.y;
-    }
-    a.placed = i + 1;
-}
-
-template <int N>
-__device__ __forceinline__ void il_init(IlAcc<N> &a) {
-#pragma unroll
-    for (int dd = 0; dd < N; ++dd) {
-        a.ser[dd] = a.ds[dd] = a.A[dd] = a.Bs[dd] = 0;
-        a.wt[dd] = 0;
-    }
-    a.runF = a.runB = 0;
-    a.placed = 0;
-}
-
-// Lower bound of every completion of the placed stages.
-template <int N>
-__device__ __forceinline__ int64_t il_bound(const IlAcc<N> &a, int prune) {
-    int64_t lb = 0;
-#pragma unroll
-    for (int dd = 0; dd < N; ++dd) {
-        int64_t v = (int64_t)a.ser[dd] + a.ds[dd];
-        if (prune == 2 && dd < a.placed)
-            v = (int64_t)a.A[dd] + a.ser[dd] + max((int64_t)a.ds[dd], (int64_t)a.Bs[dd] + a.ds[0]);
-        lb = max(lb, v);
-    }
-    return lb;
-}
-
-template <int N>
-__device__ __forceinline__ int64_t il_weight(const IlAcc<N> &a, int d) {
-    int64_t w = a.wt[0];
-#pragma unroll
-    for (int dd = 1; dd < N; ++dd) w = dd == d ? a.wt[dd] : w;
-    return w;
+    *fixed = f;
+    *moving = m;
 }
 
 }  // namespace
@@ -220,7 +240,7 @@ __device__ __forceinline__ uint4 il_meta_rt(const uint8_t *cls, int N, int n_tp,
 }
 
 template <int N>
-__global__ void __launch_bounds__(kIlThreads) il_level_kernel(IlLevelParams p) {
+__global__ void __launch_bounds__(kIlThreads, 3) il_level_kernel(IlLevelParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint64_t bar;
     const long long n_in = p.n_in;
@@ -255,57 +275,91 @@ __global__ void __launch_bounds__(kIlThreads) il_level_kernel(IlLevelParams p) {
         if (live) {
             const SliceRec &sr = p.slices[sl];
             M = sr.M;
-            const uint64_t scale = sr.scale;
+            // the largest makespan that does not beat the incumbent
+            const uint64_t lim = !p.prune ? ~0ull : sr.scale == 1 ? thr : thr / sr.scale;
+            const int32_t top = lim > 0x7fffffffull ? 0x7fffffff : (int32_t)lim;
 #pragma unroll
             for (int d = 0; d < N; ++d) cls[d] = sr.cls[d];
             IlAcc<N> a;
-            il_init(a);
-            for (int s = 0; s < x; ++s) {
-                const int c1 = cut_byte(pv, s);
-                il_add(a, t, cls, M, s, c, c1);
-                c = c1;
-            }
-            const int dn = x % N;
-            int kn = cls[0];
-#pragma unroll
-            for (int d = 1; d < N; ++d) kn = d == dn ? cls[d] : kn;
-            const int64_t w0 = il_weight(a, dn) - Pw(t, kn, c), capn = cap_of(t, kn);
+            il_sums(a, t, cls, M, pv, x, &c);
+            // the new stage's device: its class, sums and the sums at c
+            const int dn = x % N, kn = il_pick(cls, dn);
+            const int32_t An = il_pick(a.A, dn), Bn = il_pick(a.Bs, dn);
+            const int32_t sn = il_pick(a.ser, dn), tn = il_pick(a.ds, dn);
+            const Sums at = sums(t, kn, c);
+            const int64_t wn = cap_of(t, kn) - il_pick(a.wt, dn) + Pw(t, kn, c);
+            auto mem_n = [&](int l) { return Pw(t, kn, c + l) <= wn; };
+            int32_t fixed, moving;
             if (!complete) {
                 // resident bytes and the bound both grow with l: [1, hi]
                 const int lmax = L - c - (J - x - 1);
-                const int hi_mem =
-                    il_last_true(lmax, [&](int l) { return w0 + Pw(t, kn, c + l) <= capn; });
+                const int hi_mem = il_last_true(lmax, mem_n);
                 hi = hi_mem;
-                if (p.prune)
+                if (p.prune) {
+                    il_others(a, p.prune, x, dn, dn, &fixed, &moving);
                     hi = il_last_true(hi_mem, [&](int l) {
-                        IlAcc<N> b = a;
-                        il_add(b, t, cls, M, x, c, c + l);
-                        return (uint64_t)il_bound(b, p.prune) * scale <= thr;
+                        const Sums v = sums_from(t, kn, at, c + l);
+                        const int32_t ds = tn + v.d, ds0 = dn == 0 ? ds : a.ds[0];
+                        const int32_t own =
+                            il_term(p.prune, An, Bn, sn + M * (v.f + v.b), ds, ds0);
+                        return max(max(fixed, moving + ds0), own) <= top;
                     });
+                }
                 n = hi;
                 lm += (unsigned long long)(lmax - hi_mem);
                 lb += (unsigned long long)(hi_mem - hi);
             } else {
-                // stage x = J-2 takes l layers, stage J-1 the rest; each l is
-                // tested (the last stage's terms shrink as l grows)
-                const int db = (J - 1) % N;
-                int kb = cls[0];
+                // stage x = J-2 takes l layers, stage J-1 the rest.  The memory
+                // of the two devices allows a range of l (their needs grow and
+                // fall with l); within it the last stage's serial work falls
+                // with l, so the first l from the top where it alone is too
+                // large ends the walk.
+                const int db = (J - 1) % N, kb = il_pick(cls, db);
+                const int32_t Ab = il_pick(a.A, db), Bb = il_pick(a.Bs, db);
+                const int32_t sb = il_pick(a.ser, db), tb = il_pick(a.ds, db);
+                const Sums end = sums(t, kb, L);
+                const int64_t wb = cap_of(t, kb) - il_pick(a.wt, db) - Pw(t, kb, L);
+                const int lmax = L - c - 1;
+                int top_l, low_l;
+                if (db == dn) {  // one device holds both stages: no dependence on l
+                    const bool ok = Pw(t, kn, L) <= wn;
+                    top_l = ok ? lmax : 0;
+                    low_l = 1;
+                } else {
+                    top_l = il_last_true(lmax, mem_n);
+                    // the least l that leaves device db with what it can hold
+                    low_l = 1 + il_last_true(top_l, [&](int l) { return -Pw(t, kb, c + l) > wb; });
+                }
+                lm += (unsigned long long)(lmax - max(0, top_l - low_l + 1));
+                il_others(a, p.prune, J, dn, db, &fixed, &moving);
+                for (int l = top_l; l >= low_l; --l) {
+                    if (p.prune) {
+                        const Sums v = sums_from(t, kn, at, c + l), vb = sums(t, kb, c + l);
+                        const int32_t last = M * (end.f - vb.f + end.b - vb.b);
+                        if (last > top) {  // and so for every smaller l
+                            lb += (unsigned long long)(l - low_l + 1);
+                            break;
+                        }
+                        int32_t ser_n = sn + M * (v.f + v.b), ds_n = tn + v.d;
+                        int32_t ser_b = sb + last, ds_b = tb + end.d - vb.d;
+                        if (db == dn) {
+                            ser_n += last;
+                            ds_n += end.d - vb.d;
+                            ser_b = ser_n;
+                            ds_b = ds_n;
+                        }
+                        const int32_t ds0 = dn == 0 ? ds_n : db == 0 ? ds_b : a.ds[0];
+                        const int32_t g = max(max(il_term(p.prune, An, Bn, ser_n, ds_n, ds0),
+                                                  il_term(p.prune, Ab, Bb, ser_b, ds_b, ds0)),
+                                              max(fixed, moving + ds0));
+                        if (g > top) {
+                            ++lb;
+                            continue;
+                        }
+                    }
 #pragma unroll
-                for (int d = 1; d < N; ++d) kb = d == db ? cls[d] : kb;
-                const int64_t capb = cap_of(t, kb);
-                for (int l = 1; l <= L - c - 1; ++l) {
-                    IlAcc<N> b = a;
-                    il_add(b, t, cls, M, x, c, c + l);
-                    il_add(b, t, cls, M, J - 1, c + l, L);
-                    if (il_weight(b, dn) > capn || il_weight(b, db) > capb) {
-                        ++lm;
-                        continue;
-                    }
-                    if (p.prune && (uint64_t)il_bound(b, p.prune) * scale > thr) {
-                        ++lb;
-                        continue;
-                    }
-                    pass[(l - 1) >> 5] |= 1u << ((l - 1) & 31);
+                    for (int wd = 0; wd < 4; ++wd)
+                        pass[wd] |= ((l - 1) >> 5) == wd ? 1u << ((l - 1) & 31) : 0u;
                     ++n;
                 }
             }
