@@ -428,7 +428,7 @@ __device__ __forceinline__ ParentCtx parent_ctx(const Tab &t, int k, int c) {
 // (c, c+hi] from which the remaining layers still fit the remaining stages
 // (feasibility bits).
 // `top` is the largest makespan that does not beat the incumbent's objective
-// in the parent's slice (top_makespan).  Every bound tested is the length of a
+// in the parent's slice (TopMakespan).  Every bound tested is the length of a
 // DAG path of a plan of the slice, so it fits in 32 bits under the overflow
 // guard.
 __device__ __forceinline__ int expand_set(const ExpandParams &p, const Tab &t, int32_t A,
@@ -509,30 +509,37 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
     const int c = q.c;
     const int lmax = L - c - 1;
     const int hi_mem0 = min(lmax, (int)__ldg(p.lim + ((size_t)gid * S + a) * 128 + c));
-    // stage b fits [c2, L) exactly for the set feasibility bits of depth b,
-    // a suffix of positions: the smallest l is the first set bit above c
+    // stage b fits [c2, L) exactly for the set feasibility bits of depth b, the
+    // positions from some first one to L - 1
     const uint4 fb = __ldg(p.feas + (size_t)gid * (S + 1) + b);
     const int hi_mem = min(hi_mem0, q.rcap);
     cut_r += (unsigned long long)(hi_mem0 - hi_mem);
+    const int least_start = fb.x ? __ffs(fb.x) - 1 : fb.y ? 31 + __ffs(fb.y) : fb.z ? 63 + __ffs(fb.z)
+                          : fb.w ? 95 + __ffs(fb.w) : 128;
+    const int first = max(c + 1, least_start);
+    const int lo = first - c;
+    for (int i = 0; i < 4; ++i) acc.w[i] = 0;
+    const Sums end = sums(t, kb, L);
+    auto g_prefix = [&](int l) {  // g(S_{S-1}), grows with l
+        const Sums v = sums_from(t, q.k, q.at, c + l);
+        return A + M * (v.f + v.b) + max(Bm, v.d);
+    };
+    auto least_end = [&](int l, Sums &vb) {  // a part of g(S_S), falls as l grows
+        vb = sums(t, kb, c + l);
+        return A + M * (end.f - vb.f + end.b - vb.b);
+    };
+    cut_m += (unsigned long long)(lmax - hi_mem0);
+    Sums vb;
     int hi = hi_mem;
-    if (p.prune) {  // g(S_{S-1}) grows with l
-        int lo = 0;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            const Sums v = sums_from(t, q.k, q.at, c + mid);
-            if (A + M * (v.f + v.b) + max(Bm, v.d) <= top) lo = mid;
+    if (p.prune) {
+        int low = 0;
+        while (low < hi) {
+            const int mid = (low + hi + 1) >> 1;
+            if (g_prefix(mid) <= top) low = mid;
             else hi = mid - 1;
         }
     }
-    const Bits128 above = range_bits(c + 1, L - 1);
-    const uint32_t m0 = fb.x & above.w[0], m1 = fb.y & above.w[1], m2 = fb.z & above.w[2],
-                   m3 = fb.w & above.w[3];
-    const int first = m0 ? __ffs(m0) - 1 : m1 ? 31 + __ffs(m1) : m2 ? 63 + __ffs(m2)
-                    : m3 ? 95 + __ffs(m3) : 128;
-    const int lo = first - c;
-    for (int i = 0; i < 4; ++i) acc.w[i] = 0;
     int n = 0;
-    const Sums end = sums(t, kb, L);
     for (int l = hi; l >= lo; --l) {
         const int c2 = c + l;
         // ridge rule for the last stage, after this one took l layers
@@ -541,8 +548,7 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
             continue;
         }
         if (p.prune) {
-            const Sums vb = sums(t, kb, c2);
-            const int32_t least = A + M * (end.f - vb.f + end.b - vb.b);
+            const int32_t least = least_end(l, vb);
             if (least > top && !p.ridge) {  // and so for every smaller l
                 cut_b += (unsigned long long)(l - lo + 1);
                 break;
@@ -559,16 +565,9 @@ __device__ __forceinline__ int complete_set(const ExpandParams &p, const Tab &t,
         for (int wd = 0; wd < 4; ++wd) acc.w[wd] |= (c2 >> 5) == wd ? 1u << (c2 & 31) : 0u;
         ++n;
     }
-    cut_m += (unsigned long long)(lmax - hi_mem0) + (unsigned long long)(lo - 1 < hi ? lo - 1 : hi);
+    cut_m += (unsigned long long)(lo - 1 < hi ? lo - 1 : hi);
     cut_b += (unsigned long long)(hi_mem - hi);
     return n;
-}
-
-// Largest makespan T of a slice with T * scale <= thr (thr = ~0: no
-// incumbent).  Makespans are below 2^31.
-__device__ __forceinline__ int32_t top_makespan(uint64_t thr, uint64_t scale) {
-    const uint64_t top = scale == 1 ? thr : thr / scale;
-    return top > 0x7fffffffull ? 0x7fffffff : (int32_t)top;
 }
 
 // Small frontiers: one warp per parent.  Lane j tests the layer counts
@@ -583,7 +582,7 @@ __device__ __forceinline__ int32_t top_makespan(uint64_t thr, uint64_t scale) {
 template <bool COMPLETE, int X>
 __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab &t,
                                                 long long n_in, const int2 *vsm,
-                                                const int2 *vdepth, uint64_t thr,
+                                                const int2 *vdepth, TopMakespan &tops,
                                                 unsigned long long &emitted,
                                                 unsigned long long &cb, unsigned long long &cm,
                                                 unsigned long long &cr,
@@ -604,7 +603,7 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
         ridge_ctx(q, p.ridge != 0, pv.b.z, q.k, kb, t.n_tp());
         const int2 edge = p.prune == 2 ? p2p(t, q.k, kb) : make_int2(0, 0);
         const int32_t pf = edge.x, pb = edge.y;
-        const int32_t top = top_makespan(thr, sr.scale);
+        const int32_t top = tops.of(sr.scale);
         const uint32_t gid = sr.gid;
         const int32_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
         const int lmax = COMPLETE ? L - c - 1 : L - c - (S - X - 1);
@@ -713,6 +712,19 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
     }
 }
 
+// Slots [lo, hi) of the output, those below its capacity, become holes (by
+// the lanes of one warp).
+template <bool COMPLETE>
+__device__ __forceinline__ void level_holes(const ExpandParams &p, unsigned long long lo,
+                                            unsigned long long hi) {
+    const Vec32 hole = {make_uint4(COMPLETE ? kLeafHole : kPrefixHole, 0, 0, 0),
+                        make_uint4(0, 0, 0, 0)};
+    for (unsigned long long e = lo + (threadIdx.x & 31); e < hi && e < p.cap; e += 32) {
+        if (COMPLETE) store32(p.leaves + e, hole);
+        else store32(p.out + e, hole);
+    }
+}
+
 // One warp per group of 32 consecutive parents: each lane finds its
 // parent's children (a 128-bit set of cut positions), the warp reserves
 // output slots with one atomic and writes them -- or, when the output is
@@ -724,6 +736,8 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
     // completion-bound rows of depth X+1 of every slot (contiguous), by TMA;
     // all written before the previous kernel, so staged while it finishes
     __shared__ uint64_t bar;
+    __shared__ unsigned long long s_stats[5];
+    if (threadIdx.x < 5) s_stats[threadIdx.x] = 0;
     const bool use_v = !COMPLETE && p.prune == 2;
     const bool stage_v = use_v && p.vb_smem;
     // depth X+1 of the bound tables: the row of table row v is vdepth + 128 v
@@ -761,16 +775,30 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
     if ((long long)blockIdx.x * (kThreads / 32) >= (warp_mode ? n_in : n_work)) return;
     const int2 *vsm = stage_v ? reinterpret_cast<const int2 *>(sm + p.lay.bytes) : nullptr;
     const Tab t = tab_at(sm, p.lay);
-    const uint64_t thr = p.prune ? __ldcg(&p.inc->obj) : ~0ull;
+    TopMakespan tops(p.prune ? __ldcg(&p.inc->obj) : ~0ull);
     const int lane = threadIdx.x & 31;
     const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     unsigned long long emitted = 0, cb = 0, cm = 0, cr = 0, written_parents = 0;
     if (warp_mode)
-        level_warp_mode<COMPLETE, X>(p, t, n_in, vsm, vdepth, thr, emitted, cb, cm, cr,
+        level_warp_mode<COMPLETE, X>(p, t, n_in, vsm, vdepth, tops, emitted, cb, cm, cr,
                                      written_parents);
+    // Output slots are reserved by atomics on one counter, which serialise, so a
+    // warp with many groups ahead reserves a run of slots and takes its
+    // children's places from it; its last groups reserve what they need, and
+    // what is then left of the run becomes holes.  (Under the paper's bound the
+    // 70B-like search has 4 children per parent, one completion per 16.)
+    int run = 0;
+    if (!p.exact && !warp_mode)
+        run = COMPLETE ? (n_work >= 128 * n_warps ? 64 : 0)
+                       : (n_work >= 64 * n_warps ? 512 : n_work >= 16 * n_warps ? 128 : 0);
+    unsigned long long cur = 0;  // the open run: next slot, slots left
+    int left = 0;
     for (long long w = warp; !warp_mode && w < n_work; w += n_warps) {
         const long long g = p.groups ? (long long)p.groups[w] : w;
         const long long i = g * 32 + lane;
+        // the warp's next group on its way to L1 meanwhile
+        if (!p.groups && i + 32 * n_warps < n_in)
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(p.in + i + 32 * n_warps));
         Vec32 pv = {make_uint4(kPrefixHole, 0, 0, 0), make_uint4(0, 0, 0, 0)};
         if (i < n_in) pv = load32(p.in + i);
         const uint32_t slice = pv.a.x & 0xffffu;
@@ -791,7 +819,7 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
                 q.pf = e.x;
                 q.pb = e.y;
             }
-            const int32_t top = top_makespan(thr, sr.scale);
+            const int32_t top = tops.of(sr.scale);
             const int32_t A = (int32_t)pv.b.x, Bm = (int32_t)pv.b.y;
             n = COMPLETE ? complete_set(p, t, A, Bm, q, sr.cls[X + 1], sr.gid, top, acc, lb, lm, lr)
                          : expand_set(p, t, A, Bm, q, sr.gid,
@@ -806,9 +834,6 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
             if (lane >= o) incl += v;
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        unsigned long long base = 0;
-        if (lane == 0 && total > 0) base = atomicAdd(p.out_count, (unsigned long long)total);
-        base = __shfl_sync(0xffffffffu, base, 0);
         if (total == 0) {
             cb += lb;
             cm += lm;
@@ -816,73 +841,104 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
             written_parents += live;
             continue;
         }
-        unsigned long long pos = base + (unsigned long long)(incl - n);
-        if (base + (unsigned long long)total <= p.cap) {
+        // the group's first `left` children go to the warp's open run of
+        // slots, the others to a new one
+        const unsigned long long old = cur;
+        const int old_left = left, more = total - left;
+        unsigned long long base = 0;
+        bool room = true;
+        if (more > 0) {
+            const int size = w + (COMPLETE ? 64 : 8) * n_warps < n_work ? max(run, more) : more;
+            if (lane == 0) base = atomicAdd(p.out_count, (unsigned long long)size);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            room = base + (unsigned long long)size <= p.cap;
+            cur = base + (unsigned long long)more;
+            left = size - more;
+            if (!room) {
+                // what is reserved and within the capacity becomes holes
+                level_holes<COMPLETE>(p, old, old + old_left);
+                level_holes<COMPLETE>(p, base, base + size);
+                left = 0;
+                if (lane == 0) {
+                    const unsigned long long d = atomicAdd(p.n_deferred, 1ull);
+                    p.deferred[d] = (uint32_t)g;
+                }
+                continue;
+            }
+        } else {
+            cur += total;
+            left -= total;
+        }
+        int e = incl - n;  // index of the lane's next child in the group
 #pragma unroll
-            for (int wd = 0; wd < 4; ++wd) {
-                uint32_t m = acc.w[wd];
-                while (m) {
-                    const int c2 = 32 * wd + __ffs(m) - 1;
-                    m &= m - 1;
-                    if (COMPLETE) {
-                        // leaf: slice in bytes 0-3, cut[i] in byte 4+i; the
-                        // parent's cuts (bytes 2..15) move up two bytes
-                        Vec32 lf;
-                        lf.a.x = slice;
-                        lf.a.y = __funnelshift_r(pv.a.x, pv.a.y, 16);
-                        lf.a.z = __funnelshift_r(pv.a.y, pv.a.z, 16);
-                        lf.a.w = __funnelshift_r(pv.a.z, pv.a.w, 16);
-                        lf.b = make_uint4(pv.a.w >> 16, 0u, 0u, 0u);
-                        set_byte<4 + X>(lf, (uint32_t)c2);
-                        store32(p.leaves + pos++, lf);
-                    } else {
-                        Vec32 ch = pv;
-                        set_byte<2 + (X < 14 ? X : 0)>(ch, (uint32_t)c2);
-                        const Sums v = sums_from(t, q.k, q.at, c2);
-                        ch.b.x = (uint32_t)((int32_t)pv.b.x + v.f + q.pf);
-                        ch.b.y = (uint32_t)(max((int32_t)pv.b.y, v.d) + v.b + q.pb);
-                        ch.b.z = p.ridge ? ridge_next(q.rstate, q.rta, c2 - q.c) : 0u;
-                        store32(p.out + pos++, ch);
-                    }
+        for (int wd = 0; wd < 4; ++wd) {
+            uint32_t m = acc.w[wd];
+            while (m) {
+                const int c2 = 32 * wd + __ffs(m) - 1;
+                m &= m - 1;
+                const unsigned long long pos = e < old_left ? old + e : base + (e - old_left);
+                ++e;
+                if (COMPLETE) {
+                    // leaf: slice in bytes 0-3, cut[i] in byte 4+i; the
+                    // parent's cuts (bytes 2..15) move up two bytes
+                    Vec32 lf;
+                    lf.a.x = slice;
+                    lf.a.y = __funnelshift_r(pv.a.x, pv.a.y, 16);
+                    lf.a.z = __funnelshift_r(pv.a.y, pv.a.z, 16);
+                    lf.a.w = __funnelshift_r(pv.a.z, pv.a.w, 16);
+                    lf.b = make_uint4(pv.a.w >> 16, 0u, 0u, 0u);
+                    set_byte<4 + X>(lf, (uint32_t)c2);
+                    store32(p.leaves + pos, lf);
+                } else {
+                    Vec32 ch = pv;
+                    set_byte<2 + (X < 14 ? X : 0)>(ch, (uint32_t)c2);
+                    const Sums v = sums_from(t, q.k, q.at, c2);
+                    ch.b.x = (uint32_t)((int32_t)pv.b.x + v.f + q.pf);
+                    ch.b.y = (uint32_t)(max((int32_t)pv.b.y, v.d) + v.b + q.pb);
+                    ch.b.z = p.ridge ? ridge_next(q.rstate, q.rta, c2 - q.c) : 0u;
+                    store32(p.out + pos, ch);
                 }
             }
-            emitted += n;
-            cb += lb;
-            cm += lm;
-            cr += lr;
-            written_parents += live;
-        } else {
-            // no room: mark this warp's reserved slots below cap as holes
-            const Vec32 hole = {make_uint4(COMPLETE ? kLeafHole : kPrefixHole, 0, 0, 0),
-                                make_uint4(0, 0, 0, 0)};
-            for (unsigned long long e = pos; e < pos + (unsigned long long)n && e < p.cap; ++e) {
-                if (COMPLETE) store32(p.leaves + e, hole);
-                else store32(p.out + e, hole);
-            }
-            if (lane == 0) {
-                const unsigned long long d = atomicAdd(p.n_deferred, 1ull);
-                p.deferred[d] = (uint32_t)g;
-            }
         }
+        emitted += n;
+        cb += lb;
+        cm += lm;
+        cr += lr;
+        written_parents += live;
     }
+    if (left > 0) level_holes<COMPLETE>(p, cur, cur + left);
+    // Statistics: in one atomic per block and counter where many warps work (one
+    // per warp took a few microseconds at the end of such a launch), straight
+    // from the few warps of a small frontier.
+    unsigned long long mine[5] = {emitted, cb, cm, cr, written_parents};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        emitted += __shfl_xor_sync(0xffffffffu, emitted, o);
-        cb += __shfl_xor_sync(0xffffffffu, cb, o);
-        cm += __shfl_xor_sync(0xffffffffu, cm, o);
-        cr += __shfl_xor_sync(0xffffffffu, cr, o);
-        written_parents += __shfl_xor_sync(0xffffffffu, written_parents, o);
-    }
-    if (lane == 0) {
-        if (cr) atomicAdd(p.stats + kStPrunedRidge, cr);
-        if (emitted) atomicAdd(p.stats + (COMPLETE ? kStLeaves : kStPrefixes), emitted);
-        if (cb) atomicAdd(p.stats + kStPrunedBound, cb);
-        if (cm) atomicAdd(p.stats + kStPrunedMemory, cm);
-        if (written_parents) {
-            atomicAdd(p.stats + (COMPLETE ? kStParentsComplete : kStParentsExpand), written_parents);
-            atomicAdd(p.stats + kStDepthParents + X, written_parents);
+    for (int q = 0; q < 5; ++q)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mine[q] += __shfl_xor_sync(0xffffffffu, mine[q], o);
+    if (!warp_mode) {
+        if (lane == 0) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q)
+                if (mine[q]) atomicAdd(&s_stats[q], mine[q]);
         }
-        if (emitted) atomicAdd(p.stats + kStDepthChildren + X, emitted);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q) mine[q] = s_stats[q];
+        }
+    }
+    if (warp_mode ? lane == 0 : threadIdx.x == 0) {
+        if (mine[0]) {
+            atomicAdd(p.stats + (COMPLETE ? kStLeaves : kStPrefixes), mine[0]);
+            atomicAdd(p.stats + kStDepthChildren + X, mine[0]);
+        }
+        if (mine[1]) atomicAdd(p.stats + kStPrunedBound, mine[1]);
+        if (mine[2]) atomicAdd(p.stats + kStPrunedMemory, mine[2]);
+        if (mine[3]) atomicAdd(p.stats + kStPrunedRidge, mine[3]);
+        if (mine[4]) {
+            atomicAdd(p.stats + (COMPLETE ? kStParentsComplete : kStParentsExpand), mine[4]);
+            atomicAdd(p.stats + kStDepthParents + X, mine[4]);
+        }
     }
 }
 

@@ -239,10 +239,28 @@ __device__ __forceinline__ uint4 il_meta_rt(const uint8_t *cls, int N, int n_tp,
     return il_meta_pack(tcode, tpc, cls[0], N, n_tp, M, V, slot);
 }
 
+// Slots [lo, hi) of the output, those below its capacity, become holes (by
+// the lanes of one warp).
+__device__ __forceinline__ void il_holes(const IlLevelParams &p, bool complete,
+                                         unsigned long long lo, unsigned long long hi) {
+    for (unsigned long long e = lo + (threadIdx.x & 31); e < hi && e < p.cap; e += 32) {
+        if (complete) {
+            p.rec[2 * e] = make_uint4(0u, 0u, 0u, 1u << 24);  // answered: skipped
+            p.rec[2 * e + 1] = make_uint4((uint32_t)e, 0u, 0u, 0u);
+            p.leaf_slice[e] = kIlHole;
+        } else {
+            const Vec32 hole = {make_uint4(kIlHole, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+            store32(p.out + e, hole);
+        }
+    }
+}
+
 template <int N>
 __global__ void __launch_bounds__(kIlThreads, 3) il_level_kernel(IlLevelParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint64_t bar;
+    __shared__ unsigned long long s_stats[4];
+    if (threadIdx.x < 4) s_stats[threadIdx.x] = 0;
     const long long n_in = p.n_in;
     const long long n_work = p.groups ? p.n_groups : (n_in + 31) / 32;
     // blocks without work leave before staging the tables
@@ -254,16 +272,27 @@ __global__ void __launch_bounds__(kIlThreads, 3) il_level_kernel(IlLevelParams p
     const Tab t = tab_at(sm, p.lay);
     const int L = t.L(), J = p.J, x = p.x, n_tp = t.n_tp();
     const bool complete = x == J - 2;
-    const uint64_t thr = p.prune ? __ldcg(&p.inc->obj) : ~0ull;
+    TopMakespan tops(p.prune ? __ldcg(&p.inc->obj) : ~0ull);
     const int lane = threadIdx.x & 31;
     const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
     unsigned long long emitted = 0, cut_b = 0, cut_m = 0, parents = 0;
+    // runs of output slots for a warp with many groups ahead, in a pass without
+    // a work list (level_kernel)
+    int run = 0;
+    if (!p.groups && 8 * n_in <= (long long)p.cap)
+        run = complete ? (n_work >= 32 * n_warps ? 64 : 0)
+                       : (n_work >= 64 * n_warps ? 512 : n_work >= 16 * n_warps ? 128 : 0);
+    unsigned long long cur = 0;  // the open run: next slot, slots left
+    int left = 0;
     for (long long w = warp; w < n_work; w += n_warps) {
         const long long g = p.groups ? (long long)p.groups[w] : w;
         const long long i = g * 32 + lane;
         Vec32 pv = {make_uint4(kIlHole, 0, 0, 0), make_uint4(0, 0, 0, 0)};
         if (i < n_in) pv = load32(p.in + i);
+        // the warp's next group on its way to L1 meanwhile
+        if (!p.groups && i + 32 * n_warps < n_in)
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(p.in + i + 32 * n_warps));
         const uint32_t sl = pv.a.x;
         const bool live = sl != kIlHole;
         int n = 0, c = 0, hi = 0, M = 0;
@@ -275,9 +304,7 @@ __global__ void __launch_bounds__(kIlThreads, 3) il_level_kernel(IlLevelParams p
         if (live) {
             const SliceRec &sr = p.slices[sl];
             M = sr.M;
-            // the largest makespan that does not beat the incumbent
-            const uint64_t lim = !p.prune ? ~0ull : sr.scale == 1 ? thr : thr / sr.scale;
-            const int32_t top = lim > 0x7fffffffull ? 0x7fffffff : (int32_t)lim;
+            const int32_t top = tops.of(sr.scale);
 #pragma unroll
             for (int d = 0; d < N; ++d) cls[d] = sr.cls[d];
             IlAcc<N> a;
@@ -332,6 +359,19 @@ __global__ void __launch_bounds__(kIlThreads, 3) il_level_kernel(IlLevelParams p
                 }
                 lm += (unsigned long long)(lmax - max(0, top_l - low_l + 1));
                 il_others(a, p.prune, J, dn, db, &fixed, &moving);
+                if (p.prune && db != dn && top_l >= low_l) {
+                    // device dn's own term grows with l: the counts above its
+                    // last one within the bound are cut
+                    const int own = il_last_true(top_l, [&](int l) {
+                        const Sums v = sums_from(t, kn, at, c + l);
+                        const int32_t ds = tn + v.d;
+                        return il_term(p.prune, An, Bn, sn + M * (v.f + v.b), ds,
+                                       dn == 0 ? ds : a.ds[0]) <= top;
+                    });
+                    const int last_l = max(own, low_l - 1);
+                    lb += (unsigned long long)(top_l - last_l);
+                    top_l = last_l;
+                }
                 for (int l = top_l; l >= low_l; --l) {
                     if (p.prune) {
                         const Sums v = sums_from(t, kn, at, c + l), vb = sums(t, kb, c + l);
@@ -377,73 +417,89 @@ __global__ void __launch_bounds__(kIlThreads, 3) il_level_kernel(IlLevelParams p
             parents += live;
             continue;
         }
+        // the first `left` children go to the warp's open run of slots, the
+        // others to a new one (level_kernel's reservation)
+        const unsigned long long old = cur;
+        const int old_left = left, more = total - left;
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(p.out_count, (unsigned long long)total);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        unsigned long long pos = base + (unsigned long long)(incl - n);
-        if (base + (unsigned long long)total <= p.cap) {
-            if (!complete) {
-                for (int l = 1; l <= hi; ++l) {
-                    Vec32 ch = pv;
-                    put_cut(ch, x, c + l);
-                    store32(p.out + pos++, ch);
+        if (more > 0) {
+            const int size = w + (complete ? 32 : 8) * n_warps < n_work ? max(run, more) : more;
+            if (lane == 0) base = atomicAdd(p.out_count, (unsigned long long)size);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            cur = base + (unsigned long long)more;
+            left = size - more;
+            if (base + (unsigned long long)size > p.cap) {
+                // no room: the reserved slots below the capacity become holes
+                // and the group is deferred
+                il_holes(p, complete, old, old + old_left);
+                il_holes(p, complete, base, base + size);
+                left = 0;
+                if (lane == 0) {
+                    const unsigned long long d = atomicAdd(p.n_deferred, 1ull);
+                    p.deferred[d] = (uint32_t)g;
                 }
-            } else {
-#pragma unroll
-                for (int wd = 0; wd < 4; ++wd) {
-                    uint32_t m = pass[wd];
-                    while (m) {
-                        const int l = 32 * wd + __ffs(m);
-                        m &= m - 1;
-                        Vec32 lf = pv;
-                        put_cut(lf, x, c + l);
-                        // cut[1..J-1] in bytes 0..14 of the record's first word;
-                        // byte 15 = 0: not answered yet
-                        p.rec[2 * pos] = make_uint4(lf.a.y, lf.a.z, lf.a.w, lf.b.x & 0x00ffffffu);
-                        p.rec[2 * pos + 1] = il_meta(cls, n_tp, M, p.V, (uint32_t)pos);
-                        p.leaf_slice[pos] = sl;
-                        ++pos;
-                    }
-                }
+                continue;
             }
-            emitted += (unsigned long long)n;
-            parents += live;
         } else {
-            // no room: the reserved slots below the capacity become holes and
-            // the group is deferred
-            for (unsigned long long e = pos; e < pos + (unsigned long long)n && e < p.cap; ++e) {
-                if (complete) {
-                    p.rec[2 * e] = make_uint4(0u, 0u, 0u, 1u << 24);  // answered: skipped
-                    p.rec[2 * e + 1] = make_uint4((uint32_t)e, 0u, 0u, 0u);
-                    p.leaf_slice[e] = kIlHole;
-                } else {
-                    const Vec32 hole = {make_uint4(kIlHole, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-                    store32(p.out + e, hole);
+            cur += total;
+            left -= total;
+        }
+        int e = incl - n;  // index of the lane's next child in the group
+        auto slot = [&]() {
+            const unsigned long long at = e < old_left ? old + e : base + (e - old_left);
+            ++e;
+            return at;
+        };
+        if (!complete) {
+            for (int l = 1; l <= hi; ++l) {
+                Vec32 ch = pv;
+                put_cut(ch, x, c + l);
+                store32(p.out + slot(), ch);
+            }
+        } else {
+#pragma unroll
+            for (int wd = 0; wd < 4; ++wd) {
+                uint32_t m = pass[wd];
+                while (m) {
+                    const int l = 32 * wd + __ffs(m);
+                    m &= m - 1;
+                    const unsigned long long pos = slot();
+                    Vec32 lf = pv;
+                    put_cut(lf, x, c + l);
+                    // cut[1..J-1] in bytes 0..14 of the record's first word;
+                    // byte 15 = 0: not answered yet
+                    const Vec32 rec = {make_uint4(lf.a.y, lf.a.z, lf.a.w, lf.b.x & 0x00ffffffu),
+                                       il_meta(cls, n_tp, M, p.V, (uint32_t)pos)};
+                    store32(p.rec + 2 * pos, rec);
+                    p.leaf_slice[pos] = sl;
                 }
             }
-            if (lane == 0) {
-                const unsigned long long d = atomicAdd(p.n_deferred, 1ull);
-                p.deferred[d] = (uint32_t)g;
-            }
         }
+        emitted += (unsigned long long)n;
+        parents += live;
     }
+    if (left > 0) il_holes(p, complete, cur, cur + left);
+    // the block's statistics in one atomic each
+    const unsigned long long mine[4] = {emitted, cut_b, cut_m, parents};
+    __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        emitted += __shfl_xor_sync(0xffffffffu, emitted, o);
-        cut_b += __shfl_xor_sync(0xffffffffu, cut_b, o);
-        cut_m += __shfl_xor_sync(0xffffffffu, cut_m, o);
-        parents += __shfl_xor_sync(0xffffffffu, parents, o);
+    for (int q = 0; q < 4; ++q) {
+        unsigned long long v = mine[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 && v) atomicAdd(&s_stats[q], v);
     }
-    if (lane == 0) {
-        if (emitted) {
-            atomicAdd(p.stats + (complete ? kStLeaves : kStPrefixes), emitted);
-            atomicAdd(p.stats + kStDepthChildren + x, emitted);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_stats[0]) {
+            atomicAdd(p.stats + (complete ? kStLeaves : kStPrefixes), s_stats[0]);
+            atomicAdd(p.stats + kStDepthChildren + x, s_stats[0]);
         }
-        if (cut_b) atomicAdd(p.stats + kStPrunedBound, cut_b);
-        if (cut_m) atomicAdd(p.stats + kStPrunedMemory, cut_m);
-        if (parents) {
-            atomicAdd(p.stats + (complete ? kStParentsComplete : kStParentsExpand), parents);
-            atomicAdd(p.stats + kStDepthParents + x, parents);
+        if (s_stats[1]) atomicAdd(p.stats + kStPrunedBound, s_stats[1]);
+        if (s_stats[2]) atomicAdd(p.stats + kStPrunedMemory, s_stats[2]);
+        if (s_stats[3]) {
+            atomicAdd(p.stats + (complete ? kStParentsComplete : kStParentsExpand), s_stats[3]);
+            atomicAdd(p.stats + kStDepthParents + x, s_stats[3]);
         }
     }
 }

@@ -53,17 +53,19 @@ struct Vec32 {
     uint4 a, b;
 };
 
+// one 32-byte load or store: a whole sector per lane
 __device__ __forceinline__ Vec32 load32(const void *ptr) {
-    const uint4 *q = static_cast<const uint4 *>(ptr);
     Vec32 v;
-    v.a = __ldg(q);
-    v.b = __ldg(q + 1);
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v.a.x), "=r"(v.a.y), "=r"(v.a.z), "=r"(v.a.w), "=r"(v.b.x), "=r"(v.b.y),
+                   "=r"(v.b.z), "=r"(v.b.w)
+                 : "l"(ptr));
     return v;
 }
 __device__ __forceinline__ void store32(void *ptr, const Vec32 &v) {
-    uint4 *q = static_cast<uint4 *>(ptr);
-    q[0] = v.a;
-    q[1] = v.b;
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(ptr), "r"(v.a.x),
+                 "r"(v.a.y), "r"(v.a.z), "r"(v.a.w), "r"(v.b.x), "r"(v.b.y), "r"(v.b.z), "r"(v.b.w)
+                 : "memory");
 }
 __device__ __forceinline__ uint32_t &word_of(Vec32 &v, int w) {
     return w == 0 ? v.a.x : w == 1 ? v.a.y : w == 2 ? v.a.z : w == 3 ? v.a.w
@@ -109,6 +111,24 @@ __device__ __forceinline__ bool key_less(unsigned long long ao, unsigned long lo
                                          unsigned long long bo, unsigned long long bi) {
     return ao < bo || (ao == bo && ai < bi);
 }
+
+// Largest makespan T of a slice with T * scale <= thr (thr = ~0: no
+// incumbent).  Makespans are below 2^31.  A lane keeps the last scale's answer:
+// neighbouring entries nearly always share it, and a 64-bit division costs as
+// much as a quarter of a prefix's expansion.
+struct TopMakespan {
+    uint64_t thr, scale;
+    int32_t top;
+    __device__ __forceinline__ explicit TopMakespan(uint64_t t) : thr(t), scale(0), top(0) {}
+    __device__ __forceinline__ int32_t of(uint64_t s) {
+        if (s != scale) {
+            scale = s;
+            const uint64_t q = thr / s;
+            top = q > 0x7fffffffull ? 0x7fffffff : (int32_t)q;
+        }
+        return top;
+    }
+};
 
 // Lower the incumbent to (obj, idx) if that is smaller.  Bounded loop: every
 // failed CAS means another thread lowered the key; after `limit` rounds
@@ -171,6 +191,8 @@ template <int S, int PATH>
 __global__ void __launch_bounds__(256, leaf_min_blocks(S, PATH)) leaf_kernel(LeafParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint64_t bar;
+    __shared__ unsigned long long s_evaluated;
+    if (threadIdx.x == 0) s_evaluated = 0;
     // the tables were written before the previous kernel: staged while it
     // finishes; the plans and their count only after it has completed
     if (!stage_blob_bulk(sm, p.blob, p.lay.bytes, &bar)) {
@@ -253,8 +275,16 @@ __global__ void __launch_bounds__(256, leaf_min_blocks(S, PATH)) leaf_kernel(Lea
         }
         if ((threadIdx.x & 31) == 0 && obj != ~0ull) incumbent_update(p.inc, obj, idx, p.stats, p.cas_limit);
     }
+    // one atomic per block and counter (per warp when few warps had plans):
+    // they all go to the same addresses
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) evaluated += __shfl_xor_sync(0xffffffffu, evaluated, o);
+    const bool few = n <= 16384;
+    if (!few) {
+        if ((threadIdx.x & 31) == 0 && evaluated) atomicAdd(&s_evaluated, evaluated);
+        __syncthreads();
+        evaluated = threadIdx.x == 0 ? s_evaluated : 0;
+    }
     if ((threadIdx.x & 31) == 0 && evaluated) {
         atomicAdd(p.stats + kStEvaluated, evaluated);
         atomicAdd(p.stats + kStRelaxations, evaluated * 2ull * S * (unsigned long long)p.M);
