@@ -296,23 +296,98 @@ __device__ __forceinline__ bool dispatch_range(int S, const Tab &t, const uint4 
     return true;
 }
 
+// A warp's walk over the sorted positions [begin, end), 32 at a time.
+//
+// Most plans need a few steady steps and some need nearly all (makespan_fast),
+// so a warp that ran each of its 32 plans to the end would run as long as the
+// slowest.  A plan whose bounds still differ at their first comparison is put
+// on a queue of its warp instead (later), and 32 of those are run to their end
+// together.  A warp with at most two groups of 32 plans has too few to fill
+// such a group and runs every plan to its end at once.
+//
+// With a queue a warp walks one stretch of the range, or, with many groups,
+// two that lie as far from its middle as one another: the plans of a stretch
+// have one stage count and nearly one micro-batch count, so the queue's groups
+// do too, and the cost of a plan grows over the range, so two stretches
+// balance.  Blocks sms apart usually run on one SM and are neighbours in the
+// range, so that an SM's warps run the code of one stage count at a time
+// (16 million plans of 13..16 stages: 822 us with the blocks in launch order,
+// issue slots 39 % busy for want of instructions; 449 us, 62 %).
+struct GroupWalk {
+    uint32_t begin, end, g, g_end, step, second;  // second: group of the other stretch
+    uint32_t *queue;                              // 64 entries
+    int queued;
+    bool use_queue;
+    __device__ __forceinline__ GroupWalk(uint32_t b, uint32_t e, int sm_count, uint32_t *q)
+        : begin(b), end(e), queue(q), queued(0) {
+        constexpr uint32_t kWarps = kEvalThreads / 32;
+        const uint32_t sms = (uint32_t)sm_count;
+        const uint32_t block = gridDim.x % sms == 0
+                                   ? (blockIdx.x % sms) * (gridDim.x / sms) + blockIdx.x / sms
+                                   : blockIdx.x;
+        const uint32_t warps = gridDim.x * kWarps, warp = block * kWarps + (threadIdx.x >> 5);
+        const uint32_t groups = (end - begin + 31) / 32;
+        use_queue = groups > 2 * warps;
+        second = 0xffffffffu;
+        if (!use_queue) {  // every warps-th group
+            g = warp;
+            g_end = groups;
+            step = warps;
+        } else {
+            const uint32_t n = groups > 32 * warps ? 2 : 1;  // stretches
+            const uint32_t len = (groups + n * warps - 1) / (n * warps);
+            g = warp * len;
+            g_end = min(groups, g + len);
+            step = 1;
+            if (n == 2) second = (2 * warps - 1 - warp) * len;
+            span = len;
+            total = groups;
+        }
+    }
+    // The next 32 positions (whole warp): j and whether the lane has one;
+    // to_end: run the plans to their end; again: they come from the queue.
+    __device__ __forceinline__ bool next(uint32_t &j, bool &active, bool &to_end, bool &again) {
+        const int lane = threadIdx.x & 31;
+        if (g >= g_end && second != 0xffffffffu) {
+            g = second;
+            g_end = min(total, g + span);
+            second = 0xffffffffu;
+        }
+        again = queued >= 32 || (queued > 0 && g >= g_end);
+        to_end = again || !use_queue;
+        if (again) {
+            const int n = min(queued, 32);
+            queued -= n;
+            active = lane < n;
+            j = active ? queue[queued + lane] : 0u;
+            __syncwarp();  // read before later entries take their place
+            return true;
+        }
+        if (g >= g_end) return false;
+        j = begin + 32 * g + lane;
+        active = j < end;
+        g += step;
+        return true;
+    }
+    __device__ __forceinline__ void later(uint32_t j, bool put) {
+        const unsigned m = __ballot_sync(0xffffffffu, put);
+        if (put) queue[queued + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = j;
+        queued += __popc(m);
+        __syncwarp();
+    }
+
+private:
+    uint32_t span, total;
+};
+
 // Evaluates the sorted positions [offs[key_lo], offs[key_hi]): all
 // candidates with S in [SLO, SHI] on path PATH.
-//
-// Most plans need a few steady steps and some need nearly all (makespan_fast), so a warp that ran each of its 32 plans to the end
-// would run as long as the slowest.  A plan whose bounds still differ at
-// their first comparison is put on a queue of its warp instead, and 32 of
-// those are run to their end together.  A warp with at most two groups of
-// 32 plans has too few to fill such a group and runs every plan to its end
-// at once.
 template <int SLO, int SHI, int PATH, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
-    constexpr int kWarps = kEvalThreads / 32;
-    __shared__ uint32_t s_queue[kWarps][64];
-    const int key_lo = fast_key_begin(SLO), key_hi = fast_key_begin(SHI + 1);
+    __shared__ uint32_t s_queue[kEvalThreads / 32][64];
     // the key offsets come from the sort's scan, two or more kernels back
-    const uint32_t begin = p.offs[key_lo], end = p.offs[key_hi];
+    const uint32_t begin = p.offs[fast_key_begin(SLO)], end = p.offs[fast_key_begin(SHI + 1)];
     // blocks with no candidate (all of them when the range is empty) leave
     // without staging the tables, after the decode pass has completed
     if (end == begin) {
@@ -324,50 +399,10 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) 
     grid_dep_wait();  // the decoded records
     grid_dep_trigger();
     const Tab t = tab_at(sm, p.tlay);
-    const int lane = threadIdx.x & 31;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    uint32_t *queue = s_queue[threadIdx.x >> 5];
-    // blocks sms apart usually run on one SM: neighbours in the range, so
-    // that an SM's warps run the code of one stage count at a time
-    const uint32_t sms = (uint32_t)p.sms;
-    const uint32_t block = gridDim.x % sms == 0
-                               ? (blockIdx.x % sms) * (gridDim.x / sms) + blockIdx.x / sms
-                               : blockIdx.x;
-    const uint32_t warps = gridDim.x * kWarps, warp = block * kWarps + (threadIdx.x >> 5);
-    const uint32_t groups = (end - begin + 31) / 32;
-    const bool use_queue = groups > 2 * warps;
-    // The warp's groups of 32: every warps-th one, or, with a queue, two
-    // stretches (of half a warp's share each) as far from the range's middle
-    // as one another.  The plans of a stretch have one stage count and nearly
-    // one micro-batch count, so the queue's groups do too, and the cost of a
-    // plan grows over the range, so the two stretches balance.
-    const uint32_t half = use_queue ? (groups + 2 * warps - 1) / (2 * warps) : 0;
-    uint32_t g = use_queue ? warp * half : warp;
-    uint32_t g_end = use_queue ? min(groups, g + half) : groups;
-    bool second = !use_queue;  // no further stretch
-    int queued = 0;
-    // whole warps iterate together (ballots below)
-    for (;;) {
-        if (g >= g_end && !second) {
-            second = true;
-            g = (2 * warps - 1 - warp) * half;
-            g_end = min(groups, g + half);
-        }
-        const bool from_queue = queued >= 32 || (queued > 0 && g >= g_end);
-        uint32_t j;
-        bool active;
-        if (from_queue) {
-            const int n = min(queued, 32);
-            queued -= n;
-            active = lane < n;
-            j = active ? queue[queued + lane] : 0u;
-            __syncwarp();  // read before later entries take their place
-        } else {
-            if (g >= g_end) break;
-            j = begin + 32 * g + lane;
-            active = j < end;
-            g += use_queue ? 1 : warps;
-        }
+    GroupWalk walk(begin, end, p.sms, s_queue[threadIdx.x >> 5]);
+    uint32_t j;
+    bool active, to_end, again;
+    while (walk.next(j, active, to_end, again)) {
         uint32_t i = 0;
         uint4 rec = make_uint4(0, 0, 0, 0), packed = make_uint4(0, 0, 0, 0);
         if (active) {
@@ -378,7 +413,6 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) 
             rec = make_uint4(meta.w, 0u, meta.y, meta.z);
         }
         const int S = active ? (int)(rec.w & 0xff) : 0;
-        const bool to_end = from_queue || !use_queue;
         int32_t T = -1;
         bool done = true;
         unsigned pending = __ballot_sync(0xffffffffu, active);
@@ -391,10 +425,7 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) 
             pending &= ~grp;
         }
         if (active && done) p.T[i] = T;
-        const unsigned later = __ballot_sync(0xffffffffu, !done);
-        if (!done) queue[queued + __popc(later & lt_mask)] = j;
-        queued += __popc(later);
-        __syncwarp();
+        walk.later(j, !done);
     }
 }
 

@@ -310,11 +310,12 @@ pos_status eval_il_23_29(const EvalParams &p, cudaStream_t s);
 pos_status eval_il_30_31(const EvalParams &p, cudaStream_t s);
 pos_status eval_il_32_33(const EvalParams &p, cudaStream_t s);
 
-inline pos_status eval_interleaved(const EvalParams &p, cudaStream_t s) {
-    POS_TRY(eval_il_0_11(p, s));
-    POS_TRY(eval_il_12_22(p, s));
-    POS_TRY(eval_il_23_29(p, s));
-    POS_TRY(eval_il_30_31(p, s));
+// the range of one pair
+inline pos_status eval_interleaved(int pair, const EvalParams &p, cudaStream_t s) {
+    if (pair <= 11) return eval_il_0_11(p, s);
+    if (pair <= 22) return eval_il_12_22(p, s);
+    if (pair <= 29) return eval_il_23_29(p, s);
+    if (pair <= 31) return eval_il_30_31(p, s);
     return eval_il_32_33(p, s);
 }
 

@@ -664,11 +664,15 @@ __global__ void __launch_bounds__(32 * kSeedWarps) il_seed_kernel(
 // ---------------------------------------------------------------------------
 namespace {
 
+// Index and first key of the pair (N, V); -1 when there is none.
 template <int P = 0>
-int il_pair_key(int N, int V) {
+int il_pair(int N, int V, int *key) {
     if constexpr (P < kIlPairs) {
-        if (IlPair<P>::N == N && IlPair<P>::V == V) return IlPair<P>::key;
-        return il_pair_key<P + 1>(N, V);
+        if (IlPair<P>::N == N && IlPair<P>::V == V) {
+            *key = IlPair<P>::key;
+            return P;
+        }
+        return il_pair<P + 1>(N, V, key);
     } else {
         return -1;
     }
@@ -680,7 +684,7 @@ struct IlRun {
     cudaStream_t st;
     BlobLayout lay{};
     void *blob = nullptr;
-    int N = 0, V = 0, J = 0, L = 0, n_tp = 0, pair_key = 0;
+    int N = 0, V = 0, J = 0, L = 0, n_tp = 0, pair = 0, pair_key = 0;
     long long cap = 0;
     uint64_t n_map = 0;
     int grid_level = 0, grid_consider = 0;
@@ -716,7 +720,8 @@ pos_status il_leaves(IlRun &r, const unsigned long long *count) {
     ep.cuts = static_cast<uint4 *>(r.ws.il_rec.p);
     set_tables(ep, r.blob, r.lay);
     ep.nkeys = kKeysIl;
-    POS_TRY(eval_interleaved(ep, r.st));
+    ep.sms = sm_count();
+    POS_TRY(eval_interleaved(r.pair, ep, r.st));
     POS_TRY(ensure_smem(reinterpret_cast<const void *>(il_consider_kernel), r.lay.bytes));
     const int cas = r.p->cas_limit == 0 ? kCasLimit : std::max(0, r.p->cas_limit);
     il_consider_kernel<<<r.grid_consider, kIlThreads, r.lay.bytes, r.st>>>(
@@ -725,7 +730,7 @@ pos_status il_leaves(IlRun &r, const unsigned long long *count) {
         (unsigned long long)r.cap, r.d_slices, r.n_map, r.J, static_cast<Key128 *>(r.ws.d_inc.p),
         r.stats, cas, r.blob, r.lay);
     POS_CUDA(cudaGetLastError());
-    r.launches += 7;  // offsets, five makespan ranges, incumbent
+    r.launches += 3;  // offsets, makespans, incumbent
     r.n_leaf++;
     return POS_OK;
 }
@@ -853,8 +858,8 @@ pos_status search_interleaved(Workspace &ws, const pos_problem *p, const SliceSp
     r.L = p->tables.L;
     r.n_tp = p->tables.n_tp;
     if (r.J > r.L) return fail(POS_EINVAL, "S*V > L: a virtual stage would hold no layer");
-    r.pair_key = il_pair_key(r.N, r.V);
-    if (r.pair_key < 0) return fail(POS_EINVAL, "Interleaved 1F1B needs V >= 2 and S*V <= 16");
+    r.pair = il_pair(r.N, r.V, &r.pair_key);
+    if (r.pair < 0) return fail(POS_EINVAL, "Interleaved 1F1B needs V >= 2 and S*V <= 16");
     r.n_map = host_binom(r.L - 1, r.J - 1);
     const int N = r.N;  // the slices (sp) are over the N devices
     // tables: raw rows uploaded, prefix sums built on the device
