@@ -996,18 +996,26 @@ __device__ __forceinline__ void eager_steady_step(int32_t (&Fo)[S], int32_t (&Fp
     (eager_steady_op_growth<S, 1, GROWTH, i>(Fo, Fp, Bo, w, grow), ...);
 }
 
+// Stage counts whose Eager plans use the bounds.  Their tail costs about 6.5 S^2
+// instructions (the ramp-down is 4S - 3 levels), more than the steady steps
+// that it saves from 14 stages on (16 million plans of 14..16 stages on a GB300:
+// 585 us with the bounds, 517 us without).
+__host__ __device__ constexpr bool eager_bounds(int S) { return S <= 13; }
+
 // Eager 1F1B, M >= 2S-1
 template <int S, class Limit>
 __device__ __forceinline__ bool makespan_eager(const StageW<S> &w, int M, bool to_end,
                                                const Limit &limit, int32_t &T) {
     EagerTail<S> r;
+    if constexpr (eager_bounds(S)) {
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-        r.F[s] = 0;
-        r.P[s] = 0;
-        r.B[s] = w.d[s];
+        for (int s = 0; s < S; ++s) {
+            r.F[s] = 0;
+            r.P[s] = 0;
+            r.B[s] = w.d[s];
+        }
+        eager_tail_ramp<S>(r, w, std::make_integer_sequence<int, 4 * S - 3>{});
     }
-    eager_tail_ramp<S>(r, w, std::make_integer_sequence<int, 4 * S - 3>{});
     // every stage's 2(S-s)+1 warm-up forwards by the closed form of
     // makespan_fast (they precede its backwards in the chain and depend on
     // forwards of earlier stages' warm-ups only), then the ramp-up's other ops
@@ -1024,7 +1032,17 @@ __device__ __forceinline__ bool makespan_eager(const StageW<S> &w, int M, bool t
     }
     eager_ramp<S, true, 1>(Fo, Fp, Bo, w, std::make_integer_sequence<int, 2 * S - 1>{});
     int left = M - 2 * S + 1, steps = Limit::kOn ? 1 : kFirstStepsEager;
-    for (;;) {
+    if constexpr (!eager_bounds(S)) {
+        int32_t grow = 0;
+#pragma unroll 1
+        for (; left > 0; --left)
+            eager_steady_step<S, false>(Fo, Fp, Bo, w, grow, std::make_integer_sequence<int, S>{});
+        eager_ramp<S, false, -2 * S + 2>(Fo, Fp, Bo, w, std::make_integer_sequence<int, 4 * S - 3>{});
+        T = 0;
+#pragma unroll
+        for (int s = 0; s < S; ++s) T = max(T, Bo[s] + w.d[s]);
+        return true;
+    } else for (;;) {
         const int n = min(steps, left);
         left -= n;
         int32_t grow = 0;

@@ -512,11 +512,14 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
         void *scratch = nullptr;
         const int nk = il ? kKeysIl : kKeys;
         // scratch: decoded records (32 B per candidate), the sort arrays, the keys
-        const size_t sbytes = 32 * (size_t)m + sizeof(uint32_t) * (3 * (size_t)nk + 1 + (size_t)m) +
+        constexpr int kTiles = POS_MAX_STAGES + 1;
+        const size_t sbytes = 32 * (size_t)m +
+                              sizeof(uint32_t) * (kTiles + 3 * (size_t)nk + 1 + (size_t)m) +
                               sizeof(uint16_t) * (size_t)m;
         POS_CUDA(cudaMallocFromPoolAsync(&scratch, sbytes, pool, stream));
         uint4 *cuts = static_cast<uint4 *>(scratch);
-        uint32_t *hist = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + 32 * (size_t)m);
+        uint32_t *tiles = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + 32 * (size_t)m);
+        uint32_t *hist = tiles + kTiles;
         uint32_t *offs = hist + nk;
         uint32_t *cursor = offs + nk + 1;
         uint32_t *dest = cursor + nk;
@@ -525,11 +528,12 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
         p.dest = dest;
         p.offs = offs;
         p.cuts = cuts;
+        p.tiles = tiles;
         p.nkeys = nk;
         // histogram pass: 256 threads, four candidates per thread and round
         const int grid = (int)std::max<int64_t>(
             1, std::min<int64_t>((m + 1023) / 1024, 4LL * sm_count()));
-        cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(uint32_t) * nk, stream);
+        cudaError_t e = cudaMemsetAsync(tiles, 0, sizeof(uint32_t) * (kTiles + nk), stream);
         if (e == cudaSuccess) {
             const int64_t chunk = scatter_chunk(m, sm_count());
             const int sgrid = (int)std::max<int64_t>(

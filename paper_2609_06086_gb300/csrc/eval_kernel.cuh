@@ -63,6 +63,8 @@ struct EvalParams {
     // grows with M since every cost is non-negative
     uint16_t guard_m[POS_MAX_STAGES + 1];
     int sms;               // SMs of the device
+    uint32_t *tiles;       // [17] next tile of the range that starts at stage count
+                           // S (GroupWalk), zero at the start
     int nkeys;             // kKeys, or kKeysIl under Interleaved 1F1B
     int per_stage_tp;      // 1: records carry a TP index per stage (n_tp <= 4)
     // the handle's memory-limit table (Handle::lim_*): the decode pass stages
@@ -305,68 +307,76 @@ __device__ __forceinline__ bool dispatch_range(int S, const Tab &t, const uint4 
 // together.  A warp with at most two groups of 32 plans has too few to fill
 // such a group and runs every plan to its end at once.
 //
-// With a queue a warp walks one stretch of the range, or, with many groups,
-// two that lie as far from its middle as one another: the plans of a stretch
-// have one stage count and nearly one micro-batch count, so the queue's groups
-// do too, and the cost of a plan grows over the range, so two stretches
-// balance.  Blocks sms apart usually run on one SM and are neighbours in the
-// range, so that an SM's warps run the code of one stage count at a time
-// (16 million plans of 13..16 stages: 822 us with the blocks in launch order,
-// issue slots 39 % busy for want of instructions; 449 us, 62 %).
+// With a queue and many groups per warp (more than 32) the warps take tiles of
+// eight neighbouring groups from a counter, from the range's end down: the most
+// expensive plans first, so the warps finish together, and all warps at the
+// same part of the range, so that the plans of a queue and the code that an SM
+// runs have nearly one stage count at a time.  With fewer a warp walks one
+// stretch of the range, whose plans have one stage count; blocks sms apart
+// usually run on one SM and take neighbouring stretches, again so that an SM's
+// warps run the same code.  (13..16 stages, 16 million 1F1B plans: 822 us with
+// stretches in launch order, issue slots 39 % busy for want of instructions,
+// 449 us with neighbouring ones; the whole sweep of 20 million 2364 -> 2259 us
+// with tiles; 2 million Eager plans 413 us with stretches, 439 us with tiles.)
 struct GroupWalk {
-    uint32_t begin, end, g, g_end, step, second;  // second: group of the other stretch
-    uint32_t *queue;                              // 64 entries
+    static constexpr uint32_t kTile = 8;
+    uint32_t begin, end, g, g_end, tiles, groups, stride;
+    uint32_t *queue, *counter;  // 64 entries; next tile
     int queued;
-    bool use_queue;
-    __device__ __forceinline__ GroupWalk(uint32_t b, uint32_t e, int sm_count, uint32_t *q)
-        : begin(b), end(e), queue(q), queued(0) {
+    bool use_queue, more;
+    __device__ __forceinline__ GroupWalk(uint32_t b, uint32_t e, uint32_t *q, uint32_t *c,
+                                         uint32_t sms)
+        : begin(b), end(e), queue(q), counter(c), queued(0) {
         constexpr uint32_t kWarps = kEvalThreads / 32;
-        const uint32_t sms = (uint32_t)sm_count;
-        const uint32_t block = gridDim.x % sms == 0
-                                   ? (blockIdx.x % sms) * (gridDim.x / sms) + blockIdx.x / sms
-                                   : blockIdx.x;
-        const uint32_t warps = gridDim.x * kWarps, warp = block * kWarps + (threadIdx.x >> 5);
-        const uint32_t groups = (end - begin + 31) / 32;
-        use_queue = groups > 2 * warps;
-        second = 0xffffffffu;
-        if (!use_queue) {  // every warps-th group
-            g = warp;
-            g_end = groups;
-            step = warps;
-        } else {
-            const uint32_t n = groups > 32 * warps ? 2 : 1;  // stretches
-            const uint32_t len = (groups + n * warps - 1) / (n * warps);
-            g = warp * len;
+        stride = gridDim.x * kWarps;
+        groups = (end - begin + 31) / 32;
+        use_queue = groups > 2 * stride;
+        more = groups > 32 * stride;  // tiles
+        tiles = (groups + kTile - 1) / kTile;
+        if (more) {
+            g = g_end = 0;
+        } else if (use_queue) {
+            const uint32_t block = gridDim.x % sms == 0
+                                       ? (blockIdx.x % sms) * (gridDim.x / sms) + blockIdx.x / sms
+                                       : blockIdx.x;
+            const uint32_t len = (groups + stride - 1) / stride;
+            g = (block * kWarps + (threadIdx.x >> 5)) * len;
             g_end = min(groups, g + len);
-            step = 1;
-            if (n == 2) second = (2 * warps - 1 - warp) * len;
-            span = len;
-            total = groups;
+        } else {  // every stride-th group
+            g = blockIdx.x * kWarps + (threadIdx.x >> 5);
+            g_end = groups;
         }
     }
     // The next 32 positions (whole warp): j and whether the lane has one;
-    // to_end: run the plans to their end; again: they come from the queue.
-    __device__ __forceinline__ bool next(uint32_t &j, bool &active, bool &to_end, bool &again) {
+    // to_end: run the plans to their end.
+    __device__ __forceinline__ bool next(uint32_t &j, bool &active, bool &to_end) {
         const int lane = threadIdx.x & 31;
-        if (g >= g_end && second != 0xffffffffu) {
-            g = second;
-            g_end = min(total, g + span);
-            second = 0xffffffffu;
+        if (g >= g_end && more && queued < 32) {
+            uint32_t t = 0;
+            if (lane == 0) t = atomicAdd(counter, 1u);
+            t = __shfl_sync(0xffffffffu, t, 0);
+            more = t < tiles;
+            if (more) {
+                g = (tiles - 1 - t) * kTile;
+                g_end = min(groups, g + kTile);
+            }
         }
-        again = queued >= 32 || (queued > 0 && g >= g_end);
+        const bool again = queued >= 32 || (queued > 0 && g >= g_end);
         to_end = again || !use_queue;
         if (again) {
-            const int n = min(queued, 32);
-            queued -= n;
-            active = lane < n;
-            j = active ? queue[queued + lane] : 0u;
-            __syncwarp();  // read before later entries take their place
+            active = lane < queued;
+            j = active ? queue[lane] : 0u;
+            const uint32_t rest = queue[32 + lane];
+            __syncwarp();
+            queue[lane] = rest;  // the oldest entries leave first
+            __syncwarp();
+            queued = max(queued - 32, 0);
             return true;
         }
         if (g >= g_end) return false;
         j = begin + 32 * g + lane;
         active = j < end;
-        g += step;
+        g += use_queue ? 1 : stride;
         return true;
     }
     __device__ __forceinline__ void later(uint32_t j, bool put) {
@@ -375,9 +385,6 @@ struct GroupWalk {
         queued += __popc(m);
         __syncwarp();
     }
-
-private:
-    uint32_t span, total;
 };
 
 // Evaluates the sorted positions [offs[key_lo], offs[key_hi]): all
@@ -399,10 +406,11 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) 
     grid_dep_wait();  // the decoded records
     grid_dep_trigger();
     const Tab t = tab_at(sm, p.tlay);
-    GroupWalk walk(begin, end, p.sms, s_queue[threadIdx.x >> 5]);
+    GroupWalk walk(begin, end, s_queue[threadIdx.x >> 5], p.tiles + SLO,
+                   (uint32_t)p.sms);
     uint32_t j;
-    bool active, to_end, again;
-    while (walk.next(j, active, to_end, again)) {
+    bool active, to_end;
+    while (walk.next(j, active, to_end)) {
         uint32_t i = 0;
         uint4 rec = make_uint4(0, 0, 0, 0), packed = make_uint4(0, 0, 0, 0);
         if (active) {
