@@ -182,8 +182,8 @@ pos_status poseidon_tables_destroy(void *handle);
  * operation, so every effect is still ordered after earlier work on
  * `stream` and before later work on it.  Infeasible
  * plans still get their makespan.  Scratch: the batch is counting-sorted by
- * (S, M) (and by (N, V, M/N) for interleaved records) and decoded into a
- * 38*n + 56 KB (Interleaved 1F1B: 38*n + 121 KB) stream-ordered allocation
+ * S and M (and by (N, V, M/N) for interleaved records) and decoded into a
+ * 38*n + 13 KB (Interleaved 1F1B: 38*n + 78 KB) stream-ordered allocation
  * (decoded record 32 B, sorted position 4 B and sort key 2 B per candidate,
  * key histograms) from a library-owned memory pool (per device, kept
  * between calls); batches above 2^24 candidates go in chunks of 2^24, one

@@ -16,10 +16,11 @@
 // staging the cost tables.
 //
 // Sort keys: fast path (M >= S for 1F1B, M >= 2S-1 for Eager 1F1B) ->
-// (S-1)*256 + M (the other slots of each S stay empty); short path ->
-// 4096 + M*16 + S-1; Interleaved 1F1B records with V >= 2 get keys after
-// those (interleaved.cuh); records with S outside 1..16 or M = 0 are flagged
-// invalid by the sort pass and get no key.
+// (S-1)*32 + M/8 (a warp's plans end after about the same steps whatever M is,
+// see makespan_fast, so neighbouring M share a key); short path -> 512 + M*16 +
+// S-1; Interleaved 1F1B records with V >= 2 get keys after those
+// (interleaved.cuh); records with S outside 1..16 or M = 0 are flagged invalid
+// by the sort pass and get no key.
 #pragma once
 #include <algorithm>
 
@@ -27,11 +28,11 @@
 
 namespace pos {
 
-constexpr int kKeys = 4096 + 16 * 32;  // fast keys, then short-path keys
+constexpr int kKeys = 512 + 32 * 16;  // fast keys, then short-path keys
 constexpr int kEvalThreads = 128;
 
-__host__ __device__ inline int fast_key_begin(int S) { return (S - 1) * 256; }
-__host__ __device__ inline int short_key_begin(int M) { return 4096 + M * 16; }
+__host__ __device__ inline int fast_key_begin(int S) { return (S - 1) * 32; }
+__host__ __device__ inline int short_key_begin(int M) { return 512 + M * 16; }
 
 struct EvalParams {
     const uint4 *cands;    // 16-byte records (poseidon_eval_batch), or
@@ -43,6 +44,7 @@ struct EvalParams {
     const uint32_t *dest;  // sorted position of every candidate (kNoDest:
                            // no key, answered by the histogram pass)
     const uint32_t *offs;  // [nkeys + 1] start of every key in sorted order
+                           // (written by the scatter pass)
     uint4 *cuts;           // per sorted position j, two 16-byte words (read once,
                            // with evict-first loads, so that the outputs'
                            // sectors stay in L2):
@@ -393,7 +395,7 @@ template <int SLO, int SHI, int PATH, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint32_t s_queue[kEvalThreads / 32][64];
-    // the key offsets come from the sort's scan, two or more kernels back
+    // the key offsets come from the scatter pass, two or more kernels back
     const uint32_t begin = p.offs[fast_key_begin(SLO)], end = p.offs[fast_key_begin(SHI + 1)];
     // blocks with no candidate (all of them when the range is empty) leave
     // without staging the tables, after the decode pass has completed
@@ -526,7 +528,7 @@ __device__ __forceinline__ int32_t short_dispatch(int M, const Tab &t, const uin
 template <bool EAGER, int MLO, int MHI, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) short_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
-    // the key offsets come from the sort's scan, two or more kernels back
+    // the key offsets come from the scatter pass, two or more kernels back
     const uint32_t begin = p.offs[short_key_begin(MLO)], end = p.offs[short_key_begin(MHI + 1)];
     if (blockIdx.x * blockDim.x >= end - begin) {
         grid_dep_wait();
