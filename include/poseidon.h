@@ -177,7 +177,7 @@ pos_status poseidon_tables_destroy(void *handle);
  * d_feasible (uint8[n]) are DEVICE pointers on the handle's device; outputs
  * are in input order; the call is asynchronous on `stream` (a cudaStream_t,
  * NULL = legacy default stream) and returns after the launches.  Part of the
- * work runs on a library-owned second stream of the device, forked from
+ * work runs on library-owned side streams of the device, forked from
  * `stream` after the sort and joined back into it before the call's last
  * operation, so every effect is still ordered after earlier work on
  * `stream` and before later work on it.  Infeasible

@@ -1,6 +1,7 @@
 // poseidon_eval_batch, poseidon_eval_batch_host and poseidon_argmin (hot-path
 // step a9).  The evaluation kernels live in eval_kernel.cuh and the
 // eval_range_*.cu instantiation units.
+#include <iterator>
 #include <mutex>
 #include <utility>
 
@@ -446,20 +447,22 @@ static pos_status scratch_pool(cudaMemPool_t *out) {
     return POS_OK;
 }
 
-// A second stream per device for the short-path kernels (M < S under 1F1B,
-// M < 2S-1 under Eager 1F1B) and then the smallest fast-path range (under
-// Interleaved 1F1B: every 1F1B range, then the smallest interleaved range):
-// every evaluation kernel depends only on the decode pass, and the short
-// paths are bound by instruction fetch rather than by the ALU, so they run
-// beside the other fast-path kernels instead of after them (measured: the
-// side chain with the smallest fast range was faster than the short paths
-// alone, two chains splitting the fast ranges slower).  The
-// fork and join events are shared per device, so a call holds the device's
-// side mutex from the fork to the join (two calls from different host
-// threads must not interleave their record / wait pairs).
+// Side streams per device.  Every makespan kernel depends only on the decode
+// pass, so the ranges of a batch run on the caller's stream and on these: none
+// keeps every issue slot busy (small batches: the latency of a range's slowest
+// warps; large ones: the kernels' ends, and instruction fetch), the longest on
+// the caller's stream.  One side stream / three on a GB300: 1F1B 93 / 73 us at
+// 250,007 plans, 910 / 882 us at 8 million; Eager 245 / 205 us at a million;
+// Interleaved 297 / 258 us at a million, but 1748 / 1870 us at 8 million, where
+// its large kernels evict one another's code.  The fork and join events are
+// shared per device, so a call holds the device's side mutex from the fork to
+// the join (two calls from different host threads must not interleave their
+// record / wait pairs).
+constexpr int kSides = 3;
+constexpr int64_t kSpreadMaxIl = 1 << 22;  // interleaved batches on all streams
 struct SideStream {
-    cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaStream_t s[kSides] = {};
+    cudaEvent_t fork = nullptr, join[kSides] = {};
     std::mutex mu;
 };
 static std::mutex g_side_mutex;
@@ -471,12 +474,71 @@ static pos_status side_stream(SideStream **out) {
     if (dev < 0 || dev >= 64) return fail(POS_EINVAL, "device index above 63");
     std::lock_guard<std::mutex> lock(g_side_mutex);
     SideStream &ss = g_side[dev];
-    if (!ss.s) {
-        POS_CUDA(cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming));
-        POS_CUDA(cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming));
-        POS_CUDA(cudaStreamCreateWithFlags(&ss.s, cudaStreamNonBlocking));
+    if (!ss.fork) POS_CUDA(cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming));
+    for (int i = 0; i < kSides; ++i) {
+        if (!ss.join[i]) POS_CUDA(cudaEventCreateWithFlags(&ss.join[i], cudaEventDisableTiming));
+        if (!ss.s[i]) POS_CUDA(cudaStreamCreateWithFlags(&ss.s[i], cudaStreamNonBlocking));
     }
     *out = &ss;
+    return POS_OK;
+}
+
+// A makespan kernel and its stream: 0 the caller's, 1.. a side stream.
+struct RangeLaunch {
+    pos_status (*launch)(const EvalParams &, cudaStream_t);
+    int at;
+};
+static const RangeLaunch kRanges1F1B[] = {
+    {eval_short_1_9, 1}, {eval_short_10_15, 1}, {eval_fast_13_16, 0},
+    {eval_fast_9_12, 2}, {eval_fast_5_8, 3},    {eval_fast_1_4, 3}};
+static const RangeLaunch kRangesEager[] = {
+    {eval_eager_short_23_30, 1}, {eval_eager_short_15_22, 1}, {eval_eager_short_1_14, 1},
+    {eval_eager_14_16, 0},       {eval_eager_11_13, 2},       {eval_eager_7_10, 3},
+    {eval_eager_1_6, 2}};
+// interleaved handle: the 1F1B ranges hold its records with V < 2, usually none
+static const RangeLaunch kRangesIl[] = {
+    {eval_il_12_22, 0},   {eval_il_23_29, 2},    {eval_il_32_33, 3}, {eval_il_0_11, 3},
+    {eval_short_1_9, 1},  {eval_short_10_15, 1}, {eval_fast_1_4, 1}, {eval_fast_5_8, 1},
+    {eval_fast_9_12, 1},  {eval_fast_13_16, 1},  {eval_il_30_31, 2}};
+static const RangeLaunch kRangesIlLarge[] = {
+    {eval_short_1_9, 1},  {eval_short_10_15, 1}, {eval_fast_1_4, 1}, {eval_fast_5_8, 1},
+    {eval_fast_9_12, 1},  {eval_fast_13_16, 1},  {eval_il_30_31, 1}, {eval_il_0_11, 0},
+    {eval_il_12_22, 0},   {eval_il_23_29, 0},    {eval_il_32_33, 0}};
+
+static pos_status launch_ranges(const EvalParams &p, cudaStream_t stream) {
+    const RangeLaunch *r = kRanges1F1B;
+    int n = (int)std::size(kRanges1F1B), sides = kSides;
+    if (p.lay.sched == POS_SCHED_EAGER_1F1B) {
+        r = kRangesEager;
+        n = (int)std::size(kRangesEager);
+    } else if (p.lay.sched == POS_SCHED_INTERLEAVED_1F1B) {
+        const bool large = p.n > kSpreadMaxIl;
+        r = large ? kRangesIlLarge : kRangesIl;
+        n = (int)std::size(kRangesIl);
+        if (large) sides = 1;
+    }
+    SideStream *ss = nullptr;
+    POS_TRY(side_stream(&ss));
+    std::lock_guard<std::mutex> lock(ss->mu);
+    // fork: the side streams start after the decode pass
+    POS_CUDA(cudaEventRecord(ss->fork, stream));
+    pos_status st = POS_OK;
+    cudaError_t e = cudaSuccess;
+    int forked = 0;
+    for (; forked < sides && e == cudaSuccess; ++forked)
+        e = cudaStreamWaitEvent(ss->s[forked], ss->fork, 0);
+    for (int i = 0; i < n && e == cudaSuccess && st == POS_OK; ++i) {
+        st = r[i].launch(p, r[i].at == 0 ? stream : ss->s[r[i].at - 1]);
+    }
+    // join, also after a failed launch (the side streams' queued work stays
+    // ordered before the scratch is freed)
+    for (int i = 0; i < forked; ++i) {
+        cudaError_t ej = cudaEventRecord(ss->join[i], ss->s[i]);
+        if (ej == cudaSuccess) ej = cudaStreamWaitEvent(stream, ss->join[i], 0);
+        if (e == cudaSuccess) e = ej;
+    }
+    POS_TRY(st);
+    POS_CUDA(e);
     return POS_OK;
 }
 
@@ -552,54 +614,7 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
             st = il ? launch_sort<kKeysIl>(p, m, hist, offs, cursor, dest, keys, stream)
                     : launch_sort<kKeys>(p, m, hist, offs, cursor, dest, keys, stream);
         if (e == cudaSuccess && st == POS_OK) st = launch_decode(p, stream);
-        if (e == cudaSuccess && st == POS_OK) {
-            SideStream *ss = nullptr;
-            st = side_stream(&ss);
-            if (st == POS_OK) {
-                std::lock_guard<std::mutex> lock(ss->mu);
-                // fork: the side chain starts after the decode pass
-                e = cudaEventRecord(ss->fork, stream);
-                if (e == cudaSuccess) e = cudaStreamWaitEvent(ss->s, ss->fork, 0);
-                if (e == cudaSuccess) {
-                    const cudaStream_t side = ss->s;
-                    if (p.lay.sched == POS_SCHED_EAGER_1F1B) {
-                        if ((st = eval_eager_short_1_14(p, side)) == POS_OK &&
-                            (st = eval_eager_short_15_22(p, side)) == POS_OK &&
-                            (st = eval_eager_short_23_30(p, side)) == POS_OK &&
-                            (st = eval_eager_1_6(p, side)) == POS_OK &&
-                            (st = eval_eager_7_10(p, stream)) == POS_OK &&
-                            (st = eval_eager_11_13(p, stream)) == POS_OK)
-                            st = eval_eager_14_16(p, stream);
-                    } else if (il) {
-                        // interleaved handle: the 1F1B ranges (records with
-                        // V < 2, usually none) and the smallest interleaved
-                        // range on the side, the other interleaved ranges here
-                        if ((st = eval_short_1_9(p, side)) == POS_OK &&
-                            (st = eval_short_10_15(p, side)) == POS_OK &&
-                            (st = eval_fast_1_4(p, side)) == POS_OK &&
-                            (st = eval_fast_5_8(p, side)) == POS_OK &&
-                            (st = eval_fast_9_12(p, side)) == POS_OK &&
-                            (st = eval_fast_13_16(p, side)) == POS_OK &&
-                            (st = eval_il_30_31(p, side)) == POS_OK &&
-                            (st = eval_il_0_11(p, stream)) == POS_OK &&
-                            (st = eval_il_12_22(p, stream)) == POS_OK &&
-                            (st = eval_il_23_29(p, stream)) == POS_OK)
-                            st = eval_il_32_33(p, stream);
-                    } else if ((st = eval_short_1_9(p, side)) == POS_OK &&
-                               (st = eval_short_10_15(p, side)) == POS_OK &&
-                               (st = eval_fast_1_4(p, side)) == POS_OK &&
-                               (st = eval_fast_5_8(p, stream)) == POS_OK &&
-                               (st = eval_fast_9_12(p, stream)) == POS_OK) {
-                        st = eval_fast_13_16(p, stream);
-                    }
-                    // join, also after a failed launch (the side stream's
-                    // queued work stays ordered before the scratch is freed)
-                    cudaError_t ej = cudaEventRecord(ss->join, side);
-                    if (ej == cudaSuccess) ej = cudaStreamWaitEvent(stream, ss->join, 0);
-                    if (e == cudaSuccess) e = ej;
-                }
-            }
-        }
+        if (e == cudaSuccess && st == POS_OK) st = launch_ranges(p, stream);
         const cudaError_t e2 = cudaFreeAsync(scratch, stream);
         if (e != cudaSuccess) return cuda_fail(e, "eval sort launch");
         if (st != POS_OK) return st;
