@@ -57,7 +57,7 @@ __device__ __forceinline__ int popc128(const Bits128 &b) {
 // (lim_kernel) is the largest end that class k holds from c with w
 // micro-batches in flight, so a stage costs a byte load per start and a few
 // bit operations (a binary search over the memory sums by a block per slice
-// before: 1262 us for 168,000 slices, 420 of them feasible).  A slice whose
+// before: 1262 us for 168,000 slices, 420 of them feasible, on a GB300).  A slice whose
 // set empties on the way is infeasible and left alone; only the feasible ones
 // write their rows: feas[gid*(S+1) + x], lim[(gid*S + x)*128 + c] = the most
 // layers stage x holds from c (0 if none).  root[gid] = 1 when the slice has a
@@ -90,16 +90,16 @@ __global__ void __launch_bounds__(kFeasThreads) feas_kernel(const SliceRec *slic
         for (int x = S - 1; x >= 0 && some; --x) {
             const uint8_t *most = limits(x);
             Bits128 cur;
+            int after = 128;  // first feasible start of stage x + 1 in words > q
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 3; q >= 0; --q) {
                 const int c = lane + 32 * q;
-                bool ok = false;
-                if (c < L) {
-                    const Bits128 win = range_bits(c + 1, (int)__ldg(most + c));
-                    ok = ((prev.w[0] & win.w[0]) | (prev.w[1] & win.w[1]) | (prev.w[2] & win.w[2]) |
-                          (prev.w[3] & win.w[3])) != 0u;
-                }
+                // the first feasible start of stage x + 1 behind c
+                const uint32_t m = prev.w[q] & ~((2u << lane) - 1u);
+                const int next = m ? 32 * q + __ffs(m) - 1 : after;
+                const bool ok = c < L && next <= (int)__ldg(most + min(c, L));
                 cur.w[q] = __ballot_sync(0xffffffffu, ok);
+                if (prev.w[q]) after = 32 * q + __ffs(prev.w[q]) - 1;
             }
             prev = cur;
             some = (prev.w[0] | prev.w[1] | prev.w[2] | prev.w[3]) != 0u;
@@ -195,27 +195,24 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
             const int k = sr.cls[x];
             const int2 e = x + 1 < S ? p2p(t, k, sr.cls[x + 1]) : make_int2(0, 0);
             const int32_t pf = e.x, pb = e.y;
-            int64_t v1 = INT64_MAX, v2 = INT64_MAX;
+            // (path lengths of feasible plans: below 2^31)
+            int32_t v1 = kNoCompletion, v2 = kNoCompletion;
             int best_l = 0;
             if (c < L) {
                 const int most = lim[((size_t)sr.gid * S + x) * 128 + c];
                 const Sums at = sums(t, k, c);
                 const int l_lo = x == S - 1 ? L - c : 1;
-                const int l_hi = x == S - 1 ? L - c : min(most, L - c - (S - 1 - x));
-                for (int l = l_lo + part; l <= l_hi && l <= most; l += 4) {
+                const int l_hi = min(most, x == S - 1 ? L - c : L - c - (S - 1 - x));
+                for (int l = l_lo + part; l <= l_hi; l += 4) {
                     const int c2 = c + l;
                     const Sums v = sums_from(t, k, at, c2);
-                    const int64_t F = v.f, B = v.b, d = v.d;
-                    const int64_t a = (int64_t)M * (F + B);
-                    int64_t w1, w2;
-                    if (x == S - 1) {
-                        w1 = a + d;
-                        w2 = a;
-                    } else {
+                    const int32_t a = M * (v.f + v.b);
+                    int32_t w1 = a + v.d, w2 = a;
+                    if (x < S - 1) {
                         const int2 n = nxt[c2];
                         if (n.x == kNoCompletion) continue;
-                        w1 = max(a + d, F + pf + n.x);
-                        w2 = max(a, F + pf + B + pb + n.y);
+                        w1 = max(w1, v.f + pf + n.x);
+                        w2 = max(w2, v.f + pf + v.b + pb + n.y);
                     }
                     if (w1 < v1) {  // l increases: the first strict minimum is the smallest l
                         v1 = w1;
@@ -228,8 +225,8 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
             // ties in V1 go to the smallest l
 #pragma unroll
             for (int o = 1; o < 4; o <<= 1) {
-                const int64_t o1 = __shfl_xor_sync(0xffffffffu, v1, o);
-                const int64_t o2 = __shfl_xor_sync(0xffffffffu, v2, o);
+                const int32_t o1 = __shfl_xor_sync(0xffffffffu, v1, o);
+                const int32_t o2 = __shfl_xor_sync(0xffffffffu, v2, o);
                 const int ol = __shfl_xor_sync(0xffffffffu, best_l, o);
                 if (o1 < v1 || (o1 == v1 && ol < best_l)) {
                     v1 = o1;
@@ -239,8 +236,7 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
             }
             __syncthreads();  // every thread has read row x+1
             if (part == 0) {
-                const int2 out = v1 == INT64_MAX ? make_int2(kNoCompletion, kNoCompletion)
-                                                 : make_int2((int32_t)v1, (int32_t)v2);
+                const int2 out = make_int2(v1, v2);
                 nxt[c] = out;
                 arg[x][c] = (uint8_t)best_l;
                 vb[((size_t)x * n_rows + vslot) * 128 + c] = out;
@@ -321,13 +317,23 @@ __device__ __forceinline__ int nth_set(const Bits128 &b, int r) {
 // among the counts l that fit the stage's memory (l <= lim) and leave a
 // memory-feasible suffix (feasibility bit of c + l), i.e. the set bits of
 // one 128-bit window, picked with a popcount and a select.
-__global__ void sample_kernel(const SliceRec *slices, const uint32_t *feasible, int n_feasible,
-                              int n_samples, int S, uint64_t seed, const uint4 *feas,
-                              const uint8_t *lim, Leaf *out, int L) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_samples;
-         i += gridDim.x * blockDim.x) {
-        uint64_t st = seed ^ ((uint64_t)i * 0xD1B54A32D192ED03ull);
-        const uint32_t sl = feasible[splitmix64_next(st) % (uint64_t)n_feasible];
+// The samples of one M index: n_s of them, from n_feasible slices at `first`
+// of the list, to the leaf slots from `out` on.
+struct SampleSeg {
+    uint64_t n_s, seed;  // n_s first: the leaf kernel's count
+    uint32_t first, n_feasible, out, pad;
+};
+__global__ void sample_kernel(const SliceRec *slices, const uint32_t *feasible,
+                              const SampleSeg *segs, int n_segs, int n_samples, int S,
+                              const uint4 *feas, const uint8_t *lim, Leaf *out, int L) {
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < n_samples;
+         g += gridDim.x * blockDim.x) {
+        int q = 0;
+        while (q + 1 < n_segs && (uint32_t)g >= segs[q + 1].out) ++q;
+        const SampleSeg seg = segs[q];
+        const uint32_t i = (uint32_t)g - seg.out;
+        uint64_t st = seg.seed ^ ((uint64_t)i * 0xD1B54A32D192ED03ull);
+        const uint32_t sl = feasible[seg.first + splitmix64_next(st) % (uint64_t)seg.n_feasible];
         const SliceRec &sr = slices[sl];
         const uint32_t gid = sr.gid;
         uint32_t cw[4] = {0u, 0u, 0u, 0u};  // cut[0..15], byte x = cut[x]
@@ -347,7 +353,7 @@ __global__ void sample_kernel(const SliceRec *slices, const uint32_t *feasible, 
         }
         // leaf: slice in bytes 0-3, cut[x] in byte 4 + x
         const Vec32 lf = {make_uint4(sl, cw[0], cw[1], cw[2]), make_uint4(cw[3], 0u, 0u, 0u)};
-        store32(out + i, lf);
+        store32(out + g, lf);
     }
 }
 
@@ -1400,7 +1406,7 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
             return fail(POS_EOVERFLOW, "makespan bound reaches 2^31 for some M");
     // pinned staging for this search's uploads (set-up, lists of slices)
     if ((st = reserve_stage(s, pk.bytes.size() + ((size_t)64 << 10) + (size_t)n_slices * 32 +
-                                   (size_t)p->n_M * 1024)) != POS_OK)
+                                   (size_t)p->n_M * 64)) != POS_OK)
         return st;
     POS_CUDA(cudaGetDevice(&s.hd.device));
     POS_CUDA(s.ws.blob.reserve(pk.bytes.size()));
@@ -1559,30 +1565,50 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
     }
     // warm-up sampling (Sec. 4.2.3), split over the M values in proportion
     // to their feasible slices
+    // (one upload and one sampling launch for all of them)
     if (p->warmup > 0 && n_feasible > 0) {
-        POS_CUDA(s.d_feasible.reserve(sizeof(uint32_t) * n_feasible));
+        std::vector<SampleSeg> segs;
+        std::vector<int> seg_mi;
+        uint32_t first = 0, total = 0;
         for (int mi = 0; mi < p->n_M; ++mi) {
             const auto &fl = feas_by_m[mi];
             if (fl.empty()) continue;
+            const long long room = std::min<long long>(s.cap, INT32_MAX) - (long long)total;
             const long long n_s = std::min<long long>(
-                s.cap, std::max<long long>(1, (long long)p->warmup * (long long)fl.size() /
-                                                  (long long)n_feasible));
-            POS_TRY(upload(s, s.d_feasible.p, fl.data(), sizeof(uint32_t) * fl.size()));
-            sample_kernel<<<(int)std::min<long long>((n_s + 255) / 256, 4 * sm_count()), 256, 0,
-                            s.stream>>>(
-                d_all, static_cast<const uint32_t *>(s.d_feasible.p), (int)fl.size(), (int)n_s,
-                s.S, p->seed + 0x632BE59BD9B4E019ull * (uint64_t)mi,
-                static_cast<const uint4 *>(s.d_feas.p), static_cast<const uint8_t *>(s.ws.d_lim.p),
-                static_cast<Leaf *>(s.d_leaves.p), s.L);
-            POS_CUDA(cudaGetLastError());
-            s.launches++;
-            const unsigned long long cnt = (unsigned long long)n_s;
-            POS_TRY(upload(s, s.ctr + 36, &cnt, 8));
-            if ((st = run_leaves(s, static_cast<const Leaf *>(s.d_leaves.p), s.ctr + 36, d_all,
-                                 p->M_list[mi], static_cast<unsigned long long *>(s.d_best.p))) !=
-                POS_OK)
+                room, std::max<long long>(1, (long long)p->warmup * (long long)fl.size() /
+                                                 (long long)n_feasible));
+            if (n_s > 0) {
+                segs.push_back({(uint64_t)n_s, p->seed + 0x632BE59BD9B4E019ull * (uint64_t)mi,
+                                first, (uint32_t)fl.size(), total, 0u});
+                seg_mi.push_back(mi);
+                total += (uint32_t)n_s;
+            }
+            first += (uint32_t)fl.size();
+        }
+        const size_t seg_bytes = sizeof(SampleSeg) * segs.size();
+        std::vector<unsigned char> up(seg_bytes + sizeof(uint32_t) * n_feasible);
+        std::memcpy(up.data(), segs.data(), seg_bytes);
+        uint32_t *list = reinterpret_cast<uint32_t *>(up.data() + seg_bytes);
+        for (int mi = 0; mi < p->n_M; ++mi)
+            list = std::copy(feas_by_m[mi].begin(), feas_by_m[mi].end(), list);
+        POS_CUDA(s.d_feasible.reserve(up.size()));
+        POS_TRY(upload(s, s.d_feasible.p, up.data(), up.size()));
+        unsigned char *d_up = static_cast<unsigned char *>(s.d_feasible.p);
+        sample_kernel<<<(int)std::min<long long>((total + 127) / 128, 8 * sm_count()), 128, 0,
+                        s.stream>>>(
+            d_all, reinterpret_cast<const uint32_t *>(d_up + seg_bytes),
+            reinterpret_cast<const SampleSeg *>(d_up), (int)segs.size(), (int)total, s.S,
+            static_cast<const uint4 *>(s.d_feas.p), static_cast<const uint8_t *>(s.ws.d_lim.p),
+            static_cast<Leaf *>(s.d_leaves.p), s.L);
+        POS_CUDA(cudaGetLastError());
+        s.launches++;
+        for (size_t q = 0; q < segs.size(); ++q) {
+            if ((st = run_leaves(s, static_cast<const Leaf *>(s.d_leaves.p) + segs[q].out,
+                                 reinterpret_cast<unsigned long long *>(d_up + sizeof(SampleSeg) * q),
+                                 d_all, p->M_list[seg_mi[q]],
+                                 static_cast<unsigned long long *>(s.d_best.p))) != POS_OK)
                 return st;
-            warm_evals += (uint64_t)n_s;
+            warm_evals += segs[q].n_s;
         }
     }
     // the greedy plans' makespans (side stream) before anything that reads
