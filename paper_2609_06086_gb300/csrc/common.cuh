@@ -124,6 +124,10 @@ struct Handle {
     // w = 1..lim_w in-flight micro-batches; lim_bytes = 0 when the table
     // would exceed kLimMaxBytes and the pass checks the sums directly
     int lim_off, lim_w, lim_bytes;
+    // the decode pass's inverse of the binomials (fill_inverse; right before
+    // the memory-limit table, byte inv_off; 0 bytes without that table), and
+    // the largest k up to which every C(L-1, k) is below 2^32
+    int inv_off, inv_bytes, inv_narrow;
 };
 constexpr int kLimMaxBytes = 32768;
 // Threads per block of the argmin kernels (poseidon_argmin and
@@ -195,9 +199,6 @@ struct Tab {
     __device__ __forceinline__ int n_types() const { return ly->n_types; }
 };
 
-__device__ __forceinline__ int32_t ld32(const unsigned char *base, uint32_t off) {
-    return *reinterpret_cast<const int32_t *>(base + off);
-}
 __device__ __forceinline__ int64_t ld64(const unsigned char *base, uint32_t off) {
     return *reinterpret_cast<const int64_t *>(base + off);
 }
@@ -332,6 +333,43 @@ __device__ __forceinline__ int unrank_step(const Tab &t, int rem, int k, uint64_
     }
     Y -= below;
     return j;
+}
+
+// The same step for k >= 2 with the estimate read from a table, for kernels
+// that unrank many ranks.  A bucket holds the Y that share their exponent and
+// first few mantissa bits as a float; inverse_bits makes it narrower than the
+// gap between C(j, k) and C(j+1, k) for every j < 127, so with g the answer for
+// its lowest Y the answer is g or g + 1, and one comparison with C(g, k)
+// decides: about 12 instructions where the estimate and its two loops take 45
+// and five of them go to the transcendental unit.  (The decode pass is bound by
+// issue slots; whole calls on a GB300, estimate / table: 20 million 1F1B plans
+// 2122 / 1973 us, 2 million Eager 364 / 346, 250,007 with 24-byte records 77.1 /
+// 69.8.)  NARROW: Y is below 2^32 (k is at most Handle::inv_narrow).
+//
+// inv: an int2 (shift, base) for each k < 16, then the bytes g; the bucket of Y
+// is byte (bits of Y as a float >> shift) + base of inv.  The conversion
+// truncates, so the bucket's bits are Y's own.
+__host__ __device__ constexpr int inverse_bits(int k) { return k <= 3 ? 6 : k <= 7 ? 5 : 4; }
+constexpr int kInverseHeader = 16 * 8;
+
+template <bool NARROW>
+__device__ __forceinline__ int unrank_table(const Tab &t, const uint8_t *inv, int k, uint64_t &Y) {
+    const int2 row = reinterpret_cast<const int2 *>(inv)[k];
+    float yf = __uint2float_rz((uint32_t)Y);
+    if constexpr (!NARROW) yf = __fmaf_rz(__uint2float_rz((uint32_t)(Y >> 32)), 4294967296.0f, yf);
+    const int g = inv[(__float_as_int(yf) >> row.x) + row.y];
+    const unsigned char *c = t.base + t.ly->off_binom + 8u * (uint32_t)(k * kBinomN + g);
+    if constexpr (NARROW) {
+        const uint32_t y = (uint32_t)Y, below = (uint32_t)*reinterpret_cast<const int32_t *>(c - 8),
+                       at = (uint32_t)*reinterpret_cast<const int32_t *>(c);
+        Y = y - (at < y ? at : below);
+        return g + (at < y ? 1 : 0);
+    } else {
+        const uint64_t below = (uint64_t)ld64(c - 8, 0), at = (uint64_t)ld64(c, 0);
+        const bool up = at < Y;
+        Y -= up ? at : below;
+        return g + (up ? 1 : 0);
+    }
 }
 
 // Cooperative 16-byte copy of the blob into shared memory, four loads in
@@ -482,15 +520,6 @@ __device__ __forceinline__ void stage_weights(const Tab &t, const int (&cut)[S +
             w.pb[s] = e.y;
         }
     }
-}
-
-template <int S>
-__device__ __forceinline__ bool plan_fits(const Tab &t, int M, const int (&cut)[S + 1],
-                                          const int (&cls)[S]) {
-    bool ok = true;
-#pragma unroll
-    for (int s = 0; s < S; ++s) ok &= stage_fits(t, S, M, s, cls[s], cut[s], cut[s + 1]);
-    return ok;
 }
 
 // ---------------------------------------------------------------------------

@@ -304,8 +304,8 @@ static pos_status launch_sort(const EvalParams &p, int64_t m, uint32_t *hist, ui
 // window's candidates by that count (a counting sort over 16 buckets) and
 // its warps then decode 32 consecutive entries of that order at a time:
 // the lanes of a warp loop over (nearly) the same number of stages.
-// LIM: only the binomials (the blob's first off_Pw bytes) and the
-// memory-limit table are staged, the table right after the binomials.
+// LIM: only the binomials (the blob's first off_Pw bytes), their inverse and
+// the memory-limit table are staged, one after the other.
 constexpr int kDecodeThreads = 256;
 constexpr int kDecodeWindowMax = 768;
 constexpr int kDecodeBuckets = POS_MAX_STAGES + 1;  // stage counts 1..16 (0 unused)
@@ -339,8 +339,8 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) decode_kernel(EvalParams p,
     __shared__ DecodeWindow win;
     if constexpr (LIM) {
         stage_blob(sm, p.blob, p.lay.off_Pw);
-        stage_blob(sm + p.lay.off_Pw, static_cast<const unsigned char *>(p.blob) + p.lim_off,
-                   p.lim_bytes);
+        stage_blob(sm + p.lay.off_Pw, static_cast<const unsigned char *>(p.blob) + p.inv_off,
+                   p.inv_bytes + p.lim_bytes);
     } else {
         stage_blob(sm, p.blob, p.lay.bytes);
     }
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) decode_kernel(EvalParams p,
     grid_dep_wait();  // the sorted positions (scatter pass)
     grid_dep_trigger();
     const Tab t = tab_at(sm, p.lay);
-    const uint8_t *lim = sm + p.lay.off_Pw;
+    const uint8_t *inv = sm + p.lay.off_Pw, *lim = inv + p.inv_bytes;
     const int sched = p.lay.sched;
     const int lane = threadIdx.x & 31;
     for (int64_t w0 = blockIdx.x * (int64_t)window; w0 < p.n; w0 += (int64_t)gridDim.x * window) {
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) decode_kernel(EvalParams p,
             const uint32_t i = (uint32_t)(w0 + li);
             const uint4 rec = win.rec[li];
             const uint32_t tpc = win.tpc[li];
-            const uint4 out = decode_one<LIM>(t, rec, tpc, p, i, lim);
+            const uint4 out = decode_one<LIM>(t, rec, tpc, p, i, inv, lim);
             store_decoded(p.cuts + 2 * (size_t)win.dest[li], out, make_uint4(i, rec.z, rec.w, tpc));
         }
         __syncthreads();  // the window's arrays are rewritten for the next one
@@ -407,7 +407,7 @@ pos_status launch_decode(const EvalParams &p, cudaStream_t stream) {
     const bool lim = p.lim_bytes > 0;
     const void *kern = lim ? reinterpret_cast<const void *>(decode_kernel<true>)
                            : reinterpret_cast<const void *>(decode_kernel<false>);
-    const int smem = lim ? p.lay.off_Pw + p.lim_bytes : p.lay.bytes;
+    const int smem = lim ? p.lay.off_Pw + p.inv_bytes + p.lim_bytes : p.lay.bytes;
     POS_TRY(ensure_smem(kern, smem));
     int per_sm = 0;
     POS_TRY(blocks_per_sm(kern, kDecodeThreads, smem, &per_sm));
@@ -568,6 +568,9 @@ static EvalParams eval_params(const Handle *h, const void *d_cands, bool per_sta
     p.lim_off = h->lim_off;
     p.lim_w = h->lim_w;
     p.lim_bytes = h->lim_bytes;
+    p.inv_off = h->inv_off;
+    p.inv_bytes = h->inv_bytes;
+    p.inv_narrow = h->inv_narrow;
     return p;
 }
 
@@ -608,7 +611,6 @@ pos_status launch_eval(Handle *h, const void *d_cands, bool per_stage_tp, int64_
         p.offs = offs;
         p.cuts = cuts;
         p.tiles = tiles;
-        p.nkeys = nk;
         cudaError_t e = cudaMemsetAsync(tiles, 0, sizeof(uint32_t) * (kTiles + 2 * (size_t)nk), stream);
         if (e == cudaSuccess)
             st = il ? launch_sort<kKeysIl>(p, m, hist, offs, cursor, dest, keys, stream)

@@ -4,16 +4,16 @@
 // checks, overflow guard, unranking, memory check; few registers, so the
 // latency of its dependent shared-memory lookups is hidden by many warps)
 // writes every candidate's cut positions to its place in the (S, M)-sorted
-// order, and the makespan pass reads them coalesced.  The makespan loop
-// costs ~6*S*M integer ops and its live registers grow with S (about 7*S),
-// so the batch is first counting-sorted by exact (S, M) (stream-ordered
-// scratch: every candidate's sorted position), and then a family of
-// kernels, each owning the candidates of one S range with M >= S (ramps
-// unrolled, steady loop) or of one M range with M < S (short_kernel), walks
-// its contiguous range of the sorted records with launch bounds matched to
-// its register need.  Warps therefore see one (S, M)
+// order, and the makespan pass reads them coalesced.  The makespan code is
+// unrolled over the stages and its live registers grow with S (about 7*S),
+// so the batch is first counting-sorted by S and M (stream-ordered scratch:
+// every candidate's sorted position), and then a family of kernels, each
+// owning the candidates of one S range with M >= S (eval_kernel: ramps
+// unrolled, steady steps until the bounds meet) or of one M range with M < S
+// (short_kernel), walks its contiguous range of the sorted records with
+// launch bounds matched to its register need.  Warps therefore see one S
 // except at bucket boundaries, and no kernel waits at a block barrier after
-// staging the cost tables.
+// staging the cost tables.  Small batches skip the sort (lane_max).
 //
 // Sort keys: fast path (M >= S for 1F1B, M >= 2S-1 for Eager 1F1B) ->
 // (S-1)*32 + M/8 (a warp's plans end after about the same steps whatever M is,
@@ -43,7 +43,7 @@ struct EvalParams {
     uint8_t *F;
     const uint32_t *dest;  // sorted position of every candidate (kNoDest:
                            // no key, answered by the histogram pass)
-    const uint32_t *offs;  // [nkeys + 1] start of every key in sorted order
+    const uint32_t *offs;  // [keys + 1] start of every key in sorted order
                            // (written by the scatter pass)
     uint4 *cuts;           // per sorted position j, two 16-byte words (read once,
                            // with evict-first loads, so that the outputs'
@@ -67,11 +67,11 @@ struct EvalParams {
     int sms;               // SMs of the device
     uint32_t *tiles;       // [17] next tile of the range that starts at stage count
                            // S (GroupWalk), zero at the start
-    int nkeys;             // kKeys, or kKeysIl under Interleaved 1F1B
     int per_stage_tp;      // 1: records carry a TP index per stage (n_tp <= 4)
     // the handle's memory-limit table (Handle::lim_*): the decode pass stages
     // the binomials and this table and checks memory with one byte per stage
     int lim_off, lim_w, lim_bytes;
+    int inv_off, inv_bytes, inv_narrow;  // Handle::inv_*
 };
 
 // The record fields every pass reads, in the 16-byte record's word layout:
@@ -138,13 +138,31 @@ __device__ __forceinline__ int packed_cut(const uint32_t (&pw)[4], int n, int q)
     return (int)((pw[b >> 2] >> (8 * (b & 3))) & 0xffu);
 }
 
+// One unranking step of the decode pass, k stages after the one that it places
+// (unrank_step's contract): by the inverse table, or without it by the estimate.
+template <bool LIM>
+__device__ __forceinline__ int unrank_k(const Tab &t, const uint8_t *inv, int narrow, int rem,
+                                        int k, uint64_t &Y) {
+    if constexpr (LIM) {
+        if (k == 1) {  // C(j, 1) = j
+            const int j = (int)Y;
+            Y = 1;
+            return j;
+        }
+        return k > narrow ? unrank_table<false>(t, inv, k, Y) : unrank_table<true>(t, inv, k, Y);
+    } else {
+        return unrank_step(t, rem, k, Y);
+    }
+}
+
 // Decode pass for an Interleaved 1F1B record (pad byte V >= 2, S = N
 // devices): checks its fields (N*V <= 16 virtual stages, at most L, M a
 // multiple of N) and the overflow guard over the N*V virtual stages, and
 // unranks the composition of L layers into the virtual stages.  Memory is
 // checked by the makespan kernel (it needs the device chains).
+template <bool LIM>
 __device__ __forceinline__ uint4 decode_il(const Tab &t, const uint4 &rec, uint32_t tpc,
-                                           const EvalParams &p, uint32_t i) {
+                                           const EvalParams &p, uint32_t i, const uint8_t *inv) {
     const uint64_t rank = (uint64_t)rec.x | ((uint64_t)rec.y << 32);
     const uint32_t tcode = rec.z;
     const int S = rec.w & 0xff;
@@ -177,7 +195,7 @@ __device__ __forceinline__ uint4 decode_il(const Tab &t, const uint4 &rec, uint3
 #pragma unroll 1
     for (int j = 0; j < J - 1; ++j) {
         const int rem = L - c, k = J - j - 1;
-        c += rem - unrank_step(t, rem, k, Y);
+        c += rem - unrank_k<LIM>(t, inv, p.inv_narrow, rem, k, Y);
         if (j < 8) lo8 |= (uint64_t)c << (8 * j);
         else hi8 |= (uint64_t)c << (8 * (j - 8));
     }
@@ -186,16 +204,16 @@ __device__ __forceinline__ uint4 decode_il(const Tab &t, const uint4 &rec, uint3
 }
 
 // Decode pass for one candidate: checks its fields and the overflow guard,
-// unranks the composition stage by stage (unrank_step, carrying Y),
-// checks each stage's memory as soon as its cut is known (LIM: by the
-// memory-limit table staged at `lim`), and packs the cut positions
+// unranks the composition stage by stage (carrying Y; LIM: by the inverse
+// table staged at `inv`), checks each stage's memory as soon as its cut is
+// known (LIM: by the memory-limit table staged at `lim`), and packs the cut positions
 // (push_cut).  Invalid and overflowing candidates are answered here.  S is
 // a runtime value and the stage loop is not unrolled, which keeps the
 // kernel small enough to run many warps per SM.
 template <bool LIM>
 __device__ __forceinline__ uint4 decode_one(const Tab &t, const uint4 &rec, uint32_t tpc,
                                             const EvalParams &p, uint32_t i,
-                                            const uint8_t *lim) {
+                                            const uint8_t *inv, const uint8_t *lim) {
     const uint64_t rank = (uint64_t)rec.x | ((uint64_t)rec.y << 32);
     const uint32_t tcode = rec.z;
     const int S = rec.w & 0xff;
@@ -203,7 +221,7 @@ __device__ __forceinline__ uint4 decode_one(const Tab &t, const uint4 &rec, uint
     const int tp = (rec.w >> 16) & 0xff;
     const int L = t.L();
     if (t.ly->sched == POS_SCHED_INTERLEAVED_1F1B && (rec.w >> 24) >= 2)
-        return decode_il(t, rec, tpc, p, i);
+        return decode_il<LIM>(t, rec, tpc, p, i, inv);
     bool ok = S >= 1 && S <= POS_MAX_STAGES && M >= 1 && S <= L && tp < t.n_tp();
     const uint64_t n_map = ok ? binom(t, L - 1, S - 1) : 0;
     ok = ok && rank < n_map;
@@ -242,14 +260,23 @@ __device__ __forceinline__ uint4 decode_one(const Tab &t, const uint4 &rec, uint
     };
     bool fits = true;
     int c = 0;
-    // stages 0..S-2 (k stages after each), then the last one up to L
-#pragma unroll 1
-    for (int k = S - 1; k >= 1; --k) {
-        const int rem = L - c;
-        const int c2 = c + (rem - unrank_step(t, rem, k, Y));
+    // stages 0..S-2 (k stages after each; L - c layers are left), then the last
+    // one up to L
+    auto place = [&](int c2) {
         push_cut(cuts, c2);
         fits &= fits_stage(c, c2);
         c = c2;
+    };
+    int k = S - 1;
+    if constexpr (LIM) {
+#pragma unroll 1
+        for (; k > max(p.inv_narrow, 1); --k) place(L - unrank_table<false>(t, inv, k, Y));
+#pragma unroll 1
+        for (; k >= 2; --k) place(L - unrank_table<true>(t, inv, k, Y));
+        if (k == 1) place(L - (int)Y);  // C(j, 1) = j
+    } else {
+#pragma unroll 1
+        for (; k >= 1; --k) place(L - unrank_step(t, L - c, k, Y));
     }
     fits &= fits_stage(c, L);
     p.F[i] = fits ? POS_FEAS_YES : POS_FEAS_NO;

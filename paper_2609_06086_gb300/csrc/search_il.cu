@@ -719,7 +719,6 @@ pos_status il_leaves(IlRun &r, const unsigned long long *count) {
     ep.offs = static_cast<const uint32_t *>(r.ws.il_offs.p);
     ep.cuts = static_cast<uint4 *>(r.ws.il_rec.p);
     set_tables(ep, r.blob, r.lay);
-    ep.nkeys = kKeysIl;
     POS_TRY(eval_interleaved(r.pair, ep, r.st));
     POS_TRY(ensure_smem(reinterpret_cast<const void *>(il_consider_kernel), r.lay.bytes));
     const int cas = r.p->cas_limit == 0 ? kCasLimit : std::max(0, r.p->cas_limit);

@@ -265,6 +265,31 @@ pos_status launch_lim(const void *d_blob, const BlobLayout &ly, int wmax, uint8_
     return POS_OK;
 }
 
+// The inverse of the binomials for ranks of L layers (unrank_table), appended
+// to the blob; returns its bytes, a multiple of 16.
+static int fill_inverse(std::vector<unsigned char> &host, const BlobLayout &ly) {
+    const uint64_t *bn = reinterpret_cast<const uint64_t *>(host.data() + ly.off_binom);
+    std::vector<unsigned char> g(kInverseHeader, 0);
+    for (int k = 2; k < kBinomK && k < ly.L; ++k) {
+        const int bits = inverse_bits(k);
+        // the bucket of y counted from the first one of y = 1
+        auto bucket = [bits](uint64_t y) {
+            const int e = 63 - __builtin_clzll(y);
+            const uint64_t m = e >= bits ? y >> (e - bits) : y << (bits - e);
+            return (size_t)e * ((size_t)1 << bits) + (size_t)(m - ((uint64_t)1 << bits));
+        };
+        const size_t first = g.size();
+        const int32_t row[2] = {23 - bits, (int32_t)first - (127 << bits)};
+        std::memcpy(g.data() + 8 * k, row, sizeof(row));
+        // every bucket whose lowest value is at most C(j, k), not yet given
+        for (int j = k; j < ly.L; ++j)
+            g.resize(first + bucket(bn[k * kBinomN + j]) + 1, (unsigned char)j);
+    }
+    g.resize((g.size() + 15) & ~(size_t)15, 0);
+    host.insert(host.end(), g.begin(), g.end());
+    return (int)g.size();
+}
+
 pos_status create_handle(const pos_tables *t, int sched, Handle **out) {
     std::vector<unsigned char> host;
     BlobLayout ly;
@@ -280,12 +305,23 @@ pos_status create_handle(const pos_tables *t, int sched, Handle **out) {
     h->guard_P = P;
     // in-flight micro-batches of a stage: at most 16 (1F1B), 31 (Eager 1F1B)
     h->lim_w = sched == POS_SCHED_EAGER_1F1B ? 2 * POS_MAX_STAGES - 1 : POS_MAX_STAGES;
-    h->lim_off = ly.bytes;
+    h->inv_off = ly.bytes;
+    h->inv_bytes = 0;
+    h->inv_narrow = 0;
     const long long lb = (long long)ly.K * h->lim_w * (ly.L + 1);
     h->lim_bytes = lb <= kLimMaxBytes ? (int)((lb + 15) & ~15ll) : 0;
+    if (h->lim_bytes > 0) {
+        const uint64_t *bn = reinterpret_cast<const uint64_t *>(host.data() + ly.off_binom);
+        while (h->inv_narrow + 1 < kBinomK &&
+               bn[(h->inv_narrow + 1) * kBinomN + ly.L - 1] < ((uint64_t)1 << 32))
+            ++h->inv_narrow;
+        h->inv_bytes = fill_inverse(host, ly);
+    }
+    h->lim_off = h->inv_off + h->inv_bytes;
     cudaError_t e = cudaGetDevice(&h->device);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_blob, (size_t)ly.bytes + h->lim_bytes);
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_blob, host.data(), ly.bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&h->d_blob, (size_t)h->lim_off + h->lim_bytes);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(h->d_blob, host.data(), host.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && launch_prefix_rows(h->d_blob, ly, 0) != POS_OK) e = cudaErrorLaunchFailure;
     if (e == cudaSuccess && h->lim_bytes > 0) {
         if (launch_lim(h->d_blob, ly, h->lim_w, static_cast<uint8_t *>(h->d_blob) + h->lim_off, 0) !=
