@@ -348,19 +348,20 @@ __device__ __forceinline__ bool dispatch_range(int S, const Tab &t, const uint4 
 // 449 us with neighbouring ones; the whole sweep of 20 million 2364 -> 2259 us
 // with tiles; 2 million Eager plans 413 us with stretches, 439 us with tiles.)
 struct GroupWalk {
-    static constexpr uint32_t kTile = 8;
+    static constexpr uint32_t kTile = 8, kTiled = 32;
     uint32_t begin, end, g, g_end, tiles, groups, stride;
     uint32_t *queue, *counter;  // 64 entries; next tile
     int queued;
     bool use_queue, more;
+    // queued_from <= kTiled: groups per warp above which plans are queued
     __device__ __forceinline__ GroupWalk(uint32_t b, uint32_t e, uint32_t *q, uint32_t *c,
-                                         uint32_t sms)
+                                         uint32_t sms, uint32_t queued_from)
         : begin(b), end(e), queue(q), counter(c), queued(0) {
         constexpr uint32_t kWarps = kEvalThreads / 32;
         stride = gridDim.x * kWarps;
         groups = (end - begin + 31) / 32;
-        use_queue = groups > 2 * stride;
-        more = groups > 32 * stride;  // tiles
+        use_queue = groups > queued_from * stride;
+        more = groups > kTiled * stride;
         tiles = (groups + kTile - 1) / kTile;
         if (more) {
             g = g_end = 0;
@@ -416,6 +417,15 @@ struct GroupWalk {
     }
 };
 
+// With two groups per warp or fewer a queue has too few plans.  The plans of a
+// range without bounds (Eager 1F1B, 14 stages and more) have nothing to queue,
+// and their time grows with M, so up to the tiles each warp takes its share of
+// every M (2 million Eager plans on a GB300: 333 us with a stretch of the range
+// per warp, 310 us with every stride-th group; tiles from 8 groups on: 340 us).
+__host__ __device__ constexpr uint32_t queued_from(int path, int slo) {
+    return path == kPathEager && !eager_bounds(slo) ? GroupWalk::kTiled : 2u;
+}
+
 // Evaluates the sorted positions [offs[key_lo], offs[key_hi]): all
 // candidates with S in [SLO, SHI] on path PATH.
 template <int SLO, int SHI, int PATH, int MINB>
@@ -435,8 +445,8 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) 
     grid_dep_wait();  // the decoded records
     grid_dep_trigger();
     const Tab t = tab_at(sm, p.tlay);
-    GroupWalk walk(begin, end, s_queue[threadIdx.x >> 5], p.tiles + SLO,
-                   (uint32_t)p.sms);
+    GroupWalk walk(begin, end, s_queue[threadIdx.x >> 5], p.tiles + SLO, (uint32_t)p.sms,
+                   queued_from(PATH, SLO));
     uint32_t j;
     bool active, to_end;
     while (walk.next(j, active, to_end)) {
