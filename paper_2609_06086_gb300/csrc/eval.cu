@@ -304,6 +304,8 @@ static pos_status launch_sort(const EvalParams &p, int64_t m, uint32_t *hist, ui
 // window's candidates by that count (a counting sort over 16 buckets) and
 // its warps then decode 32 consecutive entries of that order at a time:
 // the lanes of a warp loop over (nearly) the same number of stages.
+// Bound by issue slots (the steps' integer work; 20 million 1F1B plans on a
+// GB300: 438 us, 609 us with estimated binomial inverses).
 // LIM: only the binomials (the blob's first off_Pw bytes), their inverse and
 // the memory-limit table are staged, one after the other.
 constexpr int kDecodeThreads = 256;

@@ -427,7 +427,11 @@ __host__ __device__ constexpr uint32_t queued_from(int path, int slo) {
 }
 
 // Evaluates the sorted positions [offs[key_lo], offs[key_hi]): all
-// candidates with S in [SLO, SHI] on path PATH.
+// candidates with S in [SLO, SHI] on path PATH.  Bound by issue slots (ramp,
+// tail and first steps are straight-line code per stage) and, from 13 stages
+// on, by instruction fetch.  Ranges of 20 million 1F1B plans on a GB300, every
+// step run / with the bounds: 13..16 stages 1054 / 621 us, 9..12 595 / 365,
+// 5..8 374 / 235.
 template <int SLO, int SHI, int PATH, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) eval_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -561,7 +565,10 @@ __device__ __forceinline__ int32_t short_dispatch(int M, const Tab &t, const uin
 }
 
 // Evaluates the sorted positions of the short pipelines with M in [MLO, MHI]
-// (sorted by M, then S: a warp's plans have one M except at a boundary).
+// (sorted by M, then S: a warp's plans have one M except at a boundary).  Bound
+// by instruction fetch, so the code is one per M and not one per (S, M) (the
+// short plans of 20 million 1F1B plans on a GB300: 144 us unrolled per (S, M),
+// 61 us so; of 2 million Eager plans 166 / 60 us).
 template <bool EAGER, int MLO, int MHI, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) short_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -638,13 +645,15 @@ inline void set_tables(EvalParams &p, const void *blob, const BlobLayout &lay) {
 pos_status launch_decode(const EvalParams &p, cudaStream_t stream);
 
 // Batches up to this many candidates take the lane-per-stage kernel of
-// eval_lanes.cu.  Random plans of 64 layers, 2..16 stages and 8..128
-// micro-batches on a GB300, lanes / sorted path: 1F1B 14.9 / 68 us at 3,001,
-// 36.6 / 63 us at 32,768 and 61.5 / 70 us at 65,536; Eager 1F1B 18.6 / 120,
-// 59.6 / 88 and 104.9 / 104 us.  The limits stay below the crossing because
-// plans that reach the steady state late cost the lanes more.
+// eval_lanes.cu.  The lanes' time grows with the micro-batches, the sorted
+// path's hardly does, so the line lies where long pipelines cross.  Random plans
+// of 64 layers and 2..16 stages on a GB300, lanes / sorted path: 1F1B with 8..128
+// micro-batches 15.0 / 55.6 us at 3,001, 36.6 / 43.5 at 32,768, 49.5 / 46.1 at
+// 49,152; with 120..255 22.5 / 46.8, 46.6 / 50.3 and 60.5 / 53.2.  Eager 1F1B
+// 18.6 / 101, 48.2 / 71.8 at 24,576, 70.8 / 67.8 at 40,960; with 120..255 25.2 /
+// 59.6, 63.4 / 63.4 and 90.0 / 66.3.
 inline int64_t lane_max(int sched) {
-    return sched == POS_SCHED_1F1B ? 49152 : sched == POS_SCHED_EAGER_1F1B ? 32768 : 0;
+    return sched == POS_SCHED_1F1B ? 36864 : sched == POS_SCHED_EAGER_1F1B ? 24576 : 0;
 }
 pos_status launch_lanes(const EvalParams &p, cudaStream_t stream);
 

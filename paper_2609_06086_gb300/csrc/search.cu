@@ -56,9 +56,10 @@ __device__ __forceinline__ int popc128(const Bits128 &b) {
 // (c, limtab] is a feasible start of stage x + 1, where limtab[k][w-1][c]
 // (lim_kernel) is the largest end that class k holds from c with w
 // micro-batches in flight, so a stage costs a byte load per start and a few
-// bit operations (a binary search over the memory sums by a block per slice
-// before: 1262 us for 168,000 slices, 420 of them feasible, on a GB300).  A slice whose
-// set empties on the way is infeasible and left alone; only the feasible ones
+// bit operations and the
+// rest is their latency (168,000 slices, 420 of them feasible, on a GB300: 135
+// us; 1261 us with a block per slice and a binary search over the memory sums
+// per start; 1,680 slices 9 and 17 us).  A slice whose set empties on the way is infeasible and left alone; only the feasible ones
 // write their rows: feas[gid*(S+1) + x], lim[(gid*S + x)*128 + c] = the most
 // layers stage x holds from c (0 if none).  root[gid] = 1 when the slice has a
 // memory-feasible plan.
@@ -153,7 +154,9 @@ __global__ void __launch_bounds__(kFeasThreads) feas_kernel(const SliceRec *slic
 // (0, 0) to write the slice's argmin completion as a plan: a memory-feasible
 // plan whose makespan is usually close to the slice's best (warm-up seed).
 // root_lb[r] = V1[0][0] * scale, a lower bound on the objective of row r's
-// slice.
+// slice.  Every length is that of a path of a plan, so 32 bits hold it; the
+// kernel is bound by the latency of its S dependent rows (420 slices of 8
+// stages and 80 layers on a GB300: 18 us, 26 us in 64 bits).
 constexpr int kBoundThreads = 512;
 
 // Row r is slice rows[r], whose table row (vslot) it becomes.  rows = NULL:
@@ -265,7 +268,8 @@ __global__ void __launch_bounds__(kBoundThreads) bound_kernel(
 
 // The slices of the batches in processing order, the root prefixes (slot j of
 // a batch, no stage placed; the first nb serve a batch of nb) and the batches'
-// counters, cleared.
+// counters, cleared.  A launch of its own (3.5 us on a GB300, for any number of
+// slices so far) in place of records gathered on the host and uploaded.
 __global__ void gather_kernel(const SliceRec *slices, const uint32_t *order, uint32_t n,
                               SliceRec *batch, uint32_t n_roots, Prefix *roots,
                               unsigned long long *ctr, uint32_t n_ctr) {
@@ -316,7 +320,9 @@ __device__ __forceinline__ int nth_set(const Bits128 &b, int r) {
 // One thread per sample: stage by stage, the layer count is drawn uniformly
 // among the counts l that fit the stage's memory (l <= lim) and leave a
 // memory-feasible suffix (feasibility bit of c + l), i.e. the set bits of
-// one 128-bit window, picked with a popcount and a select.
+// one 128-bit window, picked with a popcount and a select.  Bound by the chain
+// of dependent loads of one sample, so one launch draws for every micro-batch
+// count (three counts on a GB300: 7 us, 19 us with a launch each).
 // The samples of one M index: n_s of them, from n_feasible slices at `first`
 // of the list, to the leaf slots from `out` on.
 struct SampleSeg {
@@ -733,8 +739,14 @@ __device__ __forceinline__ void level_holes(const ExpandParams &p, unsigned long
 
 // One warp per group of 32 consecutive parents: each lane finds its
 // parent's children (a 128-bit set of cut positions), the warp reserves
-// output slots with one atomic and writes them -- or, when the output is
-// full, marks its reserved slots as holes and defers the group.
+// output slots in runs and writes them -- or, when the output is full, marks
+// its reserved slots as holes and defers the group.  Small levels are bound by
+// the latency of a parent's loads and binary searches, large ones by issue slots
+// (every bound in 32 bits; the completion level tests from the largest count
+// down and stops where a falling bound settles the rest).  All levels of a
+// 70B-like search on a GB300, Eq. 2 as printed (75 million entries): completion
+// 1951 -> 1133 us, the level before it 1082 -> 916; tightened bound: completion
+// 69 -> 48 us, the other levels 190 -> 169.
 template <bool COMPLETE, int X>
 __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
     extern __shared__ __align__(16) unsigned char sm[];

@@ -187,6 +187,11 @@ __host__ __device__ constexpr int leaf_min_blocks(int S, int path) {
                : (S <= 4 ? 4 : S <= 8 ? 3 : 2);
 }
 
+// Evaluates the complete plans and lowers the incumbent.  Bound by issue slots
+// (weights from the prefix sums, the two makespan bounds, the steps of the few
+// plans that neither bound settles); with the incumbent as the limit most plans
+// end at the bounds (70B-like search on a GB300, 1.86 million plans: 70 us for
+// all launches of a search, 110 us running every plan's steps).
 template <int S, int PATH>
 __global__ void __launch_bounds__(256, leaf_min_blocks(S, PATH)) leaf_kernel(LeafParams p) {
     extern __shared__ __align__(16) unsigned char sm[];

@@ -1,5 +1,5 @@
-"""Batches up to the lane-per-stage kernel's limits (49152 candidates under
-1F1B, 32768 under Eager 1F1B) and just above them, where the sorted path
+"""Batches up to the lane-per-stage kernel's limits (36864 candidates under
+1F1B, 24576 under Eager 1F1B) and just above them, where the sorted path
 takes over: every stage count with the fewest and the most micro-batches,
 invalid and overflowing records among them, odd batch sizes, both record
 forms, against the oracle."""
@@ -28,7 +28,7 @@ def batch(gen, w, n, per_stage, rng):
 
 @pytest.mark.parametrize("per_stage", [False, True])
 @pytest.mark.parametrize("sched", [0, 1])
-@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 5001, 32768, 32769, 49152, 49153])
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 5001, 24576, 24577, 36864, 36865])
 def test_small_batches(n, sched, per_stage):
     import gen
     import oracle
