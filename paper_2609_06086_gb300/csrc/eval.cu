@@ -305,11 +305,15 @@ static pos_status launch_sort(const EvalParams &p, int64_t m, uint32_t *hist, ui
 // its warps then decode 32 consecutive entries of that order at a time:
 // the lanes of a warp loop over (nearly) the same number of stages.
 // Bound by issue slots (the steps' integer work; 20 million 1F1B plans on a
-// GB300: 438 us, 609 us with estimated binomial inverses).
+// GB300, in blocks of 256: 438 us, 609 us with estimated binomial inverses).
+// Blocks of 512 on windows of 1536: half the table copies and rounder warps than
+// 256 on 768 at the same 32 warps per SM (calls, 256 / 512: 16 million 1496 / 1469
+// us, 250,007 with 24-byte records 60.1 / 56.1; three blocks of 512 with 40
+// registers 1473 and 56.4, but a million interleaved plans 254 / 250 / 260).
 // LIM: only the binomials (the blob's first off_Pw bytes), their inverse and
 // the memory-limit table are staged, one after the other.
-constexpr int kDecodeThreads = 256;
-constexpr int kDecodeWindowMax = 768;
+constexpr int kDecodeThreads = 512;
+constexpr int kDecodeWindowMax = 1536;
 constexpr int kDecodeBuckets = POS_MAX_STAGES + 1;  // stage counts 1..16 (0 unused)
 
 __device__ __forceinline__ int decode_bucket(int sched, uint32_t w) {
@@ -336,7 +340,7 @@ struct DecodeWindow {
 };
 
 template <bool LIM>
-__global__ void __launch_bounds__(kDecodeThreads, 4) decode_kernel(EvalParams p, int window) {
+__global__ void __launch_bounds__(kDecodeThreads, 2) decode_kernel(EvalParams p, int window) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ DecodeWindow win;
     if constexpr (LIM) {
