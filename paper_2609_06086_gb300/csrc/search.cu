@@ -751,20 +751,24 @@ template <bool COMPLETE, int X>
 __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
     // timing tables and, when expanding under prune mode 2, the
-    // completion-bound rows of depth X+1 of every slot (contiguous), by TMA;
-    // all written before the previous kernel, so staged while it finishes
+    // completion-bound rows of depth X+1 of every slot (contiguous), by TMA,
+    // staged while the previous kernel finishes: the tables come from
+    // setup_kernel, the rows from bound_kernel, and the slice records that
+    // name each slot's row from gather_kernel, all two or more kernels back
+    // -- except that gather_kernel is right before the first batch's depth 0
     __shared__ uint64_t bar;
     __shared__ unsigned long long s_stats[5];
     if (threadIdx.x < 5) s_stats[threadIdx.x] = 0;
     const bool use_v = !COMPLETE && p.prune == 2;
     const bool stage_v = use_v && p.vb_smem;
-    // depth X+1 of the bound tables: the row of table row v is vdepth + 128 v
-    const int2 *vdepth = use_v ? p.vb + (size_t)(X + 1) * p.n_vrows * 128 : nullptr;
     if (threadIdx.x == 0) {
         const uint32_t vbytes = stage_v ? (uint32_t)p.nb * 128u * 8u : 0u;
         bulk_begin(&bar, (uint32_t)p.lay.bytes + vbytes);
         bulk_copy(sm, p.blob, (uint32_t)p.lay.bytes, &bar);
     }
+    if constexpr (X == 0) grid_dep_wait();
+    // depth X+1 of the bound tables: the row of table row v is vdepth + 128 v
+    const int2 *vdepth = use_v ? p.vb + (size_t)(X + 1) * p.n_vrows * 128 : nullptr;
     if (stage_v) {
         __syncthreads();  // the barrier is armed before the other copies start
         if (threadIdx.x < 32)
