@@ -44,7 +44,10 @@ struct EvalParams {
     const uint32_t *dest;  // sorted position of every candidate (kNoDest:
                            // no key, answered by the histogram pass)
     const uint32_t *offs;  // [keys + 1] start of every key in sorted order
-                           // (written by the scatter pass)
+                           // (written by the scatter pass, the decode pass
+                           // after it)
+    int offs_last;         // 1: offs come from the kernel right before the
+                           // makespan kernel instead (interleaved search)
     uint4 *cuts;           // per sorted position j, two 16-byte words (read once,
                            // with evict-first loads, so that the outputs'
                            // sectors stay in L2):

@@ -231,7 +231,9 @@ __device__ __forceinline__ void il_dispatch(int N, int V, const Tab &t, const ui
 template <int PLO, int PHI, int MINB>
 __global__ void __launch_bounds__(kEvalThreads, MINB) il_eval_kernel(EvalParams p) {
     extern __shared__ __align__(16) unsigned char sm[];
-    // the key offsets come from the scatter pass, two or more kernels back
+    // the key offsets come from the scatter pass, two or more kernels back, or
+    // in a search from the kernel right before (il_offs_kernel)
+    if (p.offs_last) grid_dep_wait();
     const int64_t begin = p.offs[kKeys + IlPair<PLO>::key], end = p.offs[kKeys + IlPair<PHI + 1>::key];
     // blocks with no record (all of them when the range is empty) leave
     // without staging the tables, after the decode pass has completed

@@ -723,6 +723,7 @@ pos_status il_leaves(IlRun &r, const unsigned long long *count) {
     ep.T = static_cast<int32_t *>(r.ws.il_T.p);
     ep.F = static_cast<uint8_t *>(r.ws.il_F.p);
     ep.offs = static_cast<const uint32_t *>(r.ws.il_offs.p);
+    ep.offs_last = 1;
     ep.cuts = static_cast<uint4 *>(r.ws.il_rec.p);
     set_tables(ep, r.blob, r.lay);
     POS_TRY(eval_interleaved(r.pair, ep, r.st));

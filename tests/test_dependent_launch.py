@@ -25,7 +25,7 @@ EARLY = {
     "decode_kernel": {"p.blob": TABLES},
     "eval_kernel": {"p.tblob": TABLES, "p.offs": "sort_scatter_kernel; decode_kernel is between"},
     "short_kernel": {"p.tblob": TABLES, "p.offs": "sort_scatter_kernel; decode_kernel is between"},
-    "il_eval_kernel": {"p.cblob": TABLES, "p.offs": "sort_scatter_kernel; decode_kernel is between"},
+    "il_eval_kernel": {"p.cblob": TABLES},
 }
 # kernels with a first wait under a condition: the condition, and what is safe
 # between it and the wait of every instance
@@ -33,6 +33,9 @@ LATER = {
     "level_kernel": ("if constexpr (X == 0)",
                      {"p.slices": "gather_kernel; at depths above 0 a level kernel is between",
                       "p.vb": "bound_kernel; gather_kernel is between"}),
+    "il_eval_kernel": ("if (p.offs_last)",
+                       {"p.offs": "sort_scatter_kernel, decode_kernel between; offs_last is set "
+                                  "where il_offs_kernel writes them right before"}),
 }
 
 
