@@ -21,6 +21,7 @@
 #include <numeric>
 #include <vector>
 
+#include "search_batches.h"
 #include "search_host.h"
 
 namespace pos {
@@ -1685,18 +1686,8 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
     size_t max_nb = 1;
     for (const Group &g : groups) {
         const auto &fl = feas_by_m[g.mi];
-        // Eq. 2 alone: eight batches, best first, so that the incumbent
-        // improves between them.  With the completion bounds the warm-up
-        // already holds each slice's argmin completion and every launch
-        // costs more than a little extra pruning saves: a first batch of
-        // the 1/16 of the slices with the smallest root bounds (most likely
-        // to hold the optimum), then the rest in one batch.
-        const size_t bsz = p->prune == 2
-                               ? std::min<size_t>(65535, fl.size())
-                               : std::min<size_t>(65535, std::max<size_t>(32, (fl.size() + 7) / 8));
-        const size_t first = p->prune == 2 ? (fl.size() + 15) / 16 : bsz;
-        for (size_t b0 = 0; b0 < fl.size();) {
-            const size_t nb = std::min(b0 == 0 ? first : bsz, fl.size() - b0);
+        size_t b0 = 0;
+        for (const size_t nb : batch_sizes(fl.size(), p->prune)) {
             batches.push_back({p->M_list[g.mi], ordered.size(), nb});
             ordered.insert(ordered.end(), fl.begin() + b0, fl.begin() + b0 + nb);
             max_nb = std::max(max_nb, nb);
