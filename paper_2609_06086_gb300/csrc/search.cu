@@ -1581,25 +1581,26 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         }
     }
     // warm-up sampling (Sec. 4.2.3), split over the M values in proportion
-    // to their feasible slices
-    // (one upload and one sampling launch for all of them)
+    // to their feasible slices, each M value up to the leaf buffer's capacity
+    // (one upload and one sampling launch for as many M values as fit it
+    // together, nearly always all)
     if (p->warmup > 0 && n_feasible > 0) {
         std::vector<SampleSeg> segs;
         std::vector<int> seg_mi;
-        uint32_t first = 0, total = 0;
+        const long long room = std::min<long long>(s.cap, INT32_MAX);
+        uint32_t first = 0;
+        long long total = 0;
         for (int mi = 0; mi < p->n_M; ++mi) {
             const auto &fl = feas_by_m[mi];
             if (fl.empty()) continue;
-            const long long room = std::min<long long>(s.cap, INT32_MAX) - (long long)total;
             const long long n_s = std::min<long long>(
                 room, std::max<long long>(1, (long long)p->warmup * (long long)fl.size() /
                                                  (long long)n_feasible));
-            if (n_s > 0) {
-                segs.push_back({(uint64_t)n_s, p->seed + 0x632BE59BD9B4E019ull * (uint64_t)mi,
-                                first, (uint32_t)fl.size(), total, 0u});
-                seg_mi.push_back(mi);
-                total += (uint32_t)n_s;
-            }
+            if (total + n_s > room) total = 0;  // a launch of its own
+            segs.push_back({(uint64_t)n_s, p->seed + 0x632BE59BD9B4E019ull * (uint64_t)mi, first,
+                            (uint32_t)fl.size(), (uint32_t)total, 0u});
+            seg_mi.push_back(mi);
+            total += n_s;
             first += (uint32_t)fl.size();
         }
         const size_t seg_bytes = sizeof(SampleSeg) * segs.size();
@@ -1611,21 +1612,26 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         POS_CUDA(s.d_feasible.reserve(up.size()));
         POS_TRY(upload(s, s.d_feasible.p, up.data(), up.size()));
         unsigned char *d_up = static_cast<unsigned char *>(s.d_feasible.p);
-        sample_kernel<<<(int)std::min<long long>((total + 127) / 128, 8 * sm_count()), 128, 0,
-                        s.stream>>>(
-            d_all, reinterpret_cast<const uint32_t *>(d_up + seg_bytes),
-            reinterpret_cast<const SampleSeg *>(d_up), (int)segs.size(), (int)total, s.S,
-            static_cast<const uint4 *>(s.d_feas.p), static_cast<const uint8_t *>(s.ws.d_lim.p),
-            static_cast<Leaf *>(s.d_leaves.p), s.L);
-        POS_CUDA(cudaGetLastError());
-        s.launches++;
-        for (size_t q = 0; q < segs.size(); ++q) {
-            if ((st = run_leaves(s, static_cast<const Leaf *>(s.d_leaves.p) + segs[q].out,
-                                 reinterpret_cast<unsigned long long *>(d_up + sizeof(SampleSeg) * q),
-                                 d_all, p->M_list[seg_mi[q]],
-                                 static_cast<unsigned long long *>(s.d_best.p))) != POS_OK)
-                return st;
-            warm_evals += segs[q].n_s;
+        for (size_t q0 = 0, q1; q0 < segs.size(); q0 = q1) {
+            for (q1 = q0 + 1; q1 < segs.size() && segs[q1].out > 0;) ++q1;
+            const int n = (int)(segs[q1 - 1].out + segs[q1 - 1].n_s);
+            sample_kernel<<<(int)std::min<long long>((n + 127ll) / 128, 8 * sm_count()), 128, 0,
+                            s.stream>>>(
+                d_all, reinterpret_cast<const uint32_t *>(d_up + seg_bytes),
+                reinterpret_cast<const SampleSeg *>(d_up) + q0, (int)(q1 - q0), n, s.S,
+                static_cast<const uint4 *>(s.d_feas.p), static_cast<const uint8_t *>(s.ws.d_lim.p),
+                static_cast<Leaf *>(s.d_leaves.p), s.L);
+            POS_CUDA(cudaGetLastError());
+            s.launches++;
+            for (size_t q = q0; q < q1; ++q) {
+                if ((st = run_leaves(
+                         s, static_cast<const Leaf *>(s.d_leaves.p) + segs[q].out,
+                         reinterpret_cast<unsigned long long *>(d_up + sizeof(SampleSeg) * q), d_all,
+                         p->M_list[seg_mi[q]],
+                         static_cast<unsigned long long *>(s.d_best.p))) != POS_OK)
+                    return st;
+                warm_evals += segs[q].n_s;
+            }
         }
     }
     // the greedy plans' makespans (side stream) before anything that reads

@@ -75,6 +75,19 @@ def test_warmup_never_changes_the_plan(P, orc, warmup):
         assert same_plan(plan, ref), prune
 
 
+def test_warmup_capacity_is_per_micro_batch_count(P):
+    """Every micro-batch count draws up to the frontier's capacity (here
+    32 * L), also when the counts together exceed it."""
+    w = gen.config3()
+    w.M_list = [32, 64, 96]
+    want, st = gpu_search(P, w, prune=1, warmup=6000)
+    assert st["warmup_evaluated"] == 6000
+    for warmup, n in ((100_000, 3 * 32 * w.L), (4500, 4500), (3 * 32 * w.L, 3 * 32 * w.L)):
+        plan, st = gpu_search(P, w, prune=1, warmup=warmup, frontier_cap=1)
+        assert st["warmup_evaluated"] == n
+        assert same_plan(plan, want)
+
+
 @pytest.mark.parametrize("cap", [1, 3000, 20_000])
 def test_tiny_frontiers_defer_and_still_match(P, orc, cap):
     """Capacities far below the frontier sizes force many deferral passes
