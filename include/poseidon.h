@@ -306,8 +306,8 @@ typedef struct pos_problem {
     uint64_t seed;              /* warm-up sampling seed */
     int32_t schedule;           /* POS_SCHED_1F1B, POS_SCHED_EAGER_1F1B or
                                    POS_SCHED_INTERLEAVED_1F1B (with V below) */
-    int64_t frontier_cap;       /* entries per frontier buffer; 0 = default 2^24;
-                                   raised to at least 32*L */
+    int64_t frontier_cap;       /* entries that a frontier buffer holds; 0 = default
+                                   2^24; raised to at least 32*L */
     int32_t profile;            /* 1: device time per kernel kind in the stats (CUDA
                                    events around every launch); 0: those fields are 0 */
     int32_t ridge;              /* 1: layer-level pruning (Theorem 2): only plans whose
@@ -397,7 +397,9 @@ typedef struct pos_search_stats {
  * below 2^32.  Memory-feasible slices are
  * enumerated in batches of at most 65535 slices, one after another.
  * Memory: the work buffers (one frontier of frontier_cap 32-byte entries per
- * depth, a leaf buffer of the same length, slice and feasibility tables,
+ * depth, a leaf buffer of the same length, each with a share of slots that
+ * may stay empty beside them when frontier_cap is above 1.9 million (at most
+ * 25 %, 11 % at the default; GB300), slice and feasibility tables,
  * and with POS_PRUNE_TIGHT 1 KB of bound tables per stage and slice of a
  * batch),
  * a stream and pinned counters are kept per device between calls, grown on

@@ -725,6 +725,29 @@ __device__ __forceinline__ void level_warp_mode(const ExpandParams &p, const Tab
     }
 }
 
+// Output slots are reserved by atomics on one counter, which serialise, so a
+// warp with many groups ahead reserves a run of slots and takes its children's
+// places from it; its last groups reserve what they need, and what is then left
+// of the run becomes holes.  (Under the paper's bound the 70B-like search has 4
+// children per parent, one completion per 16.)  Slots of a run in a level of
+// n_work groups of 32 parents over n_warps warps; 0: no runs.
+__host__ __device__ constexpr int level_run(bool complete, long long n_work, long long n_warps) {
+    return complete ? (n_work >= 128 * n_warps ? 64 : 0)
+                    : (n_work >= 64 * n_warps ? 512 : n_work >= 16 * n_warps ? 128 : 0);
+}
+// Slots that hold `cap` children whatever holes the runs leave: a warp has one
+// open run at the end of a level.
+static long long slots_for(long long cap, long long n_warps) {
+    long long holes = 0;
+    for (;;) {  // the holes are parents of the next level too
+        const long long n_work = (cap + holes + 31) / 32;
+        const long long need = n_warps * std::max(level_run(false, n_work, n_warps),
+                                                  level_run(true, n_work, n_warps));
+        if (need <= holes) return cap + holes;
+        holes = need;
+    }
+}
+
 // Slots [lo, hi) of the output, those below its capacity, become holes (by
 // the lanes of one warp).
 template <bool COMPLETE>
@@ -805,15 +828,7 @@ __global__ void __launch_bounds__(kThreads, 3) level_kernel(ExpandParams p) {
     if (warp_mode)
         level_warp_mode<COMPLETE, X>(p, t, n_in, vsm, vdepth, tops, emitted, cb, cm, cr,
                                      written_parents);
-    // Output slots are reserved by atomics on one counter, which serialise, so a
-    // warp with many groups ahead reserves a run of slots and takes its
-    // children's places from it; its last groups reserve what they need, and
-    // what is then left of the run becomes holes.  (Under the paper's bound the
-    // 70B-like search has 4 children per parent, one completion per 16.)
-    int run = 0;
-    if (!p.exact && !warp_mode)
-        run = COMPLETE ? (n_work >= 128 * n_warps ? 64 : 0)
-                       : (n_work >= 64 * n_warps ? 512 : n_work >= 16 * n_warps ? 128 : 0);
+    const int run = p.exact || warp_mode ? 0 : level_run(COMPLETE, n_work, n_warps);
     unsigned long long cur = 0;  // the open run: next slot, slots left
     int left = 0;
     for (long long w = warp; !warp_mode && w < n_work; w += n_warps) {
@@ -1011,7 +1026,8 @@ struct Search {
     cudaEvent_t (&ev)[3];
     int S = 0, L = 0, n_tp = 0;
     uint64_t n_map = 0;
-    long long cap = 0;
+    long long cap = 0;    // entries that a frontier holds
+    long long slots = 0;  // slots of its buffer (slots_for)
     int grid_level = 0;
     const SliceSpace *sp = nullptr;  // the slices' identities, global-index order
     DevBuf &d_slices, &d_feas, &d_batch, &d_inc, &d_ctr, &d_best, &d_feasible, &d_leaves,
@@ -1209,7 +1225,7 @@ static pos_status reserve_lb(Search &s, size_t n) {
 }
 
 static pos_status ensure_depth(Search &s, int depth) {
-    POS_CUDA(s.d_front[depth].reserve(sizeof(Prefix) * (size_t)s.cap));
+    POS_CUDA(s.d_front[depth].reserve(sizeof(Prefix) * (size_t)s.slots));
     return POS_OK;
 }
 
@@ -1233,7 +1249,7 @@ static ExpandParams base_params(Search &s, const SliceRec *batch, int M) {
     p.vb = static_cast<const int2 *>(s.ws.d_vb.p);
     p.nb = s.cur_nb;
     p.n_vrows = s.n_vrows;
-    p.cap = (unsigned long long)s.cap;
+    p.cap = (unsigned long long)s.slots;
     p.inc = static_cast<const Key128 *>(s.d_inc.p);
     p.stats = s.stats;
     // level kernels read only the timing tables: stage that part alone
@@ -1248,7 +1264,7 @@ static pos_status run_leaves(Search &s, const Leaf *leaves, unsigned long long *
     LeafParams lp;
     lp.leaves = leaves;
     lp.count = count;
-    lp.cap = (unsigned long long)s.cap;
+    lp.cap = (unsigned long long)s.slots;
     lp.slices = table;
     lp.M = M;
     lp.n_map = s.n_map;
@@ -1355,7 +1371,7 @@ static pos_status process(Search &s, const SliceRec *batch, int M, int x, const 
             }
         }
         if (!last) {
-            const long long n_out = (long long)std::min<unsigned long long>(cnt[0], s.cap);
+            const long long n_out = (long long)std::min<unsigned long long>(cnt[0], s.slots);
             if (n_out > 0) {
                 st = process(s, batch, M, x + 1, static_cast<const Prefix *>(s.d_front[x + 1].p),
                              n_out);
@@ -1446,10 +1462,11 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
     POS_TRY(blocks_per_sm(reinterpret_cast<const void *>(level_kernel<false, 0>), kThreads,
                           timing_layout(s.h->lay).bytes, &per_sm));
     s.grid_level = std::max(1, per_sm) * sm_count();
+    s.slots = slots_for(s.cap, (long long)s.grid_level * (kThreads / 32));
 
     POS_CUDA(s.d_feas.reserve(sizeof(uint4) * (size_t)n_slices * (s.S + 1)));
     POS_CUDA(s.ws.d_lim.reserve((size_t)n_slices * s.S * 128));
-    POS_CUDA(s.d_leaves.reserve(sizeof(Leaf) * (size_t)s.cap));
+    POS_CUDA(s.d_leaves.reserve(sizeof(Leaf) * (size_t)s.slots));
     DevBuf &d_root = s.d_root;
     POS_CUDA(d_root.reserve(n_slices));
     {
@@ -1748,7 +1765,7 @@ static pos_status search_impl(Search &s, pos_plan *out, pos_search_stats *stats)
         for (int x = 1; x <= S - 2; ++x)
             if ((st = ensure_depth(s, x)) != POS_OK) return st;
         for (int x = 0; x <= S - 2; ++x)
-            if ((st = ensure_defer(s, x, (s.cap + 31) / 32 + 1)) != POS_OK) return st;
+            if ((st = ensure_defer(s, x, (s.slots + 31) / 32 + 1)) != POS_OK) return st;
         unsigned long long *bctr = static_cast<unsigned long long *>(s.ws.d_bctr.p);
         // timing events (profile only), S + 1 per batch: before level 0,
         // after each level kernel, after the leaf kernel

@@ -1,9 +1,16 @@
 """Large frontiers, where a warp reserves its output slots in runs and leaves
 holes behind: an exhaustive search evaluates every composition exactly once,
-and its plan is the one that the pruned searches find."""
+and its plan is the one that the pruned searches find; and children that fit the
+capacity fit whatever holes the runs leave.  A search keeps its work buffers (here
+up to 25 GB), so each check is a process of its own."""
 import math
+import os
+import subprocess
+import sys
 
 import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 pytestmark = pytest.mark.gpu
 
@@ -20,12 +27,22 @@ def workload(L, S, M):
     return w
 
 
+def few_completions():
+    """Four heavy layers at the end: the bound cuts a plan with two of them in
+    one stage, so most prefixes of 13 of the 15 stages, the largest frontier,
+    have no completion."""
+    w = workload(29, 15, 20)
+    w.fwd[:, :-4] //= 50
+    w.bwd[:, :-4] //= 50
+    return w
+
+
 def prefixes(L, S, x):
     """Placements of x stages that leave a layer for each of the other S - x."""
     return math.comb(L - S + x, x)
 
 
-def test_1f1b_runs():
+def check_1f1b_runs():
     import gen
     import paper_2609_06086_gb300 as P
     L, S = 36, 10
@@ -41,7 +58,7 @@ def test_1f1b_runs():
         assert P.poseidon_search(prob)[0] == plan
 
 
-def test_interleaved_runs():
+def check_interleaved_runs():
     import gen
     import paper_2609_06086_gb300 as P
     L, N, V = 34, 5, 2
@@ -56,3 +73,42 @@ def test_interleaved_runs():
     assert st["prefixes"] == sum(prefixes(L, J, x) for x in range(1, J - 1))
     prob, keep = P.make_problem(w, warmup=0, prune=2, schedule=sched, V=V)
     assert P.poseidon_search(prob)[0] == plan
+
+
+def check_exact_fit():
+    """The largest frontier has 14.8 million entries, from 9.6 million parents
+    by warps that open runs of 512 slots: a capacity of exactly that many
+    entries still holds them."""
+    import paper_2609_06086_gb300 as P
+    w = few_completions()
+    prob, keep = P.make_problem(w, warmup=100_000, prune=1)
+    plan, st = P.poseidon_search(prob)
+    children = st["children_depth"][:w.S - 1]
+    assert st["reruns"] == 0 and 9_000_000 < children[-3] < max(children) == children[-2] < 1 << 24
+    prob, keep = P.make_problem(w, warmup=100_000, prune=1, frontier_cap=max(children))
+    again, st = P.poseidon_search(prob)
+    assert st["reruns"] == 0 and st["children_depth"][:w.S - 1] == children
+    assert again == plan
+
+
+def in_child(check):
+    r = subprocess.run([sys.executable, os.path.abspath(__file__), check], capture_output=True,
+                       text=True, timeout=600)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_1f1b_runs():
+    in_child("check_1f1b_runs")
+
+
+def test_interleaved_runs():
+    in_child("check_interleaved_runs")
+
+
+def test_exact_fit():
+    in_child("check_exact_fit")
+
+
+if __name__ == "__main__":
+    sys.path.insert(0, ROOT)
+    globals()[sys.argv[1]]()
