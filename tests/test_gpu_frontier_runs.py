@@ -1,7 +1,8 @@
 """Large frontiers, where a warp reserves its output slots in runs and leaves
 holes behind: an exhaustive search evaluates every composition exactly once,
-and its plan is the one that the pruned searches find; and children that fit the
-capacity fit whatever holes the runs leave.  A search keeps its work buffers (here
+and its plan is the one that the pruned searches find; children that fit the
+capacity fit whatever holes the runs leave; and a batch that runs out of slots
+while runs are open is finished exactly.  A search keeps its work buffers (here
 up to 25 GB), so each check is a process of its own."""
 import math
 import os
@@ -91,6 +92,32 @@ def check_exact_fit():
     assert again == plan
 
 
+def check_no_room_with_open_runs():
+    """Slots run out while warps have open runs: at an expansion level, and at
+    the completion level of an exhaustive search.  What the pipelined pass wrote
+    is evaluated once, holes are not, and the batch is run again exactly."""
+    import gen
+    import paper_2609_06086_gb300 as P
+    w = few_completions()
+    prob, keep = P.make_problem(w, warmup=100_000, prune=1)
+    want, _ = P.poseidon_search(prob)
+    for cap in (11_000_000, 12_345_678):
+        prob, keep = P.make_problem(w, warmup=100_000, prune=1, frontier_cap=cap)
+        plan, st = P.poseidon_search(prob)
+        assert st["reruns"] == 1 and st["evaluated"] == st["leaves"] + st["warmup_evaluated"]
+        assert plan == want, cap
+    L, S = 36, 10
+    w = workload(L, S, 12)
+    prob, keep = P.make_problem(w, warmup=100, prune=1)
+    want, _ = P.poseidon_search(prob)
+    prob, keep = P.make_problem(w, warmup=0, prune=0, frontier_cap=prefixes(L, S, S - 2) + 1_000_000)
+    plan, st = P.poseidon_search(prob)
+    # the completion level alone overflowed: its parents all fit
+    assert prefixes(L, S, S - 2) > 15_000_000 and st["reruns"] == 1
+    assert gen.n_compositions(L, S) < st["evaluated"] == st["leaves"]
+    assert plan == want
+
+
 def in_child(check):
     r = subprocess.run([sys.executable, os.path.abspath(__file__), check], capture_output=True,
                        text=True, timeout=600)
@@ -107,6 +134,10 @@ def test_interleaved_runs():
 
 def test_exact_fit():
     in_child("check_exact_fit")
+
+
+def test_no_room_with_open_runs():
+    in_child("check_no_room_with_open_runs")
 
 
 if __name__ == "__main__":
