@@ -429,7 +429,10 @@ pos_status launch_decode(const EvalParams &p, cudaStream_t stream) {
 }
 
 // Stream-ordered scratch comes from a library-owned pool per device that
-// keeps its memory between calls (release threshold: unlimited).
+// keeps its memory between calls (release threshold: unlimited), so what is
+// taken from it is bounded: 39 bytes per candidate of a chunk of 2^24, an
+// argmin's partial results, and host batches up to kHostPoolBytes.
+constexpr size_t kHostPoolBytes = 64ull << 20;
 static std::mutex g_pool_mutex;
 static cudaMemPool_t g_pool[64];
 
@@ -668,13 +671,17 @@ pos_status poseidon_eval_batch_host(void *handle, const pos_candidate *cands, in
     if (n < 0) return pos::fail(POS_EINVAL, "n < 0");
     if (n == 0) return POS_OK;
     if (!cands || !makespan || !feasible) return pos::fail(POS_EINVAL, "NULL buffer");
-    // stream-ordered on the default stream, from the library's pool: a
-    // cudaMalloc and cudaFree pair takes 60 us per call here
+    // stream-ordered on the default stream.  Up to kHostPoolBytes the buffers
+    // come from the library's pool (a cudaMalloc and cudaFree pair takes 60 us
+    // per call); larger ones, whose copies take 100 times that, are given back,
+    // since the pool keeps what it once held
     cudaMemPool_t pool;
     POS_TRY(pos::scratch_pool(&pool));
     void *d = nullptr;
     const size_t bc = sizeof(pos_candidate) * (size_t)n, bt = sizeof(int32_t) * (size_t)n;
-    POS_CUDA(cudaMallocFromPoolAsync(&d, bc + bt + (size_t)n, pool, 0));
+    const size_t bytes = bc + bt + (size_t)n;
+    const bool pooled = bytes <= pos::kHostPoolBytes;
+    POS_CUDA(pooled ? cudaMallocFromPoolAsync(&d, bytes, pool, 0) : cudaMalloc(&d, bytes));
     pos_candidate *dc = static_cast<pos_candidate *>(d);
     int32_t *dt = reinterpret_cast<int32_t *>(static_cast<char *>(d) + bc);
     uint8_t *df = reinterpret_cast<uint8_t *>(static_cast<char *>(d) + bc + bt);
@@ -686,8 +693,9 @@ pos_status poseidon_eval_batch_host(void *handle, const pos_candidate *cands, in
         if (st == POS_OK && e == cudaSuccess)
             e = cudaMemcpyAsync(feasible, df, (size_t)n, cudaMemcpyDeviceToHost, 0);
     }
-    const cudaError_t e2 = cudaFreeAsync(d, 0);
+    cudaError_t e2 = pooled ? cudaFreeAsync(d, 0) : cudaSuccess;
     const cudaError_t e3 = cudaStreamSynchronize(0);
+    if (!pooled) e2 = cudaFree(d);
     if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
     if (e != cudaSuccess) return pos::cuda_fail(e, "eval_batch_host copies");
     return st;

@@ -257,3 +257,20 @@ def test_config3_whole_space_sample(P, orc):
     c = gen.search_space_sample(w, 50_000, seed=7)
     T, F, Tr, Fr = _both(P, orc, w, c)
     assert np.array_equal(T, Tr) and np.array_equal(F, Fr)
+
+
+@pytest.mark.parametrize("n", [3_195_660, 3_195_661, 8_000_000])
+def test_host_batch_keeps_a_bounded_pool(P, n):
+    """A host batch's buffers (21 bytes per candidate) above 64 MB go back to
+    the device; both sides of that limit give the device call's results."""
+    import torch
+    w = gen.config5_tables()
+    h = P.Handle(P.Tables.from_workload(w))
+    c = gen.config5_candidates(n, seed=9)
+    T, F = eval_device(P, h, c)  # the pool now holds the scratch of n candidates
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    T2, F2 = P.poseidon_eval_batch_host(h, c)
+    assert free - torch.cuda.mem_get_info()[0] <= 96 << 20
+    assert np.array_equal(T, T2) and np.array_equal(F, F2)
+    h.close()
