@@ -48,7 +48,7 @@ extern "C" pos_status poseidon_argmin_noalloc(const int32_t *d_makespan,
                                               int64_t *d_out, void *stream) {
     if (n < 0 || !d_out || (n > 0 && (!d_makespan || !d_feasible)))
         return pos::fail(POS_EINVAL, "bad argmin arguments");
-    const int64_t parts = pos::argmin_parts(n);
+    const int64_t parts = pos::argmin_parts(d_makespan, d_feasible, n);
     if (parts > pos::kNoAllocParts)
         return pos::fail(POS_EINVAL,
                          "poseidon_argmin_noalloc: this GPU needs more than 4096 partial "

@@ -136,7 +136,7 @@ constexpr int kLimMaxBytes = 32768;
 constexpr int kArgminThreads = 256;
 // Partial results of an argmin over n entries (1: none are stored), and its
 // launches (eval.cu).
-int64_t argmin_parts(int64_t n);
+int64_t argmin_parts(const int32_t *T, const uint8_t *F, int64_t n);
 pos_status launch_argmin(const int32_t *T, const uint8_t *F, int64_t n, int32_t *part_t,
                          long long *part_i, int64_t *out, cudaStream_t stream);
 

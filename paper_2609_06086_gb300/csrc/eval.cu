@@ -103,22 +103,29 @@ __global__ void __launch_bounds__(kArgminThreads) argmin_final(const int32_t *pa
     if (threadIdx.x == 0) *out = bi;
 }
 
-// Blocks of the partial kernel: one up to 16384 entries (four 16-entry words
-// per thread cost less than a second launch), else a thread per 16 entries
-// up to four blocks per SM.
-int64_t argmin_parts(int64_t n) {
-    if (n <= 4 * 16 * kArgminThreads) return 1;
-    const int64_t per = 16 * kArgminThreads;
+// Does the partial kernel read 16 entries at a time?
+static bool argmin_vec(const int32_t *T, const uint8_t *F) {
+    return ((reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(F)) & 15) == 0;
+}
+
+// Blocks of the partial kernel: one where each thread has few dependent loads
+// (up to 16384 entries in words of 16, 1024 one by one: less than a second
+// launch costs), else a thread per word or entry up to four blocks per SM.
+// Entries one by one, all in one block / so, on a GB300: 8.2 / 6.2 us for
+// 3,001, 14.3 / 6.9 for 8,192, 24.6 / 7.3 for 16,384.
+int64_t argmin_parts(const int32_t *T, const uint8_t *F, int64_t n) {
+    const bool vec = argmin_vec(T, F);
+    if (n <= (vec ? 64 : 4) * kArgminThreads) return 1;
+    const int64_t per = (vec ? 16 : 1) * kArgminThreads;
     return std::min<int64_t>((n + per - 1) / per, 4LL * sm_count());
 }
 
-// part_t, part_i: argmin_parts(n) entries each (not used when that is 1).
+// part_t, part_i: argmin_parts() entries each (not used when that is 1).
 pos_status launch_argmin(const int32_t *T, const uint8_t *F, int64_t n, int32_t *part_t,
                          long long *part_i, int64_t *out, cudaStream_t stream) {
-    const int parts = (int)argmin_parts(n);
-    const bool vec = ((reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(F)) & 15) == 0;
+    const int parts = (int)argmin_parts(T, F, n);
     int64_t *direct = parts == 1 ? out : nullptr;
-    if (vec)
+    if (argmin_vec(T, F))
         argmin_partial<true><<<parts, kArgminThreads, 0, stream>>>(T, F, n, part_t, part_i, direct);
     else
         argmin_partial<false><<<parts, kArgminThreads, 0, stream>>>(T, F, n, part_t, part_i, direct);
@@ -706,7 +713,7 @@ pos_status poseidon_argmin(const int32_t *d_makespan, const uint8_t *d_feasible,
     if (n < 0 || !d_out || (n > 0 && (!d_makespan || !d_feasible)))
         return pos::fail(POS_EINVAL, "bad argmin arguments");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int64_t parts = pos::argmin_parts(n);
+    const int64_t parts = pos::argmin_parts(d_makespan, d_feasible, n);
     if (parts == 1) return pos::launch_argmin(d_makespan, d_feasible, n, nullptr, nullptr, d_out, s);
     // from the library's pool, which keeps its memory: the device's default
     // pool gives its memory back at every synchronisation, and a call then
