@@ -2,6 +2,16 @@
 buffers through the C ABI."""
 import numpy as np
 
+# above the lane-per-stage kernel's limits (36864 candidates under 1F1B, 24576
+# under Eager 1F1B): such a batch takes the sorted path
+SORTED = 40_000
+
+
+def repeated(n_records, n, seed=0):
+    """Indices of a batch of n that holds every one of n_records records about
+    equally often, in random order."""
+    return np.random.default_rng(seed).permutation(n) % n_records
+
 
 def eval_device(P, handle, cands, stream=None):
     import torch

@@ -1,7 +1,8 @@
 """Eager 1F1B on the GPU (App. B: warm-up of 2(N-i)+1 forwards) against the
 oracle with the same schedule: makespans and feasibility flags bit-exact,
-search plans identical.  Covers both GPU paths: M >= 2S-1 (compile-time
-ramps and a steady loop) and M < 2S-1 (level programs)."""
+search plans identical.  Covers the lane-per-stage kernel of small batches
+and both paths of large ones: M >= 2S-1 (compile-time ramps and a steady
+loop) and M < 2S-1 (the short pipelines' kernels)."""
 import json
 import os
 import random
@@ -10,7 +11,7 @@ import numpy as np
 import pytest
 
 import gen
-from tests.gpu_util import eval_device
+from tests.gpu_util import SORTED, eval_device, repeated
 from tests.test_oracle import _random_problem
 
 pytestmark = pytest.mark.gpu
@@ -51,8 +52,8 @@ def test_eager_config5_sample(P, orc):
 
 
 def test_eager_every_stage_count_around_the_path_switch(P, orc):
-    """S = 1..16 with M = 1..40: every (S, M) of the level programs and the
-    first M values of the fast path."""
+    """S = 1..16 with M = 1..40: every short pipeline and the first M values of
+    the fast path, by the lanes and, repeated, by the sorted path."""
     w = gen.config5_tables()
     rng = np.random.default_rng(11)
     cs = []
@@ -64,6 +65,9 @@ def test_eager_every_stage_count_around_the_path_switch(P, orc):
     c = np.concatenate(cs)
     T, F, Tr, Fr = _both(P, orc, w, c)
     assert np.array_equal(T, Tr) and np.array_equal(F, Fr)
+    pick = repeated(len(c), SORTED)
+    T, F = eval_device(P, P.Handle(P.Tables.from_workload(w), schedule=EAGER), c[pick])
+    assert np.array_equal(T, Tr[pick]) and np.array_equal(F, Fr[pick])
 
 
 def test_eager_config4_tables(P, orc):

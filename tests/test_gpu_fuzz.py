@@ -1,14 +1,15 @@
 """Randomised small tables and records under every schedule, GPU against
 the oracle element by element: degenerate shapes (one layer, one type, one
 TP index, S = L, M = 1), zero costs and transfers, zero or huge capacities,
-and records of both formats mixed with invalid ones."""
+and records of both formats mixed with invalid ones; as small batches and,
+repeated, as batches of the sorted path."""
 import math
 
 import numpy as np
 import pytest
 
 import gen
-from tests.gpu_util import eval_device, eval_device_ex
+from tests.gpu_util import SORTED, eval_device, eval_device_ex, repeated
 
 pytestmark = pytest.mark.gpu
 
@@ -77,6 +78,9 @@ def test_random_small_tables(P, orc, schedule):
         T, F = eval_device(P, h, c)
         Tr, Fr = orc.eval_batch(orc.OracleTables(**tab, schedule=schedule), c)
         assert np.array_equal(T, Tr) and np.array_equal(F, Fr), trial
+        pick = repeated(len(c), SORTED, trial)
+        T, F = eval_device(P, h, c[pick])
+        assert np.array_equal(T, Tr[pick]) and np.array_equal(F, Fr[pick]), trial
         if tab["n_tp"] <= 4:
             ex = np.zeros(len(c), dtype=gen.CANDIDATE_EX_DTYPE)
             for f in ("map_rank", "type_code", "S", "M", "V"):
@@ -86,4 +90,6 @@ def test_random_small_tables(P, orc, schedule):
             Te, Fe = eval_device_ex(P, h, ex)
             Tre, Fre = orc.eval_batch_ex(orc.OracleTables(**tab, schedule=schedule), ex)
             assert np.array_equal(Te, Tre) and np.array_equal(Fe, Fre), trial
+            Te, Fe = eval_device_ex(P, h, ex[pick])
+            assert np.array_equal(Te, Tre[pick]) and np.array_equal(Fe, Fre[pick]), trial
         h.close()

@@ -1,5 +1,6 @@
 """Short pipelines (M < S under 1F1B, M < 2S-1 under Eager 1F1B): every
-(S, M) of their kernels, and the first M beyond, against the oracle."""
+(S, M), and the first M beyond, against the oracle, in a batch of the
+lane-per-stage kernel and, repeated, in one of the sorted path's kernels."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,7 @@ def test_every_short_pipeline(sched, per_stage):
     import gen
     import oracle
     import paper_2609_06086_gb300 as P
-    from gpu_util import eval_device, eval_device_ex
+    from gpu_util import SORTED, eval_device, eval_device_ex, repeated
     w = gen.config4(seed=5)
     rng = np.random.default_rng(sched)
     tab = w.tables_dict()
@@ -34,7 +35,9 @@ def test_every_short_pipeline(sched, per_stage):
     ot = oracle.OracleTables(**tab, schedule=sched)
     T_ref, F_ref = (oracle.eval_batch_ex if per_stage else oracle.eval_batch)(ot, c)
     h = P.Handle(P.Tables(**tab), sched)
-    T, F = (eval_device_ex if per_stage else eval_device)(P, h, c)
-    bad = np.flatnonzero((T != T_ref) | (F != F_ref))
-    assert len(bad) == 0, (len(bad), c[bad[:5]], T[bad[:5]], T_ref[bad[:5]])
+    for pick in (np.arange(n), repeated(n, SORTED)):
+        T, F = (eval_device_ex if per_stage else eval_device)(P, h, c[pick])
+        bad = np.flatnonzero((T != T_ref[pick]) | (F != F_ref[pick]))
+        assert len(bad) == 0, (len(pick), len(bad), c[pick[bad[:5]]], T[bad[:5]],
+                               T_ref[pick[bad[:5]]])
     h.close()
