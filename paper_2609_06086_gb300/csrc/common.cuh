@@ -36,7 +36,9 @@ pos_status blocks_per_sm(const void *kernel, int threads, int smem, int *out);
 // the next such kernel be scheduled: a kernel's pre-wait part can therefore
 // only overlap the post-wait part of its predecessor, so it may read
 // whatever was written two or more kernels earlier (the cost tables, slice
-// records and bound tables of a search).  Every block of such a kernel
+// records and bound tables of a search; a kernel that can also follow the
+// writer itself waits first: level_kernel at depth 0, il_eval_kernel in a
+// search).  Every block of such a kernel
 // executes grid_dep_wait() before it exits, even when it has no work: a grid
 // completes only after its predecessor has, which keeps the chain's order
 // transitive for the kernels after it.  Without the launch attribute the two
@@ -108,9 +110,6 @@ BlobLayout timing_layout(const BlobLayout &ly);
 // The same with the memory part before it (everything but the binomials);
 // it starts at byte ly.off_Pw of the full blob.
 BlobLayout cost_layout(const BlobLayout &ly);
-// The memory part (Pw, Pa, cap: the three tables after the binomials),
-// rebased likewise; it starts at byte ly.off_Pw of the full blob.
-BlobLayout memory_layout(const BlobLayout &ly);
 
 struct Handle {
     int device;

@@ -581,7 +581,6 @@ static EvalParams eval_params(const Handle *h, const void *d_cands, bool per_sta
     }
     p.guard_m[0] = 0;
     p.sms = sm_count();
-    p.lim_off = h->lim_off;
     p.lim_w = h->lim_w;
     p.lim_bytes = h->lim_bytes;
     p.inv_off = h->inv_off;

@@ -73,7 +73,7 @@ struct EvalParams {
     int per_stage_tp;      // 1: records carry a TP index per stage (n_tp <= 4)
     // the handle's memory-limit table (Handle::lim_*): the decode pass stages
     // the binomials and this table and checks memory with one byte per stage
-    int lim_off, lim_w, lim_bytes;
+    int lim_w, lim_bytes;
     int inv_off, inv_bytes, inv_narrow;  // Handle::inv_*
 };
 
@@ -654,7 +654,11 @@ pos_status launch_decode(const EvalParams &p, cudaStream_t stream);
 // micro-batches 15.0 / 55.6 us at 3,001, 36.6 / 43.5 at 32,768, 49.5 / 46.1 at
 // 49,152; with 120..255 22.5 / 46.8, 46.6 / 50.3 and 60.5 / 53.2.  Eager 1F1B
 // 18.6 / 101, 48.2 / 71.8 at 24,576, 70.8 / 67.8 at 40,960; with 120..255 25.2 /
-// 59.6, 63.4 / 63.4 and 90.0 / 66.3.
+// 59.6, 63.4 / 63.4 and 90.0 / 66.3.  Few stages suit the lanes better (1F1B,
+// 36,864 plans of 1..2 stages 12 us, of 2..4 23..31), batches of 16 stages
+// alone worse: their Eager plans with 120..255 micro-batches take 82 us at
+// 24,576, more than the sorted path did before its queues and bounds (63), and
+// the rule, which sees the batch's size alone, leaves them to the lanes.
 inline int64_t lane_max(int sched) {
     return sched == POS_SCHED_1F1B ? 36864 : sched == POS_SCHED_EAGER_1F1B ? 24576 : 0;
 }

@@ -10,7 +10,8 @@
 //     stage time M (F + B) (a dynamic program over (stage, first layer));
 //     evaluated like every complete plan, they give the first incumbent;
 //  2. enumeration, level by level over the virtual stages (one thread per
-//     partial plan, 32-parent groups reserve their output with one atomic):
+//     partial plan; a warp takes the output slots of its 32-parent groups from
+//     runs that it reserves, or one reservation per group in small levels):
 //     the layer counts l of the next virtual stage that keep its device's
 //     resident bytes within capacity and the prefix's lower bound within
 //     the incumbent form a range [1, hi] (both grow with l); the last two

@@ -47,8 +47,8 @@ struct Leaf {
 };
 static_assert(sizeof(Leaf) == 32, "Leaf layout");
 
-// 32-byte entries move as two 16-byte vectors; byte I of an entry is
-// addressed at compile time (word I/4, shift 8*(I%4)).
+// 32-byte entries move as one 256-bit load or store (load32, store32); byte I
+// of an entry is addressed at compile time (word I/4, shift 8*(I%4)).
 struct Vec32 {
     uint4 a, b;
 };

@@ -125,17 +125,6 @@ BlobLayout cost_layout(const BlobLayout &ly) {
     return t;
 }
 
-BlobLayout memory_layout(const BlobLayout &ly) {
-    BlobLayout t = ly;
-    const int base = ly.off_Pw;
-    t.off_binom = t.off_P = t.off_pp = -1;  // not staged
-    t.off_Pw -= base;
-    t.off_Pa -= base;
-    t.off_cap -= base;
-    t.bytes = ly.off_P - base;
-    return t;
-}
-
 __global__ void __launch_bounds__(kPrefixThreads) prefix_rows_kernel(unsigned char *blob,
                                                                      BlobLayout ly) {
     prefix_row(blob, ly, blockIdx.x);
